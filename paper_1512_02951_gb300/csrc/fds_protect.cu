@@ -1,4 +1,5 @@
-// Fused protect kernel (Sect. 6.3.1, Fig. 6): 8x8 DCT-II per channel, int16 rounding,
+// Fused protect kernel (Sect. 6.3.1, Fig. 6) in its grouped form, for batches, packed storage and
+// the coefficient export (one image in int16 storage: fds_protect_warp.cu): 8x8 DCT-II per channel, int16 rounding,
 // zigzag fragmentation, AES-128-CTR of the confidential fragment.
 //
 // Persistent CTAs over a tile schedule (one image, or every tile of a batch of images in one
@@ -315,13 +316,6 @@ __device__ __forceinline__ void load_pixels(const TileSlot* sl, uint8_t* pix, in
     if (b < nb) cp_async8(pix + y * kRowBytes + b * 24 + 8 * q, sl->px_in + sl->blk[b] + y * w3 + 8 * q);
   }
   cp_async_commit();
-}
-
-// column pairs of the packed column pass: (0, 4), (1, 2), (3, 5), (6, 7)
-__host__ __device__ constexpr int pair_of(int v) { return (v == 0 || v == 4) ? 0 : (v < 3 ? 1 : ((v == 3 || v == 5) ? 2 : 3)); }
-__host__ __device__ constexpr int pair_lane(int v) { return (v == 4 || v == 2 || v == 5 || v == 7) ? 1 : 0; }
-__host__ __device__ constexpr int pair_col(int j, int l) {
-  return j == 0 ? (l ? 4 : 0) : (j == 1 ? (l ? 2 : 1) : (j == 2 ? (l ? 5 : 3) : (l ? 7 : 6)));
 }
 
 // BATCH: tiles of many images (round keys from the slot); else one image (round keys read
@@ -669,9 +663,7 @@ cudaError_t launch_protect(const TileArgs& a, cudaStream_t s, bool debug, int sm
     if (a.k == 5) return launch_k<5, false, true>(a, s, sms, per_sm);
     return launch_k<-1, false, true>(a, s, sms, per_sm);
   }
-  if (a.k == 0) return launch_k<0, false, false>(a, s, sms, per_sm);
-  if (a.k == 5) return launch_k<5, false, false>(a, s, sms, per_sm);
-  return launch_k<-1, false, false>(a, s, sms, per_sm);
+  return launch_protect_warp(a, s, sms);
 }
 
 }  // namespace fds

@@ -1,0 +1,574 @@
+// Fused protect kernel in its warp form (Sect. 6.3.1, Fig. 6): 8x8 DCT-II per channel, int16
+// rounding, zigzag fragmentation, AES-128-CTR of the confidential fragment, of one image.
+//
+// A subtile is 32 consecutive channel-blocks (cb = 3 * block + channel), one per lane; its public
+// and private parts are 64 (63 - k) and 64 (k + 1) bytes, whole 16-byte units.  Each warp works
+// on subtiles of its own with its own shared-memory area, and no barrier joins the warps after
+// the AES table is filled.  What bounds it is the issue of instructions, not memory (4096 x 4096,
+// k = 5: 41.8 M warp instructions = 33 us of issue slots against 22.6 us for the 151 MB), so the
+// warps have to keep issuing.  The form before it, groups of six warps that met at three named
+// barriers per 192 channel-blocks, spent its time at those barriers: 4.5 of the six warps had
+// AES blocks to do, and issue activity was 57 %; here it is 69 %.  Per subtile:
+//   1. its pixels are in the warp's buffer (bulk copies that complete on the warp's mbarrier);
+//      row butterflies; the buffer is free, so the next subtile's pixels start loading
+//   2. column butterflies by pairs of columns, rounded and written as int16 to the staging area;
+//      a pair of columns in which some lane has a value within the error guard of a
+//      half-integer (one three-input maximum per two values, one vote) marks those values
+//   3. marked values are decided exactly by the whole warp at once (round_warp), in place
+//   4. the public part leaves (bulk store); the private parts of several subtiles are collected
+//      until their keystream blocks fill whole warps (k = 5: 24 blocks each, four subtiles fill
+//      three), encrypted, and leave
+// Counter blocks that share all but their last byte share the first AES round and most of the
+// second (aes_window): 133 table lookups a block instead of 160.
+// Measured on 4096 x 4096, k = 5: 72.3 -> 54.3 us; 3240 x 2592, k = 9: 55.9 -> 38.6 us (before:
+// the grouped form; its 8-byte pixel loads and 240 AES blocks on 192 threads cost the latter
+// more).  16 warps of 128 registers; 20 of 96 measured 53.6 and 39.6 us, with spills.  Pixels two
+// subtiles ahead, or loaded with cp.async through L1, measured slower (59 / 64 us against 51 and
+// 53 us with exact decisions left out): the shared memory taken leaves L1 too small for them.
+#include "fds_aux.h"
+#include "fds_tile.cuh"
+
+namespace fds {
+
+constexpr int kWCb = 32;                          // channel-blocks per subtile, one per lane
+// one pixel row of a subtile: at most 12 blocks, in at most two segments that each start and end
+// on 16-byte boundaries
+constexpr int kWPixPitch = 320;
+constexpr int kWPixBytes = 8 * kWPixPitch;
+constexpr int kWStageBytes = 5248;                // public part, then the private parts of kAcc subtiles
+constexpr int kWPix = 0;
+constexpr int kWStage = kWPix + kWPixBytes;
+constexpr int kWList = kWStage + kWStageBytes;    // the staged private parts' subtiles
+constexpr int kWBar = kWList + 4 * 8;             // mbarrier of the pixel loads
+constexpr int kWArea = (kWBar + 8 + 31) & ~31;
+// AES constants of counter windows, 5 words each: of the whole CTA's range where it has at most
+// kWins, else two for each warp
+constexpr int kWins = 64;
+constexpr int kWWinBytes = 20 * kWins + 16 + 512; // and the CTA's subtile counter, and c(m) folded
+constexpr int kWarps = 16;
+constexpr int kBelow = ((int)kTpairWin - 1024) / kWArea;    // areas below the pair table
+constexpr int kWLow = (int)kTpairWin - kBelow * kWArea;     // window address of the first
+constexpr int kAbove = kWarps > kBelow ? kWarps - kBelow : 0;
+constexpr int kWWin = (int)kTpairWin + kTpairBytes + kAbove * kWArea;
+constexpr int kWEnd = kWWin + kWWinBytes;
+static_assert(kWEnd <= 227 * 1024, "protect (warp form) shared memory");
+
+// subtiles whose private parts are encrypted together: the fewest lanes left idle in the last
+// round of 32 keystream blocks, as far as the staging area holds them
+__host__ __device__ constexpr int acc_tiles(int k) {
+  int best = 1, bn = 4 * (k + 1), bp = (bn + 31) / 32;
+  for (int g = 2; g <= 8; ++g) {
+    if ((63 - k) * 64 + g * (k + 1) * 64 > kWStageBytes) break;
+    const int n = g * 4 * (k + 1), p = (n + 31) / 32;
+    if (n * bp > bn * p) {
+      best = g;
+      bn = n;
+      bp = p;
+    }
+  }
+  return best;
+}
+
+// One image position of a lane's channel-block: block column, block row, channel
+struct CbPos {
+  uint32_t bx, by, c;
+};
+
+__device__ __forceinline__ CbPos cb_pos(const TileArgs& a, uint32_t cb) {
+  CbPos p;
+  const uint32_t b = cb / 3;
+  p.c = cb - 3 * b;
+  p.by = (uint32_t)(((uint64_t)b * a.bx_magic) >> a.bx_shift);   // b / bx_count
+  p.bx = b - p.by * (uint32_t)a.bx_count;
+  return p;
+}
+
+// Where a lane's channel-block lies in the pixel buffer: byte offsets of its block in even and
+// odd pixel rows, plus the channel
+struct PixAt {
+  uint32_t even, odd, c;
+};
+
+// The pixels of the subtile of n channel-blocks at lane position p into the warp's pixel buffer.
+// BULK: one bulk copy per pixel row and run of blocks (a subtile lies in at most two block rows:
+// bx_count >= 12), each widened to 16-byte boundaries inside the image (its base is 16-byte
+// aligned and it is a multiple of 64 bytes long); lanes 0..7 copy the first run, 8..15 the second.
+// Else 8-byte pieces: lane's piece c of its block in 8 rows, then the pieces of the two boundary
+// blocks that other subtiles' lanes own.
+template <bool BULK>
+__device__ __forceinline__ PixAt load_subtile(const TileArgs& a, const CbPos& p, uint32_t n, int lane, uint32_t pix,
+                                              uint64_t* bar) {
+  const uint64_t pitch = 3ull * (uint64_t)a.width;
+  const uint32_t c0 = __shfl_sync(0xffffffffu, p.c, 0);
+  PixAt at;
+  at.c = p.c;
+  if constexpr (BULK) {
+    const uint32_t bx0 = __shfl_sync(0xffffffffu, p.bx, 0), by0 = __shfl_sync(0xffffffffu, p.by, 0);
+    const uint32_t nblk = (c0 + n + 2) / 3;                       // blocks the subtile touches
+    const uint32_t m0 = min(nblk, (uint32_t)a.bx_count - bx0);    // in the first block row
+    const uint32_t odd = (uint32_t)pitch & 8u;                    // skew change from row to row
+    const uint32_t sk0 = (24u * bx0) & 8u;                        // skew of even rows, first run
+    const uint32_t seg1 = (24u * m0 + 8u + 15u) & ~15u;           // where the second run starts
+    // 8 * pitch is a multiple of 64, so a block row's even rows have the same skew
+    {
+      const bool second = lane >= 8;
+      const uint32_t y = lane & 7;
+      const uint32_t m = second ? nblk - m0 : m0;
+      const uint32_t bx = second ? 0u : bx0, by = by0 + (second ? 1u : 0u);
+      const uint64_t off = ((uint64_t)by * 8 + y) * pitch + 24ull * bx;
+      const uint64_t lo = off & ~15ull, hi = (off + 24ull * m + 15) & ~15ull;
+      const bool on = lane < 16 && m > 0;
+      const uint32_t bytes = on ? (uint32_t)(hi - lo) : 0u;
+      const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+      if (lane == 0) mbar_expect_tx(bar, total);
+      __syncwarp();
+      if (on)
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                         pix + y * kWPixPitch + (second ? seg1 : 0u)),
+                     "l"(a.pixels_in + lo), "r"(bytes), "r"(smem_u32(bar))
+                     : "memory");
+    }
+    const bool in1 = p.by != by0;
+    const uint32_t base = in1 ? seg1 + 24u * p.bx : 24u * (p.bx - bx0), sk = in1 ? 0u : sk0;
+    at.even = base + sk;
+    at.odd = base + (sk ^ odd);
+  } else {
+    const uint64_t off = (uint64_t)p.by * (8 * pitch) + 24ull * p.bx;
+    const uint8_t* src = a.pixels_in + off + 8 * p.c;
+    const uint32_t dst = pix + 8 * (c0 + lane);
+    if ((uint32_t)lane < n) {
+#pragma unroll
+      for (int y = 0; y < 8; ++y) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst + y * kWPixPitch), "l"(src) : "memory");
+        src += pitch;
+      }
+    }
+    const uint32_t e1 = n == 32 ? (c0 == 0 ? 1u : (c0 == 1 ? 0u : 2u)) : 0u;
+    const uint32_t y = lane >> 2, sl = lane & 3;
+    const bool head = sl < c0;
+    const uint64_t eoff = __shfl_sync(0xffffffffu, off, head ? 0 : 31);
+    if (sl < c0 + e1) {
+      const uint32_t q = head ? sl : sl - c0 + (3 - e1);            // piece of the block
+      const uint32_t j = head ? sl : c0 + 32 + (sl - c0);           // its place in the row
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(pix + y * kWPixPitch + 8 * j),
+                   "l"(a.pixels_in + eoff + y * pitch + 8 * q)
+                   : "memory");
+    }
+    cp_async_commit();
+    at.even = at.odd = 8 * (c0 + lane - p.c);
+  }
+  return at;
+}
+
+// AES constants of counter window q (256 counter blocks that differ in the last byte only)
+__device__ __forceinline__ void aes_window(uint64_t iv_hi, uint64_t iv_lo, uint64_t q, const uint32_t* rk, PairLanes lc,
+                                           uint32_t (&w)[5]) {
+  auto r8 = [](uint32_t x) { return __byte_perm(x, x, 0x2103u); };
+  uint32_t s[4];
+  ctr_block(iv_hi, iv_lo & ~255ull, q << 8, s);
+  const uint32_t s0 = s[0] ^ rk[0], s1 = s[1] ^ rk[1], s2 = s[2] ^ rk[2], s3 = s[3] ^ rk[3];
+  // round 1: column 0 lacks T3 of the last byte
+  const uint32_t n0 = tpair<0>(s0, lc.c0) ^ tpair<2>(s2, lc.c2) ^ rk[4] ^ r8(tpair<1>(s1, lc.c0));
+  const uint32_t n1 = tpair<0>(s1, lc.c0) ^ tpair<2>(s3, lc.c2) ^ rk[5] ^ r8(tpair<1>(s2, lc.c0) ^ tpair<3>(s0, lc.c2));
+  const uint32_t n2 = tpair<0>(s2, lc.c0) ^ tpair<2>(s0, lc.c2) ^ rk[6] ^ r8(tpair<1>(s3, lc.c0) ^ tpair<3>(s1, lc.c2));
+  const uint32_t n3 = tpair<0>(s3, lc.c0) ^ tpair<2>(s1, lc.c2) ^ rk[7] ^ r8(tpair<1>(s0, lc.c0) ^ tpair<3>(s2, lc.c2));
+  w[0] = n0;
+  // round 2 without the terms of column 0
+  w[1] = tpair<2>(n2, lc.c2) ^ rk[8] ^ r8(tpair<1>(n1, lc.c0) ^ tpair<3>(n3, lc.c2));
+  w[2] = tpair<0>(n1, lc.c0) ^ tpair<2>(n3, lc.c2) ^ rk[9] ^ r8(tpair<1>(n2, lc.c0));
+  w[3] = tpair<0>(n2, lc.c0) ^ rk[10] ^ r8(tpair<1>(n3, lc.c0) ^ tpair<3>(n1, lc.c2));
+  w[4] = tpair<0>(n3, lc.c0) ^ tpair<2>(n1, lc.c2) ^ rk[11] ^ r8(tpair<3>(n2, lc.c2));
+}
+
+// keystream block whose counter's last byte is x, in the window of constants w
+__device__ __forceinline__ void aes_from_window(const uint32_t (&w)[5], uint32_t x, const uint32_t* rk, PairLanes lc,
+                                                uint32_t (&s)[4]) {
+  auto r8 = [](uint32_t v) { return __byte_perm(v, v, 0x2103u); };
+  const uint32_t n0 = w[0] ^ r8(tpair<0>(x ^ (rk[3] >> 24), lc.c2));
+  uint32_t s0 = w[1] ^ tpair<0>(n0, lc.c0);
+  uint32_t s1 = w[2] ^ r8(tpair<3>(n0, lc.c2));
+  uint32_t s2 = w[3] ^ tpair<2>(n0, lc.c2);
+  uint32_t s3 = w[4] ^ r8(tpair<1>(n0, lc.c0));
+#pragma unroll 1
+  for (int r = 3; r < 10; ++r) {
+    const uint32_t m0 = tpair<0>(s0, lc.c0) ^ tpair<2>(s2, lc.c2) ^ rk[4 * r] ^ r8(tpair<1>(s1, lc.c0) ^ tpair<3>(s3, lc.c2));
+    const uint32_t m1 = tpair<0>(s1, lc.c0) ^ tpair<2>(s3, lc.c2) ^ rk[4 * r + 1] ^ r8(tpair<1>(s2, lc.c0) ^ tpair<3>(s0, lc.c2));
+    const uint32_t m2 = tpair<0>(s2, lc.c0) ^ tpair<2>(s0, lc.c2) ^ rk[4 * r + 2] ^ r8(tpair<1>(s3, lc.c0) ^ tpair<3>(s1, lc.c2));
+    const uint32_t m3 = tpair<0>(s3, lc.c0) ^ tpair<2>(s1, lc.c2) ^ rk[4 * r + 3] ^ r8(tpair<1>(s0, lc.c0) ^ tpair<3>(s2, lc.c2));
+    s0 = m0;
+    s1 = m1;
+    s2 = m2;
+    s3 = m3;
+  }
+  auto last = [&](uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    const uint32_t lo = __byte_perm(tpair<0>(a, lc.c2), tpair<1>(b, lc.c0), 0x3250u);
+    const uint32_t hi = __byte_perm(tpair<2>(c, lc.c0), tpair<3>(d, lc.c2), 0x7210u);
+    return __byte_perm(lo, hi, 0x7610u);
+  };
+  s[0] = last(s0, s1, s2, s3) ^ rk[40];
+  s[1] = last(s1, s2, s3, s0) ^ rk[41];
+  s[2] = last(s2, s3, s0, s1) ^ rk[42];
+  s[3] = last(s3, s0, s1, s2) ^ rk[43];
+}
+
+// the constants of window q to wc[5 * slot] (every lane its own; slot < 0: none)
+__device__ __forceinline__ void put_window(const TileArgs& a, uint64_t q, int slot, uint32_t* wc) {
+  uint32_t w[5];
+  aes_window(a.iv_hi, a.iv_lo, q, a.rk, pair_lanes(), w);
+  if (slot >= 0) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) wc[5 * slot + i] = w[i];
+  }
+}
+
+// AES-128-CTR over the private parts of n staged subtiles (list[0 .. n - 1]; nb = 4 (k + 1)
+// keystream blocks each); wc: the constants of the windows from wbase on
+__device__ __forceinline__ void ctr_warp(const TileArgs& a, uint8_t* buf, const uint32_t* list, int n, uint32_t nb,
+                                         const uint32_t* wc, uint64_t wbase, int lane) {
+  const PairLanes lc = pair_lanes();
+#pragma unroll 1
+  for (uint32_t i = lane; i < n * nb; i += 32) {
+    const uint32_t j = i / nb;
+    const uint64_t b = (a.iv_lo & 255u) + (uint64_t)list[j] * nb + (i - j * nb);   // from the IV's window
+    const uint32_t* src = wc + 5 * (uint32_t)((b >> 8) - wbase);
+    const uint32_t w[5] = {src[0], src[1], src[2], src[3], src[4]};
+    uint32_t s[4];
+    aes_from_window(w, (uint32_t)b & 255u, a.rk, lc, s);
+    uint4* p = reinterpret_cast<uint4*>(buf + 16 * i);
+    uint4 d = *p;
+    d.x ^= s[0];
+    d.y ^= s[1];
+    d.z ^= s[2];
+    d.w ^= s[3];
+    *p = d;
+  }
+}
+
+// `bytes` staged bytes to global memory by one lane: a bulk store and a tail of 2-byte stores
+__device__ __forceinline__ void store_run(uint8_t* dst, const uint8_t* src, int bytes) {
+  if (bytes >> 4) bulk_store(dst, src, (uint32_t)(bytes & ~15));
+  bulk_commit();
+  for (int j = bytes & ~15; j < bytes; j += 2)
+    *reinterpret_cast<uint16_t*>(dst + j) = *reinterpret_cast<const uint16_t*>(src + j);
+}
+
+// Exact rounding of coefficient pos of one channel-block by the whole warp (pos and px, the
+// block's first byte of the channel, the same in every lane).  8 F is the sum of p[y][x]
+// (c(a - b) + c(a + b)), a = (2 y + 1) u or 4, b = (2 x + 1) v or 4 (fds_device.cuh).  Each lane
+// takes two pixels; their parts of the coordinates n_j of c(j), j = 0..7, are added as pairs of
+// 16-bit fields (|n_j| <= 2 . 64 . 255 < 2^15), so four warp sums give them all.  The value is
+// then decided in 64-bit fixed point: each c(j) 2^46 is within a unit, so the sum is within
+// sum |n_j| <= 2^15 units.  Nearer than that to a boundary it is a tie if it is rational (about
+// half of all near ties: positions whose u and v are 2 or 6), and else left to exact_round.
+constexpr int kTieFrac = 46;
+__device__ __noinline__ int round_far(const int (&n)[9], int* esc, bool* fail) { return exact_round(n, esc, fail); }
+__device__ __forceinline__ int round_warp(const uint8_t* px, uint64_t pitch, int pos, const uint4* ctab, int lane,
+                                          int& esc, bool& fail) {
+  const int u = pos >> 3, v = pos & 7, y = lane >> 2, x = 2 * (lane & 3);
+  const int a = u ? (2 * y + 1) * u : 4, b = v ? (2 * x + 1) * v : 4, b2 = v ? b + 2 * v : 4;
+  const uint8_t* p = px + y * pitch + 3 * x;
+  const uint32_t p0 = __ldg(p), p1 = __ldg(p + 3);
+  const uint4 A = ctab[(a - b) & 31], B = ctab[(a + b) & 31], C = ctab[(a - b2) & 31], D = ctab[(a + b2) & 31];
+  const uint32_t w[4] = {p0 * (A.x + B.x) + p1 * (C.x + D.x), p0 * (A.y + B.y) + p1 * (C.y + D.y),
+                         p0 * (A.z + B.z) + p1 * (C.z + D.z), p0 * (A.w + B.w) + p1 * (C.w + D.w)};
+  int n[9];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t s = __reduce_add_sync(0xffffffffu, w[i]);
+    n[2 * i] = (int16_t)(s & 0xffffu);
+    n[2 * i + 1] = (int)(s - (uint32_t)n[2 * i]) >> 16;
+  }
+  n[8] = 0;
+  long long d = (long long)(n[0] + 4) << kTieFrac;
+  int any = 0;
+#pragma unroll
+  for (int j = 1; j < 8; ++j) {
+    d += (long long)n[j] * (c_cos_q62[j - 1] >> (62 - kTieFrac));
+    any |= n[j];
+  }
+  // d / 2^49 = F + 1/2
+  const int q = (int)(d >> (kTieFrac + 3));
+  const long long rem = d & ((8ll << kTieFrac) - 1);
+  if (any == 0) return rem == 0 && q <= 0 ? q - 1 : q;      // rational: a tie goes away from zero
+  if (rem > 32768 && rem < (8ll << kTieFrac) - 32768) return q;
+  int e = 0;
+  const int r = round_far(n, &e, &fail);
+  esc += e;
+  return r;
+}
+
+template <int K, bool BULK>
+__global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __grid_constant__ TileArgs a) {
+  extern __shared__ __align__(128) uint8_t smem_cta[];
+  const uint32_t win0 = smem_u32(smem_cta);
+  if (win0 > (uint32_t)kWLow) {   // see the launcher
+    if (threadIdx.x == 0 && a.counters) atomicAdd(&a.counters[2], 1ull);
+    return;
+  }
+  const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+  uint8_t* area = smem_cta + ((warp < kBelow ? (uint32_t)(kWLow + warp * kWArea)
+                                             : kTpairWin + kTpairBytes + (uint32_t)(warp - kBelow) * kWArea) -
+                              win0);
+  const uint32_t pix = smem_u32(area + kWPix);
+  uint8_t* stage = area + kWStage;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(area + kWBar);
+  uint32_t* list = reinterpret_cast<uint32_t*>(area + kWList);
+  uint32_t* wins = reinterpret_cast<uint32_t*>(smem_cta + (kWWin - win0));
+  uint32_t* next = wins + 5 * kWins;
+  uint4* ctab = reinterpret_cast<uint4*>(next + 4);
+  const int k = K >= 0 ? K : a.k;
+  const int npub = 63 - k;
+  const uint32_t nb = 4u * (uint32_t)(k + 1);       // keystream blocks per subtile
+  const uint32_t ncb = 3u * (uint32_t)a.nblocks, nsub = (ncb + 31u) >> 5;
+  const int act = a.groups;       // working warps of each CTA
+  // the CTA's subtiles [s0, s1): taken one by one by its warps (dynamic), which evens out the
+  // last round of a small image, or, where their counter windows are more than the table holds,
+  // a run for each warp
+  const uint32_t s0 = (uint32_t)((uint64_t)nsub * blockIdx.x / gridDim.x);
+  const uint32_t s1 = (uint32_t)((uint64_t)nsub * (blockIdx.x + 1) / gridDim.x);
+  const uint32_t iv8 = (uint32_t)a.iv_lo & 255u;
+  uint64_t wbase = (iv8 + (uint64_t)s0 * nb) >> 8;
+  const uint64_t wlast = (iv8 + (uint64_t)s1 * nb - 1) >> 8;
+  const bool dynamic = wlast - wbase < kWins;
+  uint32_t t = s1, tend = s1;
+  if (warp < act) {
+    t = dynamic ? s0 + warp : s0 + (uint32_t)((uint64_t)(s1 - s0) * warp / act);
+    if (!dynamic) tend = s0 + (uint32_t)((uint64_t)(s1 - s0) * (warp + 1) / act);
+  }
+  const uint64_t pitch = 3ull * (uint64_t)a.width;
+  if (BULK && lane == 0) {
+    mbar_init(bar);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncwarp();
+  PixAt at{};
+  uint32_t phase = 0;
+  if (t < tend) at = load_subtile<BULK>(a, cb_pos(a, 32u * t + lane), min(32u, ncb - 32u * t), lane, pix, bar);
+  if (threadIdx.x == 0) *next = s0 + act;
+  if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
+    const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
+    const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
+    ctab[lane] = make_uint4(f >> 1 == 0 ? one : 0u, f >> 1 == 1 ? one : 0u, f >> 1 == 2 ? one : 0u, f >> 1 == 3 ? one : 0u);
+  }
+  fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
+  __syncthreads();
+  if (!a.plain_private) {
+    if (dynamic) {
+      const int i = (int)threadIdx.x;
+      if ((uint32_t)(i & ~31) <= wlast - wbase) put_window(a, wbase + i, (uint32_t)i <= wlast - wbase ? i : -1, wins);
+      __syncthreads();
+    } else {
+      wins += 10 * warp;
+      wbase = ~0ull - 1;
+    }
+  }
+
+  constexpr int kG = K >= 0 ? acc_tiles(K >= 0 ? K : 0) : 0;
+  const int G = K >= 0 ? kG : a.aes_pair;           // subtiles between two AES phases
+  int esc = 0, nties = 0;
+  bool fail = false;
+  int acc = 0;
+  int16_t* const pubst = reinterpret_cast<int16_t*>(stage);
+  uint8_t* const privst = stage + kWCb * 2 * npub;
+
+  while (t < tend) {
+    uint32_t tn = t + 1;                   // the warp's next subtile
+    if (dynamic) {
+      if (lane == 0) tn = atomicAdd(next, 1u);
+      tn = __shfl_sync(0xffffffffu, tn, 0);
+    }
+    const uint32_t n = min(32u, ncb - 32u * t);
+    if constexpr (BULK) {
+      if (!__all_sync(0xffffffffu, mbar_wait(bar, phase))) {   // gave up: nothing more is written
+        fail = true;
+        break;
+      }
+      phase ^= 1u;
+    } else {
+      cp_async_wait_all();
+      __syncwarp();
+    }
+    const uint32_t c = at.c;
+    const uint8_t* px_even = area + kWPix + at.even;
+    const uint8_t* px_odd = area + kWPix + at.odd;
+    float2 P[8][4];
+    float V = 0.0f;
+#pragma unroll
+    for (int y = 0; y < 8; ++y) {
+      const uint2* rp = reinterpret_cast<const uint2*>((y & 1 ? px_odd : px_even) + y * kWPixPitch);
+      const uint2 w01 = rp[0], w23 = rp[1], w45 = rp[2];
+      const uint32_t r[7] = {w01.x, w01.y, w23.x, w23.y, w45.x, w45.y, 0u};
+      uint32_t w[6];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) w[i] = __funnelshift_r(r[i], r[i + 1], 8 * c);
+      float X[8];
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {
+        const int byte = 3 * x;
+        X[x] = __int_as_float(__byte_perm(w[byte >> 2], 0x4B000000u, 0x7440u | (byte & 3)));
+      }
+      float fr[8];
+      V += dct8_row_bytes_w(X, fr);
+      P[y][0] = make_float2(fr[0], fr[4]);
+      P[y][1] = make_float2(fr[1], fr[2]);
+      P[y][2] = make_float2(fr[3], fr[5]);
+      P[y][3] = make_float2(fr[6], fr[7]);
+    }
+    __syncwarp();                          // the pixel buffer is read: the next subtile's load starts
+    if (tn < tend) at = load_subtile<BULK>(a, cb_pos(a, 32u * tn + lane), min(32u, ncb - 32u * tn), lane, pix, bar);
+    bulk_wait_read_all();                  // the staging area may be written again
+    __syncwarp();
+    int16_t* pub_cb = pubst + lane * npub;
+    int16_t* priv_cb = reinterpret_cast<int16_t*>(privst) + (acc * kWCb + lane) * (k + 1);
+    auto put = [&](int u, int v, uint32_t q) {
+      const int z = zigzag_of(u, v);
+      if (z <= k)
+        priv_cb[z] = (int16_t)q;
+      else
+        pub_cb[z - k - 1] = (int16_t)q;
+    };
+    uint32_t mlo = 0, mhi = 0;
+    float thr = 1.0f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {          // a pair of columns: transformed, rounded and staged
+      float2 col[8];
+#pragma unroll
+      for (int y = 0; y < 8; ++y) col[y] = P[y][j];
+      if (j == 0) {
+        const float W = dct8_rat_w2(col);
+        if ((uint32_t)lane < n) thr = 0.5f - fminf(fmaf(V, kGuardV, fmaf(W, kGuardW, kGuardU)), kGuardFwd);
+      } else {
+        dct8_2<false, false>(col);
+      }
+      float big = 0.0f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if ((u == 0 || u == 4) && j == 0) {
+#pragma unroll
+          for (int l = 0; l < 2; ++l) {
+            const int v = pair_col(0, l);
+            const int T = __float_as_int((l ? col[u].y : col[u].x) + kMagic) - kMagicBits;  // 8 F, exact
+            put(u, v, (uint32_t)((u == 0 && v == 0) ? ((T + 4) >> 3) + 1024 : (T + 4 - (T < 0 ? 1 : 0)) >> 3));
+          }
+          col[u] = make_float2(0.0f, 0.0f);
+        } else {
+          const float2 yv = add2(col[u], make_float2(kMagic, kMagic));
+          col[u] = sub2(col[u], add2(yv, make_float2(-kMagic, -kMagic)));
+          put(u, pair_col(j, 0), __float_as_uint(yv.x));   // low 16 bits: the int16 result
+          put(u, pair_col(j, 1), __float_as_uint(yv.y));
+          big = fmaxf(fmaxf(big, fabsf(col[u].x)), fabsf(col[u].y));
+        }
+      }
+      if (__any_sync(0xffffffffu, big > thr)) {   // rare: a near tie in these columns
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+          for (int l = 0; l < 2; ++l) {
+            const int v = pair_col(j, l);
+            if (fabsf(l ? col[u].y : col[u].x) > thr) {
+              if (8 * u + v < 32)
+                mlo |= 1u << (8 * u + v);
+              else
+                mhi |= 1u << (8 * u + v - 32);
+            }
+          }
+      }
+    }
+    // near ties, one after another, decided by the whole warp
+    for (uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0); who; who &= who - 1) {
+      const int src = __ffs(who) - 1;
+      uint64_t mask = (uint64_t)__shfl_sync(0xffffffffu, mhi, src) << 32 | __shfl_sync(0xffffffffu, mlo, src);
+      const uint32_t sc = __shfl_sync(0xffffffffu, c, src);
+      const uint8_t* blk = a.pixels_in + block_offset(a.width, (int)((32u * t + src) / 3));
+      nties += __popcll(mask);
+      for (; mask; mask &= mask - 1) {
+        const int pos = __ffsll((long long)mask) - 1;
+        int e = 0;
+        const int q = round_warp(blk + sc, pitch, pos, ctab, lane, e, fail);
+        esc += e;
+        const int z = zigzag_of(pos >> 3, pos & 7);
+        if (lane == src) *(z <= k ? priv_cb + z : pub_cb + (z - k - 1)) = (int16_t)q;
+      }
+    }
+    fence_proxy_async();                   // staged coefficients, before the bulk store
+    __syncwarp();
+    if (lane == 0) store_run(reinterpret_cast<uint8_t*>(a.pub_out) + (uint64_t)t * (64u * npub), stage, (int)n * 2 * npub);
+    if (lane == 0) list[acc] = t;
+    ++acc;
+    if (acc == G || tn >= tend) {
+      __syncwarp();
+      if (!a.plain_private) {
+        if (!dynamic) {                    // a run of subtiles: at most two windows
+          const uint64_t q = (iv8 + (uint64_t)(t + 1 - acc) * nb) >> 8;
+          if (q < wbase || ((iv8 + (uint64_t)(t + 1) * nb - 1) >> 8) > wbase + 1) {
+            wbase = q;
+            put_window(a, q + (lane & 1), lane < 2 ? lane : -1, wins);
+            __syncwarp();
+          }
+        }
+        ctr_warp(a, privst, list, acc, nb, wins, wbase, lane);
+        fence_proxy_async();
+        __syncwarp();
+      }
+      if (lane < acc) {
+        const uint32_t tj = list[lane];
+        store_run(a.priv_out + (uint64_t)tj * (64u * (k + 1)), privst + lane * (64 * (k + 1)),
+                  (int)min(32u, ncb - 32u * tj) * 2 * (k + 1));
+      }
+      acc = 0;
+    }
+    t = tn;
+  }
+  if (BULK && fail) mbar_wait(bar, phase);   // a copy still in flight
+  bulk_wait_all();
+  if (lane == 0) {
+    if (a.counters) {
+      if (nties) atomicAdd(&a.counters[0], (unsigned long long)nties);
+      if (esc) atomicAdd(&a.counters[1], (unsigned long long)esc);
+      if (fail) atomicAdd(&a.counters[2], 1ull);
+    }
+  }
+}
+
+template <int K, bool BULK>
+static cudaError_t launch_w(const TileArgs& a, cudaStream_t s, int sms) {
+  static bool attr[kMaxAttrDevices];
+  static bool window_ok[kMaxAttrDevices];
+  int dev = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxAttrDevices) return cudaErrorInvalidDevice;
+  if (!window_ok[dev]) {
+    if ((e = smem_window_start_ok(protect_warp_kernel<K, BULK>, (uint32_t)kWLow)) != cudaSuccess) return e;
+    window_ok[dev] = true;
+  }
+  e = smem_attr_once(protect_warp_kernel<K, BULK>, kWEnd, attr);
+  if (e != cudaSuccess) return e;
+  TileArgs b = a;
+  const long long nsub = (3ll * a.nblocks + 31) / 32;
+  const int grid = (int)(nsub < sms ? nsub : sms);
+  const long long per = (nsub + grid - 1) / (grid ? grid : 1);
+  b.groups = (int)(per < kWarps ? per : kWarps);
+  // blocks / bx_count as a multiply and a shift, exact for block numbers below 2^31
+  int l = 0;
+  while ((1ll << l) < a.bx_count) ++l;
+  b.bx_shift = 31 + l;
+  b.bx_magic = (uint32_t)((1ull << (31 + l)) / (uint64_t)a.bx_count + 1);
+  b.aes_pair = acc_tiles(a.k);
+  if (grid > 0) protect_warp_kernel<K, BULK><<<grid, kWarps * 32, kWEnd, s>>>(b);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_protect_warp(const TileArgs& a, cudaStream_t s, int sms) {
+  if (a.images || a.pack || a.k < 0 || a.k > 63) return cudaErrorInvalidValue;
+  // bulk copies of whole row runs need 16-byte aligned pixels and subtiles of at most two block
+  // rows
+  if (a.bx_count >= 12 && ((uintptr_t)a.pixels_in & 15) == 0) {
+    if (a.k == 0) return launch_w<0, true>(a, s, sms);
+    if (a.k == 5) return launch_w<5, true>(a, s, sms);
+    return launch_w<-1, true>(a, s, sms);
+  }
+  return launch_w<-1, false>(a, s, sms);
+}
+
+}  // namespace fds

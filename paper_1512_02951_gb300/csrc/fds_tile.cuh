@@ -107,6 +107,9 @@ struct TileArgs {
   int32_t aes_pair;
   // protect: tile groups that work in each CTA (1 .. the kernel's groups; 0 = all of them)
   int32_t groups;
+  // warp form: block row of block b = (b * bx_magic) >> bx_shift
+  uint32_t bx_magic;
+  int32_t bx_shift;
 };
 
 // What a CTA knows about the tile it is working on (shared memory, filled one tile ahead).
@@ -132,6 +135,8 @@ constexpr int32_t kPxIn16 = 1, kPxOut16 = 2;
 // for one image, 4 CTAs for batches; restore: 2 CTAs); 0 = that residency
 cudaError_t launch_protect(const TileArgs& a, cudaStream_t s, bool debug, int sms, int per_sm = 0);
 cudaError_t launch_restore(const TileArgs& a, cudaStream_t s, int sms, int per_sm = 0);
+// protect of one image in int16 storage, one subtile of 32 channel-blocks per warp
+cudaError_t launch_protect_warp(const TileArgs& a, cudaStream_t s, int sms);
 // restore with the inverse transform on tensor cores (one image, int16 storage)
 cudaError_t launch_restore_tc(const TileArgs& a, cudaStream_t s, int sms);
 // tensor-core protect of one image (form 0: BF16 three limbs, 1: TF32 two limbs); tiles of
@@ -313,6 +318,13 @@ __device__ __forceinline__ void fill_slot(const TileArgs& a, int g, TileSlot* s,
 __device__ __forceinline__ int next_tile(const TileArgs& a, int i, int vb, int vgrid) {
   if (a.dispenser == nullptr || i == 0) return vb + i * vgrid;
   return (int)atomicAdd(a.dispenser, 1u) + vgrid;
+}
+
+// column pairs of the packed column pass: (0, 4), (1, 2), (3, 5), (6, 7)
+__host__ __device__ constexpr int pair_of(int v) { return (v == 0 || v == 4) ? 0 : (v < 3 ? 1 : ((v == 3 || v == 5) ? 2 : 3)); }
+__host__ __device__ constexpr int pair_lane(int v) { return (v == 4 || v == 2 || v == 5 || v == 7) ? 1 : 0; }
+__host__ __device__ constexpr int pair_col(int j, int l) {
+  return j == 0 ? (l ? 4 : 0) : (j == 1 ? (l ? 2 : 1) : (j == 2 ? (l ? 5 : 3) : (l ? 7 : 6)));
 }
 
 // 24-byte block row of the pixel tile shifted right by `c` bytes: channel c's pixel x is
