@@ -1,4 +1,6 @@
-// Fused restore kernel (defragmentation, Sect. 3.2, Fig. 3; inverse of Sect. 6.3.1): CTR
+// Fused restore kernel (defragmentation, Sect. 3.2, Fig. 3; inverse of Sect. 6.3.1) in its tiled
+// form, for batches, packed storage and the tensor-core inverse (one image in int16 storage and
+// the public-image form: fds_restore_warp.cu): CTR
 // decryption of the confidential fragment, merge with the public fragment by zigzag
 // position, inverse 8x8 DCT, round half away from zero (exact), clamp to [0, 255].
 //
@@ -21,11 +23,6 @@
 // packed streams lands in a separate shared-memory area (bulk copies when 16-byte aligned,
 // else 8-byte cp.async pieces), its private bytes are decrypted there and both parts are
 // unpacked into the int16 staging area, all one tile ahead, before the transform reads it.
-//
-// Public-image form (PUBIMG; the paper's public fragment as an image, Sect. 6.5.1 Fig. 10):
-// the same kernel with the private positions "padded with zeros" -- the private staging
-// holds the constant (1024, 0, .., 0) per channel-block (DC 8 x 128: the zero-mean block
-// shifted to mid-grey), nothing private is loaded or decrypted.
 #include "fds_mma.cuh"
 
 namespace fds {
@@ -205,23 +202,20 @@ __device__ __forceinline__ void gather_coefs(const int16_t* pubst, const int16_t
 // cp.async the public and private ranges of slot sl's tile into staging area st
 // True if both fragment ranges of the tile are whole 16-byte units (then each arrives as one
 // bulk copy completing on an mbarrier; else as 16-byte cp.async pieces)
-// PUB_ONLY: the public range alone
-template <bool PUB_ONLY = false>
 __device__ __forceinline__ bool frag_bulk(const TileSlot* sl) {
   const int k = sl->k, nb = sl->nb;
-  return ((nb * 6 * (63 - k)) & 15) == 0 && (PUB_ONLY || ((nb * 6 * (k + 1)) & 15) == 0);
+  return ((nb * 6 * (63 - k)) & 15) == 0 && ((nb * 6 * (k + 1)) & 15) == 0;
 }
 // Load the public and private ranges of slot sl's tile into staging area st (all threads call
 // it; thread 0 issues the bulk copies)
-template <bool PUB_ONLY = false>
 __device__ __forceinline__ void load_fragments(const TileSlot* sl, uint8_t* st, uint64_t* bar) {
   const int t = threadIdx.x;
   const int k = sl->k, npub = 63 - k, nb = sl->nb;
-  const int pub_bytes = nb * 6 * npub, priv_bytes = PUB_ONLY ? 0 : nb * 6 * (k + 1);
+  const int pub_bytes = nb * 6 * npub, priv_bytes = nb * 6 * (k + 1);
   const uint8_t* psrc = sl->pub_in + (uint64_t)sl->local * kTileBlocks * 6ull * npub;
   const uint8_t* vsrc = sl->priv_in + (uint64_t)sl->local * kTileBlocks * 6ull * (k + 1);
   uint8_t* vdst = st + kTileCb * 2 * npub;
-  if (frag_bulk<PUB_ONLY>(sl)) {
+  if (frag_bulk(sl)) {
     if (t == 0) {
       mbar_expect_tx(bar, (uint32_t)(pub_bytes + priv_bytes));
       if (pub_bytes) bulk_load(st, psrc, (uint32_t)pub_bytes, bar);
@@ -244,9 +238,8 @@ __device__ __forceinline__ void load_fragments(const TileSlot* sl, uint8_t* st, 
 }
 // Wait until this thread may read what load_fragments loaded (a barrier must follow);
 // phase: the next phase of bar; lost counts bulk loads that did not complete in time
-template <bool PUB_ONLY = false>
 __device__ __forceinline__ void wait_fragments(const TileSlot* sl, uint64_t* bar, uint32_t& phase, int& lost) {
-  if (frag_bulk<PUB_ONLY>(sl)) {
+  if (frag_bulk(sl)) {
     if (!mbar_wait(bar, phase)) ++lost;
     phase ^= 1u;
   } else {
@@ -273,13 +266,13 @@ __device__ __forceinline__ void decrypt_fragments(const TileSlot* sl, const uint
 // TC: the inverse transform as tcgen05 MMAs (one image, int16 storage; a.tc_b = the inverse
 // basis table); a tile holding a coefficient of magnitude 2048 or more takes the float32
 // butterflies instead.
-template <int K, bool BATCH, bool PUBIMG = false, int PACK = 0, bool TC = false>
+template <int K, bool BATCH, int PACK = 0, bool TC = false>
 __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel(const __grid_constant__ TileArgs a) {
-  static_assert(!TC || (!BATCH && !PUBIMG && PACK == 0), "tensor-core inverse: one image, int16 storage");
+  static_assert(!TC || (!BATCH && PACK == 0), "tensor-core inverse: one image, int16 storage");
   extern __shared__ __align__(128) uint8_t smem[];
   // AES tables: T0 replicated per lane (one image, int16 storage, private fragment decrypted),
   // else the four T-tables
-  constexpr bool REP = !BATCH && PACK == 0 && !PUBIMG;
+  constexpr bool REP = !BATCH && PACK == 0;
   __shared__ __align__(16) uint32_t T4[REP ? 4 : 1024];
   uint32_t* Ts = REP ? reinterpret_cast<uint32_t*>(smem + kSmemTrep) : T4;
   uint32_t* queue = reinterpret_cast<uint32_t*>(smem + kSmemQueue);
@@ -328,14 +321,6 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
     if constexpr (TC) mbar_init(tbar);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if constexpr (PUBIMG) {   // the private staging of both areas: (1024, 0, .., 0) per channel-block
-    const int kk = a.k, np = kTileCb * (kk + 1);
-    for (int i = t; i < 2 * np; i += kThreads) {
-      const int j = i < np ? i : i - np;
-      reinterpret_cast<int16_t*>(stage(i < np ? 0 : 1) + kTileCb * 2 * (63 - kk))[j] =
-          (int16_t)(j % (kk + 1) == 0 ? 1024 : 0);
-    }
-  }
   __syncthreads();
   uint8_t* land = smem + kSmemLand;   // PACK only
   if constexpr (PACK != 0) {
@@ -346,10 +331,10 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
     __syncthreads();
     unpack_tile<PACK>(slot(0), land, stage(0));
   } else {
-    load_fragments<PUBIMG>(slot(0), stage(0), bars);
-    wait_fragments<PUBIMG>(slot(0), bars, phase[0], lost);
+    load_fragments(slot(0), stage(0), bars);
+    wait_fragments(slot(0), bars, phase[0], lost);
     __syncthreads();
-    if (!PUBIMG && !a.plain_private)
+    if (!a.plain_private)
       decrypt_fragments<REP>(slot(0), BATCH ? slot(0)->rk : a.rk, stage(0), Ts, BATCH && a.aes_pair);
   }
   int esc = 0;
@@ -382,7 +367,7 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
       if constexpr (PACK != 0)
         load_packed<PACK>(slot((it + 1) % 3), land, bars + (buf ^ 1));
       else
-        load_fragments<PUBIMG>(slot((it + 1) % 3), stage(buf ^ 1), bars + (buf ^ 1));
+        load_fragments(slot((it + 1) % 3), stage(buf ^ 1), bars + (buf ^ 1));
     }
     const int k = K >= 0 ? K : sl->k;
     const int npub = 63 - k;
@@ -553,7 +538,7 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
       if constexpr (PACK != 0)
         wait_packed<PACK>(slot((it + 1) % 3), bars + (buf ^ 1), phase[buf ^ 1], lost);
       else
-        wait_fragments<PUBIMG>(slot((it + 1) % 3), bars + (buf ^ 1), phase[buf ^ 1], lost);
+        wait_fragments(slot((it + 1) % 3), bars + (buf ^ 1), phase[buf ^ 1], lost);
     }
     __syncthreads();                                                       // B
     {
@@ -579,7 +564,7 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
         __syncthreads();                                                   // B2
         unpack_tile<PACK>(slot((it + 1) % 3), land, stage(buf ^ 1));
       }
-    } else if (!PUBIMG && nxt < ntiles && !a.plain_private) {
+    } else if (nxt < ntiles && !a.plain_private) {
       decrypt_fragments<REP>(slot((it + 1) % 3), BATCH ? slot((it + 1) % 3)->rk : a.rk, stage(buf ^ 1), Ts,
                         BATCH && a.aes_pair);
     }
@@ -627,18 +612,18 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
   }
 }
 
-template <int K, bool BATCH, bool PUBIMG = false, int PACK = 0, bool TC = false>
+template <int K, bool BATCH, int PACK = 0, bool TC = false>
 static cudaError_t launch_k(const TileArgs& a, cudaStream_t s, int sms, int per_sm) {
   static bool attr[kMaxAttrDevices];
   static int resident[kMaxAttrDevices];
-  constexpr int smem = TC ? kSmemBytesTc : (PACK ? kSmemBytesPacked : (BATCH || PUBIMG ? kSmemBytes : kSmemBytesRep));
-  cudaError_t e = smem_attr_once(restore_kernel<K, BATCH, PUBIMG, PACK, TC>, smem, attr);
+  constexpr int smem = TC ? kSmemBytesTc : (PACK ? kSmemBytesPacked : (BATCH ? kSmemBytes : kSmemBytesRep));
+  cudaError_t e = smem_attr_once(restore_kernel<K, BATCH, PACK, TC>, smem, attr);
   if (e != cudaSuccess) return e;
   const int ntiles = total_tiles(a);
-  const int r = resident_ctas(restore_kernel<K, BATCH, PUBIMG, PACK, TC>, kThreads, smem, resident);
+  const int r = resident_ctas(restore_kernel<K, BATCH, PACK, TC>, kThreads, smem, resident);
   const int cap = (per_sm >= 1 && per_sm < r ? per_sm : r) * sms;
   const int grid = ntiles < cap ? ntiles : cap;
-  if (grid > 0) restore_kernel<K, BATCH, PUBIMG, PACK, TC><<<grid, kThreads, smem, s>>>(a);
+  if (grid > 0) restore_kernel<K, BATCH, PACK, TC><<<grid, kThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -646,32 +631,26 @@ static cudaError_t launch_k(const TileArgs& a, cudaStream_t s, int sms, int per_
 // one CTA per SM (the operands and TMEM take what a second CTA would need)
 cudaError_t launch_restore_tc(const TileArgs& a, cudaStream_t s, int sms) {
   if (a.images || a.k < 0 || a.public_image || a.pack || a.plain_private || !a.tc_b) return cudaErrorInvalidValue;
-  if (a.k == 0) return launch_k<0, false, false, 0, true>(a, s, sms, 1);
-  if (a.k == 5) return launch_k<5, false, false, 0, true>(a, s, sms, 1);
-  return launch_k<-1, false, false, 0, true>(a, s, sms, 1);
+  if (a.k == 0) return launch_k<0, false, 0, true>(a, s, sms, 1);
+  if (a.k == 5) return launch_k<5, false, 0, true>(a, s, sms, 1);
+  return launch_k<-1, false, 0, true>(a, s, sms, 1);
 }
 
 // k is uniform over the launch when a.k >= 0; a.k < 0 (batches of mixed k) reads k per tile;
-// a.public_image (one image) selects the public-image form
+// one image in int16 storage, and the public-image form, go to the warp form
 cudaError_t launch_restore(const TileArgs& a, cudaStream_t s, int sms, int per_sm) {
   if (a.pack) {   // one image, packed streams in pub_in / priv_in
     if (a.images || a.k < 0 || a.public_image || (a.pack != 11 && a.pack != 8)) return cudaErrorInvalidValue;
-    if (a.pack == 11) return a.k == 5 ? launch_k<5, false, false, 11>(a, s, sms, per_sm)
-                                      : launch_k<-1, false, false, 11>(a, s, sms, per_sm);
-    return a.k == 5 ? launch_k<5, false, false, 8>(a, s, sms, per_sm) : launch_k<-1, false, false, 8>(a, s, sms, per_sm);
-  }
-  if (a.public_image) {
-    if (a.images || a.k < 0) return cudaErrorInvalidValue;
-    return a.k == 5 ? launch_k<5, false, true>(a, s, sms, per_sm) : launch_k<-1, false, true>(a, s, sms, per_sm);
+    if (a.pack == 11) return a.k == 5 ? launch_k<5, false, 11>(a, s, sms, per_sm)
+                                      : launch_k<-1, false, 11>(a, s, sms, per_sm);
+    return a.k == 5 ? launch_k<5, false, 8>(a, s, sms, per_sm) : launch_k<-1, false, 8>(a, s, sms, per_sm);
   }
   if (a.images) {
     if (a.k == 0) return launch_k<0, true>(a, s, sms, per_sm);
     if (a.k == 5) return launch_k<5, true>(a, s, sms, per_sm);
     return launch_k<-1, true>(a, s, sms, per_sm);
   }
-  if (a.k == 0) return launch_k<0, false>(a, s, sms, per_sm);
-  if (a.k == 5) return launch_k<5, false>(a, s, sms, per_sm);
-  return launch_k<-1, false>(a, s, sms, per_sm);
+  return launch_restore_warp(a, s, sms);
 }
 
 }  // namespace fds

@@ -1,0 +1,454 @@
+// Fused restore kernel in its warp form (defragmentation, Sect. 3.2, Fig. 3): CTR decryption of
+// the confidential fragment, merge by zigzag position, inverse 8x8 DCT, round half away from zero
+// (exact), clamp to [0, 255], of one image; and the public-image form (Sect. 6.5.1).
+//
+// As in the warp form of protect, each warp works on subtiles of 32 channel-blocks of its own,
+// with no barrier between warps after the AES table is filled.  It is bound by the issue of
+// instructions (4096 x 4096, k = 5: 47.5 M warp instructions = 37.7 us of issue slots against
+// 22.6 us for the 151 MB); two CTAs of six warps that met at three barriers per 192
+// channel-blocks issued in 61 % of the cycles, sixteen independent warps in 72 %.  Per subtile:
+//   1. its public part has arrived (bulk copy on the warp's mbarrier); two columns at a time the
+//      coefficients are gathered, converted and transformed (the loads of the next two stay
+//      behind: with all 64 in flight the kernel spilled 200 bytes and took 78 us); the buffer is
+//      free, so the next subtile's public part starts loading
+//   2. row butterflies, round and clamp, bytes into the warp's pixel buffer; a row in which some
+//      lane has a value within the error guard of a half-integer marks those values
+//   3. marked values are decided exactly by the whole warp at once (round_warp_inv): public
+//      coefficients from global memory, private ones from the decrypted buffer
+//   4. the ten whole blocks go out as 8-byte pieces, each lane its block's piece c; the two
+//      channel-blocks of a block shared with a neighbouring subtile as bytes
+// Private parts come in runs of subtiles whose keystream blocks fill whole warps (k = 5: four
+// subtiles, 96 blocks), one run ahead, and are decrypted in place.  The last two or so subtiles a
+// warp are claimed one by one, so that a CTA's warps end together.
+// Measured on 4096 x 4096: k = 5 79.0 -> 59.9 us.  Testing a row for values outside [0, 255] and
+// clamping only then (96 instructions a subtile less) measured no faster: 60.6 us.
+#include "fds_aux.h"
+#include "fds_warp.cuh"
+
+namespace fds {
+
+constexpr int kRPitch = 12 * 24;                  // one pixel row of a subtile: at most 12 blocks
+constexpr int kRPix = 0;
+constexpr int kRFrag = kRPix + 8 * kRPitch;       // public part, then the private parts of a run of
+constexpr int kRFragBytes = 6784;                 // subtiles, twice where that fits
+constexpr int kRBar = kRFrag + kRFragBytes;       // mbarriers: public, private (two)
+constexpr int kRSlot = kRBar + 3 * 8;             // what a warp looks at once per run (WarpSlot)
+constexpr int kRArea = (kRSlot + 32 + 31) & ~31;
+constexpr int kRWinBytes = 20 * kWins + 16 + 512 + 128;   // windows, subtile counter, folded c(m), (u, v) by zigzag
+constexpr int kRBelow = ((int)kTpairWin - 1024) / kRArea;
+constexpr int kRLow = (int)kTpairWin - kRBelow * kRArea;
+constexpr int kRAbove = kWarps > kRBelow ? kWarps - kRBelow : 0;
+constexpr int kRWin = (int)kTpairWin + kTpairBytes + kRAbove * kRArea;
+constexpr int kREnd = kRWin + kRWinBytes;
+static_assert(kREnd <= 227 * 1024, "restore (warp form) shared memory");
+
+// subtiles whose private parts are loaded and decrypted together (the fewest idle lanes), and
+// whether two such runs fit
+__host__ __device__ constexpr int run_tiles(int k) {
+  int best = 1, bn = 4 * (k + 1), bp = (bn + 31) / 32;
+  for (int g = 2; g <= 8; ++g) {
+    if ((63 - k) * 64 + 2 * g * (k + 1) * 64 > kRFragBytes) break;
+    const int n = g * 4 * (k + 1), p = (n + 31) / 32;
+    if (n * bp > bn * p) {
+      best = g;
+      bn = n;
+      bp = p;
+    }
+  }
+  return best;
+}
+__host__ __device__ constexpr bool run_twice(int k) { return (63 - k) * 64 + 2 * run_tiles(k) * (k + 1) * 64 <= kRFragBytes; }
+
+// bytes of a fragment part to shared memory: a bulk copy completing on bar (lane 0 announces it),
+// and a tail of 2-byte copies
+__device__ __forceinline__ void load_part(uint8_t* dst, const uint8_t* src, int bytes, int lane, uint64_t* bar) {
+  const int b16 = bytes & ~15;
+  if (lane == 0) {
+    mbar_expect_tx(bar, (uint32_t)b16);
+    if (b16) bulk_load(dst, src, (uint32_t)b16, bar);
+  }
+  const int j = b16 + 2 * lane;
+  if (j < bytes) *reinterpret_cast<uint16_t*>(dst + j) = *reinterpret_cast<const uint16_t*>(src + j);
+}
+
+// per-warp state that is not worth registers: counts, own subtiles still to claim, first window
+struct WarpSlot {
+  int ties, esc, fail;
+  uint32_t rt, rend, pad;
+  uint64_t wbase;
+};
+static_assert(sizeof(WarpSlot) == 32, "WarpSlot");
+
+// Exact rounding of pixel pos of one channel-block by the whole warp: pub / priv its public and
+// (decrypted) private coefficients.  As in protect (round_warp there), with 32-bit coordinates:
+// int16 coefficients of any value make |n_j| <= 2^22, so the constants carry 40 fraction bits and
+// the error bound is the sum of the |n_j|.
+__device__ __noinline__ int round_far_inv(const int (&n)[9], int* esc, bool* fail) { return exact_round(n, esc, fail); }
+template <bool PUBIMG>
+__device__ __forceinline__ int round_warp_inv(const int16_t* pub, const int16_t* priv, int k, int pos, const uint4* ctab,
+                                              const uint8_t* uv, int lane, WarpSlot* slot) {
+  const int y = pos >> 3, x = pos & 7;
+  uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int z = 2 * lane + i, t = uv[z], u = t >> 3, v = t & 7;
+    const int q = z <= k ? (PUBIMG ? (z == 0 ? 1024 : 0) : priv[z]) : __ldg(pub + z - k - 1);
+    const int a = u ? (2 * y + 1) * u : 4, b = v ? (2 * x + 1) * v : 4;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint4 f = ctab[(h ? a + b : a - b) & 31];            // +-1 in one 16-bit field
+      const uint32_t fw[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int lo = (int16_t)(fw[j] & 0xffffu), hi = (int)(fw[j] - (uint32_t)lo) >> 16;
+        w[2 * j] += (uint32_t)(q * lo);
+        w[2 * j + 1] += (uint32_t)(q * hi);
+      }
+    }
+  }
+  int n[9];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) n[j] = (int)__reduce_add_sync(0xffffffffu, w[j]);
+  n[8] = 0;
+  constexpr int kFrac = 40;
+  long long d = ((long long)n[0] + 4) << kFrac;
+  long long err = 0;
+#pragma unroll
+  for (int j = 1; j < 8; ++j) {
+    d += (long long)n[j] * (c_cos_q62[j - 1] >> (62 - kFrac));
+    err += n[j] < 0 ? -n[j] : n[j];
+  }
+  // d / 2^43 = p + 1/2
+  const int q = (int)(d >> (kFrac + 3));
+  const long long rem = d & ((8ll << kFrac) - 1);
+  if (err == 0) return rem == 0 && q <= 0 ? q - 1 : q;      // rational: a tie goes away from zero
+  if (rem > err && rem < (8ll << kFrac) - err) return q;
+  int e = 0;
+  bool fail = false;
+  const int r = round_far_inv(n, &e, &fail);
+  if (lane == 0) {
+    slot->esc += e;
+    slot->fail |= fail;
+  }
+  return r;
+}
+
+template <int K, bool PUBIMG>
+__global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __grid_constant__ TileArgs a) {
+  extern __shared__ __align__(128) uint8_t smem_cta[];
+  const uint32_t win0 = smem_u32(smem_cta);
+  if (win0 > (uint32_t)kRLow) {   // see the launcher
+    if (threadIdx.x == 0 && a.counters) atomicAdd(&a.counters[2], 1ull);
+    return;
+  }
+  const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+  uint8_t* area = smem_cta + ((warp < kRBelow ? (uint32_t)(kRLow + warp * kRArea)
+                                              : kTpairWin + kTpairBytes + (uint32_t)(warp - kRBelow) * kRArea) -
+                              win0);
+  uint8_t* const pix = area + kRPix;
+  uint64_t* const bars = reinterpret_cast<uint64_t*>(area + kRBar);
+  uint32_t* wins = reinterpret_cast<uint32_t*>(smem_cta + (kRWin - win0));
+  uint32_t* const next = wins + 5 * kWins;
+  uint4* const ctab = reinterpret_cast<uint4*>(next + 4);
+  uint8_t* const uv = reinterpret_cast<uint8_t*>(ctab + 32);
+  const int k = K >= 0 ? K : a.k;
+  const int npub = 63 - k;
+  const uint32_t nb = 4u * (uint32_t)(k + 1);       // keystream blocks per subtile
+  const int G = K >= 0 ? run_tiles(K >= 0 ? K : 0) : a.aes_pair & 15;
+  const bool twice = K >= 0 ? run_twice(K >= 0 ? K : 0) : (a.aes_pair & 16) != 0;
+  const bool cipher = !PUBIMG && !a.plain_private;
+  uint8_t* const pubst = area + kRFrag;
+  uint8_t* const privst = pubst + kWCb * 2 * npub;
+  const int priv_half = twice ? G * 64 * (k + 1) : 0;
+  const uint32_t ncb = 3u * (uint32_t)a.nblocks, nsub = (ncb + 31u) >> 5;
+  const int act = a.groups;       // working warps of each CTA
+  const uint32_t s0 = (uint32_t)((uint64_t)nsub * blockIdx.x / gridDim.x);
+  const uint32_t s1 = (uint32_t)((uint64_t)nsub * (blockIdx.x + 1) / gridDim.x);
+  const uint32_t iv8 = (uint32_t)a.iv_lo & 255u;
+  uint64_t wbase = (iv8 + (uint64_t)s0 * nb) >> 8;
+  const uint64_t wlast = (iv8 + (uint64_t)s1 * nb - 1) >> 8;
+  const bool table = wlast - wbase < kWins;         // the CTA's windows fit the table
+  // the CTA's subtiles: the first ones as runs of G for each warp in turn, the last (about two a
+  // warp) one by one to whichever warp is free
+  const uint32_t per = (s1 - s0) / (uint32_t)act;
+  const uint32_t own = per > 2 ? (per - 2) / G * G : 0;
+  const uint32_t sfree = s0 + own * act;
+  WarpSlot* const slot = reinterpret_cast<WarpSlot*>(area + kRSlot);
+  if (lane == 0) {
+    slot->ties = slot->esc = slot->fail = 0;
+    slot->rt = s0 + own * (uint32_t)warp;
+    slot->rend = slot->rt + own;
+  }
+  // claim the next run: its first subtile and length (start >= s1: none left)
+  auto claim = [&](int& cnt) -> uint32_t {
+    uint32_t t = 0;
+    if (lane == 0) {
+      t = slot->rt;
+      if (t < slot->rend)
+        slot->rt = t + G;
+      else
+        t = atomicAdd(next, 1u) | 0x80000000u;
+    }
+    t = __shfl_sync(0xffffffffu, t, 0);
+    cnt = t >> 31 ? 1 : G;
+    return t & 0x7fffffffu;
+  };
+  auto nof = [&](uint32_t t) { return (int)min(32u, ncb - 32u * t); };
+  auto load_pub = [&](uint32_t t) {
+    load_part(pubst, reinterpret_cast<const uint8_t*>(a.pub_in) + (uint64_t)t * (64u * npub), nof(t) * 2 * npub, lane, bars);
+  };
+  auto load_priv = [&](uint32_t t, int cnt, int half) {
+    load_part(privst + half * priv_half, a.priv_in + (uint64_t)t * (64u * (k + 1)),
+              ((cnt - 1) * 32 + nof(t + cnt - 1)) * 2 * (k + 1), lane, bars + 1 + half);
+  };
+
+  if (threadIdx.x == 0) *next = sfree;
+  if (lane == 0) {
+    mbar_init(bars);
+    mbar_init(bars + 1);
+    mbar_init(bars + 2);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
+    const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
+    const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
+    ctab[lane] = make_uint4(f >> 1 == 0 ? one : 0u, f >> 1 == 1 ? one : 0u, f >> 1 == 2 ? one : 0u, f >> 1 == 3 ? one : 0u);
+  }
+  if (threadIdx.x < 64) uv[zigzag_of((int)threadIdx.x >> 3, (int)threadIdx.x & 7)] = (uint8_t)threadIdx.x;
+  if (cipher) fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
+  __syncthreads();
+  if (cipher) {
+    if (table) {
+      const int i = (int)threadIdx.x;
+      if ((uint32_t)(i & ~31) <= wlast - wbase) put_window(a, wbase + i, (uint32_t)i <= wlast - wbase ? i : -1, wins);
+      __syncthreads();
+    } else {
+      wins += 10 * warp;
+      wbase = ~0ull - 1;
+    }
+    if (lane == 0) slot->wbase = wbase;
+    __syncwarp();
+  }
+  bool lost = false;
+  uint32_t ph = 0;                         // phases: bit 0 public, bits 1 and 2 the private buffers
+  int cnt = 0, cnt_n = 0, half = 0;
+  uint32_t run = s1, run_n = s1;
+  if (warp < act) {
+    run = claim(cnt);
+    if (run < s1) {
+      load_pub(run);
+      if (!PUBIMG) load_priv(run, cnt, 0);
+    }
+  }
+
+  while (run < s1) {
+    run_n = claim(cnt_n);
+    if (!PUBIMG) {
+      if (twice && run_n < s1) {
+        fence_proxy_async();               // the buffer was decrypted in place
+        __syncwarp();
+        load_priv(run_n, cnt_n, half ^ 1);
+      }
+      if (!__all_sync(0xffffffffu, mbar_wait(bars + 1 + half, (ph >> (1 + half)) & 1u))) {
+        lost = true;
+        break;
+      }
+      __syncwarp();
+      ph ^= 2u << half;
+      if (cipher) {
+        uint8_t* const buf = privst + half * priv_half;
+        const uint32_t total = (uint32_t)cnt * nb;
+        const uint64_t b0 = iv8 + (uint64_t)run * nb;     // from the IV's window
+        uint64_t wbase = slot->wbase;
+        if (!table && ((b0 >> 8) < wbase || ((b0 + total - 1) >> 8) > wbase + 1)) {
+          wbase = b0 >> 8;
+          __syncwarp();
+          put_window(a, wbase + (lane & 1), lane < 2 ? lane : -1, wins);
+          if (lane == 0) slot->wbase = wbase;
+          __syncwarp();
+        }
+        const PairLanes lc = pair_lanes();
+#pragma unroll 1
+        for (uint32_t i = lane; i < total; i += 32) {
+          const uint64_t b = b0 + i;
+          const uint32_t* src = wins + 5 * (uint32_t)((b >> 8) - wbase);
+          const uint32_t w[5] = {src[0], src[1], src[2], src[3], src[4]};
+          uint32_t s[4];
+          aes_from_window(w, (uint32_t)b & 255u, a.rk, lc, s);
+          uint4* p = reinterpret_cast<uint4*>(buf + 16 * i);
+          uint4 d = *p;
+          d.x ^= s[0];
+          d.y ^= s[1];
+          d.z ^= s[2];
+          d.w ^= s[3];
+          *p = d;
+        }
+      }
+    }
+#pragma unroll 1
+    for (int ti = 0; ti < cnt; ++ti) {
+      const uint32_t t = run + ti;
+      const int n = nof(t);
+      const CbPos at = cb_pos(a, 32u * t + lane);
+      if (!__all_sync(0xffffffffu, mbar_wait(bars, ph & 1u))) {   // gave up: nothing more is written
+        lost = true;
+        break;
+      }
+      __syncwarp();
+      ph ^= 1u;
+      const int16_t* pub_cb = reinterpret_cast<const int16_t*>(pubst) + lane * npub;
+      const int16_t* priv_cb = reinterpret_cast<const int16_t*>(privst + half * priv_half) + (ti * kWCb + lane) * (k + 1);
+      float2 G2[8][4];
+      float l1 = 0.0f;  // sum |F|, exact (integers below 2^24)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {        // two columns: gathered and transformed
+        float2 col[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int z0 = zigzag_of(u, 2 * j), z1 = zigzag_of(u, 2 * j + 1);
+          const int q0 = z0 <= k ? (PUBIMG ? (z0 == 0 ? 1024 : 0) : priv_cb[z0]) : pub_cb[z0 - k - 1];
+          const int q1 = z1 <= k ? (PUBIMG ? 0 : priv_cb[z1]) : pub_cb[z1 - k - 1];
+          col[u] = add2(make_float2(__int_as_float(kMagicBits + q0), __int_as_float(kMagicBits + q1)),
+                        make_float2(-kMagic, -kMagic));
+          l1 += fabsf(col[u].x);
+          l1 += fabsf(col[u].y);
+        }
+        idct8_2(col);
+#pragma unroll
+        for (int y = 0; y < 8; ++y) G2[y][j] = col[y];
+        if (j < 3) asm volatile("" ::: "memory");   // the next columns' loads stay behind
+      }
+      __syncwarp();                        // the public part is read: the next one starts loading
+      {
+        const uint32_t tn = ti + 1 < cnt ? t + 1 : run_n;
+        if (tn < s1) load_pub(tn);
+      }
+      const uint32_t c0 = __shfl_sync(0xffffffffu, at.c, 0);
+      uint8_t* const out = pix + 8 * (c0 + lane - at.c) + at.c;
+      const float thr = lane < n ? 0.5f - l1 * kGuardInvScale : 1.0f;
+      uint32_t mlo = 0, mhi = 0;
+#pragma unroll
+      for (int y = 0; y < 8; ++y) {
+        float row[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          row[2 * j] = G2[y][j].x;
+          row[2 * j + 1] = G2[y][j].y;
+        }
+        idct8(row);
+        float2 r[4];
+        float big = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float2 pc = make_float2(fminf(fmaxf(row[2 * j], 0.0f), 255.0f), fminf(fmaxf(row[2 * j + 1], 0.0f), 255.0f));
+          const float2 yv = add2(pc, make_float2(kMagic, kMagic));
+          r[j] = sub2(pc, add2(yv, make_float2(-kMagic, -kMagic)));
+          big = fmaxf(fmaxf(big, fabsf(r[j].x)), fabsf(r[j].y));
+          out[y * kRPitch + 6 * j] = (uint8_t)__float_as_uint(yv.x);
+          out[y * kRPitch + 6 * j + 3] = (uint8_t)__float_as_uint(yv.y);
+        }
+        if (__any_sync(0xffffffffu, big > thr)) {   // rare: a near tie in this row
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int l = 0; l < 2; ++l)
+              if (fabsf(l ? r[j].y : r[j].x) > thr) {
+                if (8 * y + 2 * j + l < 32)
+                  mlo |= 1u << (8 * y + 2 * j + l);
+                else
+                  mhi |= 1u << (8 * y + 2 * j + l - 32);
+              }
+        }
+      }
+      // near ties, one after another, decided by the whole warp
+      for (uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0); who; who &= who - 1) {
+        const int src = __ffs(who) - 1;
+        uint64_t mask = (uint64_t)__shfl_sync(0xffffffffu, mhi, src) << 32 | __shfl_sync(0xffffffffu, mlo, src);
+        const int16_t* pub_s = a.pub_in + (uint64_t)(32u * t + src) * npub;
+        const int16_t* priv_s = priv_cb + (src - lane) * (k + 1);
+        if (lane == 0) slot->ties += __popcll(mask);
+        for (; mask; mask &= mask - 1) {
+          const int pos = __ffsll((long long)mask) - 1;
+          const int p = round_warp_inv<PUBIMG>(pub_s, priv_s, k, pos, ctab, uv, lane, slot);
+          if (lane == src) out[(pos >> 3) * kRPitch + 3 * (pos & 7)] = (uint8_t)(p < 0 ? 0 : (p > 255 ? 255 : p));
+        }
+      }
+      if (!PUBIMG && !twice) fence_proxy_async();
+      __syncwarp();                        // the pixel rows are complete
+      if (!PUBIMG && !twice && ti + 1 == cnt && run_n < s1) load_priv(run_n, cnt_n, 0);
+      // whole blocks: lane's 8-byte piece c of its block in 8 rows; a block shared with the next
+      // or previous subtile: its channels' bytes
+      const uint64_t pitch = 3ull * (uint64_t)a.width;
+      uint8_t* const blk = a.pixels_out + ((uint64_t)at.by * (8 * pitch) + 24ull * at.bx);
+      const int b0l = lane - (int)at.c;
+      const bool whole = b0l >= 0 && b0l + 2 < n;
+      if (whole) {
+        uint8_t* dst = blk + 8 * at.c;
+        const uint8_t* src = pix + 8 * (c0 + lane);
+#pragma unroll
+        for (int y = 0; y < 8; ++y) {
+          *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(src + y * kRPitch);
+          dst += pitch;
+        }
+      }
+      for (uint32_t who = __ballot_sync(0xffffffffu, !whole && lane < n); who; who &= who - 1) {
+        const int src = __ffs(who) - 1;
+        const uint32_t sc = __shfl_sync(0xffffffffu, at.c, src);
+        uint8_t* const sb = reinterpret_cast<uint8_t*>(__shfl_sync(0xffffffffu, (unsigned long long)blk, src));
+        const uint8_t* sp = pix + 8 * (c0 + src - sc) + sc;
+        const int x3 = 3 * (lane & 7), y0 = lane >> 3;
+        sb[y0 * pitch + x3 + sc] = sp[y0 * kRPitch + x3];
+        sb[(y0 + 4) * pitch + x3 + sc] = sp[(y0 + 4) * kRPitch + x3];
+      }
+      __syncwarp();                        // the pixel buffer may be written again
+    }
+    if (lost) break;
+    run = run_n;
+    cnt = cnt_n;
+    if (twice) half ^= 1;
+  }
+  if (lost) {                              // copies still in flight
+    mbar_wait(bars, ph & 1u);
+    if (!PUBIMG && twice && run_n < s1) mbar_wait(bars + 1 + (half ^ 1), (ph >> (1 + (half ^ 1))) & 1u);
+  }
+  if (lane == 0 && a.counters) {
+    if (slot->ties) atomicAdd(&a.counters[0], (unsigned long long)slot->ties);
+    if (slot->esc) atomicAdd(&a.counters[1], (unsigned long long)slot->esc);
+    if (slot->fail || lost) atomicAdd(&a.counters[2], 1ull);
+  }
+}
+
+template <int K, bool PUBIMG>
+static cudaError_t launch_w(const TileArgs& a, cudaStream_t s, int sms) {
+  static bool attr[kMaxAttrDevices];
+  static bool window_ok[kMaxAttrDevices];
+  int dev = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxAttrDevices) return cudaErrorInvalidDevice;
+  if (!window_ok[dev]) {
+    if ((e = smem_window_start_ok(restore_warp_kernel<K, PUBIMG>, (uint32_t)kRLow)) != cudaSuccess) return e;
+    window_ok[dev] = true;
+  }
+  e = smem_attr_once(restore_warp_kernel<K, PUBIMG>, kREnd, attr);
+  if (e != cudaSuccess) return e;
+  TileArgs b = a;
+  const long long nsub = (3ll * a.nblocks + 31) / 32;
+  const int grid = (int)(nsub < sms ? nsub : sms);
+  const long long per = (nsub + grid - 1) / (grid ? grid : 1);
+  b.groups = (int)(per < kWarps ? per : kWarps);
+  bx_division(b);
+  b.aes_pair = run_tiles(a.k) | (run_twice(a.k) ? 16 : 0);
+  if (grid > 0) restore_warp_kernel<K, PUBIMG><<<grid, kWarps * 32, kREnd, s>>>(b);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_restore_warp(const TileArgs& a, cudaStream_t s, int sms) {
+  if (a.images || a.pack || a.k < 0 || a.k > 63) return cudaErrorInvalidValue;
+  if (a.public_image) return a.k == 5 ? launch_w<5, true>(a, s, sms) : launch_w<-1, true>(a, s, sms);
+  if (a.k == 0) return launch_w<0, false>(a, s, sms);
+  if (a.k == 5) return launch_w<5, false>(a, s, sms);
+  return launch_w<-1, false>(a, s, sms);
+}
+
+}  // namespace fds
