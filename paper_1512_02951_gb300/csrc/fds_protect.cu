@@ -658,11 +658,7 @@ cudaError_t launch_protect(const TileArgs& a, cudaStream_t s, bool debug, int sm
                     : launch_k<-1, false, false, 8>(a, s, sms, per_sm);
   }
   if (debug) return launch_k<-1, true, false>(a, s, sms, per_sm);
-  if (a.images) {
-    if (a.k == 0) return launch_k<0, false, true>(a, s, sms, per_sm);
-    if (a.k == 5) return launch_k<5, false, true>(a, s, sms, per_sm);
-    return launch_k<-1, false, true>(a, s, sms, per_sm);
-  }
+  if (a.images) return launch_protect_plan(a, s, sms, per_sm);
   return launch_protect_warp(a, s, sms);
 }
 

@@ -77,16 +77,15 @@ struct PixAt {
 // Else 8-byte pieces: lane's piece c of its block in 8 rows, then the pieces of the two boundary
 // blocks that other subtiles' lanes own.
 template <bool BULK>
-__device__ __forceinline__ PixAt load_subtile(const TileArgs& a, const CbPos& p, uint32_t n, int lane, uint32_t pix,
-                                              uint64_t* bar) {
-  const uint64_t pitch = 3ull * (uint64_t)a.width;
+__device__ __forceinline__ PixAt load_subtile(const uint8_t* img, uint64_t pitch, uint32_t bx_count, const CbPos& p,
+                                              uint32_t n, int lane, uint32_t pix, uint64_t* bar) {
   const uint32_t c0 = __shfl_sync(0xffffffffu, p.c, 0);
   PixAt at;
   at.c = p.c;
   if constexpr (BULK) {
     const uint32_t bx0 = __shfl_sync(0xffffffffu, p.bx, 0), by0 = __shfl_sync(0xffffffffu, p.by, 0);
     const uint32_t nblk = (c0 + n + 2) / 3;                       // blocks the subtile touches
-    const uint32_t m0 = min(nblk, (uint32_t)a.bx_count - bx0);    // in the first block row
+    const uint32_t m0 = min(nblk, bx_count - bx0);    // in the first block row
     const uint32_t odd = (uint32_t)pitch & 8u;                    // skew change from row to row
     const uint32_t sk0 = (24u * bx0) & 8u;                        // skew of even rows, first run
     const uint32_t seg1 = (24u * m0 + 8u + 15u) & ~15u;           // where the second run starts
@@ -106,7 +105,7 @@ __device__ __forceinline__ PixAt load_subtile(const TileArgs& a, const CbPos& p,
       if (on)
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
                          pix + y * kWPixPitch + (second ? seg1 : 0u)),
-                     "l"(a.pixels_in + lo), "r"(bytes), "r"(smem_u32(bar))
+                     "l"(img + lo), "r"(bytes), "r"(smem_u32(bar))
                      : "memory");
     }
     const bool in1 = p.by != by0;
@@ -115,7 +114,7 @@ __device__ __forceinline__ PixAt load_subtile(const TileArgs& a, const CbPos& p,
     at.odd = base + (sk ^ odd);
   } else {
     const uint64_t off = (uint64_t)p.by * (8 * pitch) + 24ull * p.bx;
-    const uint8_t* src = a.pixels_in + off + 8 * p.c;
+    const uint8_t* src = img + off + 8 * p.c;
     const uint32_t dst = pix + 8 * (c0 + lane);
     if ((uint32_t)lane < n) {
 #pragma unroll
@@ -132,7 +131,7 @@ __device__ __forceinline__ PixAt load_subtile(const TileArgs& a, const CbPos& p,
       const uint32_t q = head ? sl : sl - c0 + (3 - e1);            // piece of the block
       const uint32_t j = head ? sl : c0 + 32 + (sl - c0);           // its place in the row
       asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(pix + y * kWPixPitch + 8 * j),
-                   "l"(a.pixels_in + eoff + y * pitch + 8 * q)
+                   "l"(img + eoff + y * pitch + 8 * q)
                    : "memory");
     }
     cp_async_commit();
@@ -217,6 +216,120 @@ __device__ __forceinline__ int round_warp(const uint8_t* px, uint64_t pitch, int
   return r;
 }
 
+// Row butterflies of a lane's channel-block from its pixel buffer: outputs as pairs of columns
+// (0, 4), (1, 2), (3, 5), (6, 7), so that the column pass runs on two columns per packed f32x2
+// instruction; returns the row passes' error weight
+__device__ __forceinline__ float transform_rows(const uint8_t* px_even, const uint8_t* px_odd, uint32_t c, float2 (&P)[8][4]) {
+  float V = 0.0f;
+#pragma unroll
+  for (int y = 0; y < 8; ++y) {
+    const uint2* rp = reinterpret_cast<const uint2*>((y & 1 ? px_odd : px_even) + y * kWPixPitch);
+    const uint2 w01 = rp[0], w23 = rp[1], w45 = rp[2];
+    const uint32_t r[7] = {w01.x, w01.y, w23.x, w23.y, w45.x, w45.y, 0u};
+    uint32_t w[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) w[i] = __funnelshift_r(r[i], r[i + 1], 8 * c);
+    float X[8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+      const int byte = 3 * x;
+      X[x] = __int_as_float(__byte_perm(w[byte >> 2], 0x4B000000u, 0x7440u | (byte & 3)));
+    }
+    float fr[8];
+    V += dct8_row_bytes_w(X, fr);
+    P[y][0] = make_float2(fr[0], fr[4]);
+    P[y][1] = make_float2(fr[1], fr[2]);
+    P[y][2] = make_float2(fr[3], fr[5]);
+    P[y][3] = make_float2(fr[6], fr[7]);
+  }
+  return V;
+}
+
+// Column butterflies, rounding and staging of a lane's channel-block (z = 0 .. k at priv_cb, the
+// rest at pub_cb); bit 8 u + v of mhi:mlo marks a value within the error guard of a half-integer
+// (none where the lane is not live)
+__device__ __forceinline__ void stage_columns(const float2 (&P)[8][4], float V, int k, bool live, int16_t* pub_cb,
+                                              int16_t* priv_cb, uint32_t& mlo, uint32_t& mhi) {
+  auto put = [&](int u, int v, uint32_t q) {
+    const int z = zigzag_of(u, v);
+    if (z <= k)
+      priv_cb[z] = (int16_t)q;
+    else
+      pub_cb[z - k - 1] = (int16_t)q;
+  };
+  mlo = mhi = 0;
+  float thr = 1.0f;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {          // a pair of columns: transformed, rounded and staged
+    float2 col[8];
+#pragma unroll
+    for (int y = 0; y < 8; ++y) col[y] = P[y][j];
+    if (j == 0) {
+      const float W = dct8_rat_w2(col);
+      if (live) thr = 0.5f - fminf(fmaf(V, kGuardV, fmaf(W, kGuardW, kGuardU)), kGuardFwd);
+    } else {
+      dct8_2<false, false>(col);
+    }
+    float big = 0.0f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if ((u == 0 || u == 4) && j == 0) {
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+          const int v = pair_col(0, l);
+          const int T = __float_as_int((l ? col[u].y : col[u].x) + kMagic) - kMagicBits;  // 8 F, exact
+          put(u, v, (uint32_t)((u == 0 && v == 0) ? ((T + 4) >> 3) + 1024 : (T + 4 - (T < 0 ? 1 : 0)) >> 3));
+        }
+        col[u] = make_float2(0.0f, 0.0f);
+      } else {
+        const float2 yv = add2(col[u], make_float2(kMagic, kMagic));
+        col[u] = sub2(col[u], add2(yv, make_float2(-kMagic, -kMagic)));
+        put(u, pair_col(j, 0), __float_as_uint(yv.x));   // low 16 bits: the int16 result
+        put(u, pair_col(j, 1), __float_as_uint(yv.y));
+        big = fmaxf(fmaxf(big, fabsf(col[u].x)), fabsf(col[u].y));
+      }
+    }
+    if (__any_sync(0xffffffffu, big > thr)) {   // rare: a near tie in these columns
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+          const int v = pair_col(j, l);
+          if (fabsf(l ? col[u].y : col[u].x) > thr) {
+            if (8 * u + v < 32)
+              mlo |= 1u << (8 * u + v);
+            else
+              mhi |= 1u << (8 * u + v - 32);
+          }
+        }
+    }
+  }
+}
+
+// The marked values of the subtile whose first channel-block is cb0, one after another, each
+// decided by the whole warp and staged by its lane (c, pub_cb, priv_cb: the lane's own)
+__device__ __forceinline__ void decide_ties(const uint8_t* img, uint64_t pitch, uint32_t bx_count, uint32_t cb0, uint32_t c,
+                                            int k, uint32_t mlo, uint32_t mhi, int16_t* pub_cb, int16_t* priv_cb,
+                                            const uint4* ctab, int lane, int& nties, int& esc,
+                                            bool& fail) {
+  for (uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0); who; who &= who - 1) {
+    const int src = __ffs(who) - 1;
+    uint64_t mask = (uint64_t)__shfl_sync(0xffffffffu, mhi, src) << 32 | __shfl_sync(0xffffffffu, mlo, src);
+    const uint32_t sc = __shfl_sync(0xffffffffu, c, src);
+    const uint32_t b = (cb0 + src) / 3, by = b / bx_count;
+    const uint8_t* blk = img + (uint64_t)by * (8 * pitch) + 24ull * (b - by * bx_count);
+    nties += __popcll(mask);
+    for (; mask; mask &= mask - 1) {
+      const int pos = __ffsll((long long)mask) - 1;
+      int e = 0;
+      const int q = round_warp(blk + sc, pitch, pos, ctab, lane, e, fail);
+      esc += e;
+      const int z = zigzag_of(pos >> 3, pos & 7);
+      if (lane == src) *(z <= k ? priv_cb + z : pub_cb + (z - k - 1)) = (int16_t)q;
+    }
+  }
+}
+
 template <int K, bool BULK>
 __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __grid_constant__ TileArgs a) {
   extern __shared__ __align__(128) uint8_t smem_cta[];
@@ -263,7 +376,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
   __syncwarp();
   PixAt at{};
   uint32_t phase = 0;
-  if (t < tend) at = load_subtile<BULK>(a, cb_pos(a, 32u * t + lane), min(32u, ncb - 32u * t), lane, pix, bar);
+  if (t < tend) at = load_subtile<BULK>(a.pixels_in, pitch, (uint32_t)a.bx_count, cb_pos(a, 32u * t + lane), min(32u, ncb - 32u * t), lane, pix, bar);
   if (threadIdx.x == 0) *next = s0 + act;
   if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
     const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
@@ -312,104 +425,16 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
     const uint8_t* px_even = area + kWPix + at.even;
     const uint8_t* px_odd = area + kWPix + at.odd;
     float2 P[8][4];
-    float V = 0.0f;
-#pragma unroll
-    for (int y = 0; y < 8; ++y) {
-      const uint2* rp = reinterpret_cast<const uint2*>((y & 1 ? px_odd : px_even) + y * kWPixPitch);
-      const uint2 w01 = rp[0], w23 = rp[1], w45 = rp[2];
-      const uint32_t r[7] = {w01.x, w01.y, w23.x, w23.y, w45.x, w45.y, 0u};
-      uint32_t w[6];
-#pragma unroll
-      for (int i = 0; i < 6; ++i) w[i] = __funnelshift_r(r[i], r[i + 1], 8 * c);
-      float X[8];
-#pragma unroll
-      for (int x = 0; x < 8; ++x) {
-        const int byte = 3 * x;
-        X[x] = __int_as_float(__byte_perm(w[byte >> 2], 0x4B000000u, 0x7440u | (byte & 3)));
-      }
-      float fr[8];
-      V += dct8_row_bytes_w(X, fr);
-      P[y][0] = make_float2(fr[0], fr[4]);
-      P[y][1] = make_float2(fr[1], fr[2]);
-      P[y][2] = make_float2(fr[3], fr[5]);
-      P[y][3] = make_float2(fr[6], fr[7]);
-    }
+    const float V = transform_rows(px_even, px_odd, c, P);
     __syncwarp();                          // the pixel buffer is read: the next subtile's load starts
-    if (tn < tend) at = load_subtile<BULK>(a, cb_pos(a, 32u * tn + lane), min(32u, ncb - 32u * tn), lane, pix, bar);
+    if (tn < tend) at = load_subtile<BULK>(a.pixels_in, pitch, (uint32_t)a.bx_count, cb_pos(a, 32u * tn + lane), min(32u, ncb - 32u * tn), lane, pix, bar);
     bulk_wait_read_all();                  // the staging area may be written again
     __syncwarp();
     int16_t* pub_cb = pubst + lane * npub;
     int16_t* priv_cb = reinterpret_cast<int16_t*>(privst) + (acc * kWCb + lane) * (k + 1);
-    auto put = [&](int u, int v, uint32_t q) {
-      const int z = zigzag_of(u, v);
-      if (z <= k)
-        priv_cb[z] = (int16_t)q;
-      else
-        pub_cb[z - k - 1] = (int16_t)q;
-    };
-    uint32_t mlo = 0, mhi = 0;
-    float thr = 1.0f;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {          // a pair of columns: transformed, rounded and staged
-      float2 col[8];
-#pragma unroll
-      for (int y = 0; y < 8; ++y) col[y] = P[y][j];
-      if (j == 0) {
-        const float W = dct8_rat_w2(col);
-        if ((uint32_t)lane < n) thr = 0.5f - fminf(fmaf(V, kGuardV, fmaf(W, kGuardW, kGuardU)), kGuardFwd);
-      } else {
-        dct8_2<false, false>(col);
-      }
-      float big = 0.0f;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        if ((u == 0 || u == 4) && j == 0) {
-#pragma unroll
-          for (int l = 0; l < 2; ++l) {
-            const int v = pair_col(0, l);
-            const int T = __float_as_int((l ? col[u].y : col[u].x) + kMagic) - kMagicBits;  // 8 F, exact
-            put(u, v, (uint32_t)((u == 0 && v == 0) ? ((T + 4) >> 3) + 1024 : (T + 4 - (T < 0 ? 1 : 0)) >> 3));
-          }
-          col[u] = make_float2(0.0f, 0.0f);
-        } else {
-          const float2 yv = add2(col[u], make_float2(kMagic, kMagic));
-          col[u] = sub2(col[u], add2(yv, make_float2(-kMagic, -kMagic)));
-          put(u, pair_col(j, 0), __float_as_uint(yv.x));   // low 16 bits: the int16 result
-          put(u, pair_col(j, 1), __float_as_uint(yv.y));
-          big = fmaxf(fmaxf(big, fabsf(col[u].x)), fabsf(col[u].y));
-        }
-      }
-      if (__any_sync(0xffffffffu, big > thr)) {   // rare: a near tie in these columns
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-#pragma unroll
-          for (int l = 0; l < 2; ++l) {
-            const int v = pair_col(j, l);
-            if (fabsf(l ? col[u].y : col[u].x) > thr) {
-              if (8 * u + v < 32)
-                mlo |= 1u << (8 * u + v);
-              else
-                mhi |= 1u << (8 * u + v - 32);
-            }
-          }
-      }
-    }
-    // near ties, one after another, decided by the whole warp
-    for (uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0); who; who &= who - 1) {
-      const int src = __ffs(who) - 1;
-      uint64_t mask = (uint64_t)__shfl_sync(0xffffffffu, mhi, src) << 32 | __shfl_sync(0xffffffffu, mlo, src);
-      const uint32_t sc = __shfl_sync(0xffffffffu, c, src);
-      const uint8_t* blk = a.pixels_in + block_offset(a.width, (int)((32u * t + src) / 3));
-      nties += __popcll(mask);
-      for (; mask; mask &= mask - 1) {
-        const int pos = __ffsll((long long)mask) - 1;
-        int e = 0;
-        const int q = round_warp(blk + sc, pitch, pos, ctab, lane, e, fail);
-        esc += e;
-        const int z = zigzag_of(pos >> 3, pos & 7);
-        if (lane == src) *(z <= k ? priv_cb + z : pub_cb + (z - k - 1)) = (int16_t)q;
-      }
-    }
+    uint32_t mlo, mhi;
+    stage_columns(P, V, k, (uint32_t)lane < n, pub_cb, priv_cb, mlo, mhi);
+    decide_ties(a.pixels_in, pitch, (uint32_t)a.bx_count, 32u * t, c, k, mlo, mhi, pub_cb, priv_cb, ctab, lane, nties, esc, fail);
     fence_proxy_async();                   // staged coefficients, before the bulk store
     __syncwarp();
     if (lane == 0) store_run(reinterpret_cast<uint8_t*>(a.pub_out) + (uint64_t)t * (64u * npub), stage, (int)n * 2 * npub);
@@ -450,6 +475,152 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
   }
 }
 
+// ---- batches ---------------------------------------------------------------------------------
+
+constexpr int kPSlot = kWBar + 8;                 // two slots after the single-image area
+constexpr int kPWins = kPSlot + 2 * (int)sizeof(PlanSlot);   // the warp's two windows
+constexpr int kPArea = (kPWins + 40 + 31) & ~31;
+constexpr int kPBelow = ((int)kTpairWin - 1024) / kPArea;
+constexpr int kPLow = (int)kTpairWin - kPBelow * kPArea;
+constexpr int kPAbove = kWarps > kPBelow ? kWarps - kPBelow : 0;
+constexpr int kPTail = (int)kTpairWin + kTpairBytes + kPAbove * kPArea;   // counter, folded c(m)
+constexpr int kPEnd = kPTail + 16 + 512;
+static_assert(kPEnd <= 227 * 1024 && kPSlot % 8 == 0, "protect (batches) shared memory");
+
+// acc_tiles(k), at most a tile
+struct AccTable {
+  uint8_t n[64];
+};
+constexpr AccTable make_acc_table() {
+  AccTable t{};
+  for (int k = 0; k < 64; ++k) t.n[k] = (uint8_t)(acc_tiles(k) < kTileSubs ? acc_tiles(k) : kTileSubs);
+  return t;
+}
+static __constant__ AccTable c_acc = make_acc_table();
+
+// Protect of a batch: every tile of 64 blocks of every image, six subtiles a tile.  A CTA has a
+// run of the batch's tiles, taken by its warps one by one, the last few subtile by subtile; or
+// (a.dispenser) every warp takes tiles from one counter.
+template <int K>
+__global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __grid_constant__ TileArgs a) {
+  extern __shared__ __align__(128) uint8_t smem_cta[];
+  const uint32_t win0 = smem_u32(smem_cta);
+  if (win0 > (uint32_t)kPLow) {   // see the launcher
+    if (threadIdx.x == 0 && a.counters) atomicAdd(&a.counters[2], 1ull);
+    return;
+  }
+  const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+  uint8_t* area = smem_cta + ((warp < kPBelow ? (uint32_t)(kPLow + warp * kPArea)
+                                              : kTpairWin + kTpairBytes + (uint32_t)(warp - kPBelow) * kPArea) -
+                              win0);
+  const uint32_t pix = smem_u32(area + kWPix);
+  uint8_t* const stage = area + kWStage;
+  uint64_t* const bar = reinterpret_cast<uint64_t*>(area + kWBar);
+  PlanSlot* const slots = reinterpret_cast<PlanSlot*>(area + kPSlot);
+  uint32_t* const wins = reinterpret_cast<uint32_t*>(area + kPWins);
+  uint32_t* const next = reinterpret_cast<uint32_t*>(smem_cta + (kPTail - win0));
+  uint4* const ctab = reinterpret_cast<uint4*>(next + 4);
+  const int act = a.groups;
+  PlanClaim claim(a, act);
+  // subtile t of slot s starts loading; bulk: by bulk copies (they complete on the mbarrier)
+  auto load = [&](const PlanSlot* s, uint32_t t, bool& bulk) {
+    const uint32_t cb = 32u * t + lane, b = cb / 3, bxc = s->bx_count;
+    CbPos p;
+    p.c = cb - 3 * b;
+    p.by = b / bxc;
+    p.bx = b - p.by * bxc;
+    const uint64_t pitch = 3ull * s->width;
+    const uint32_t n = min(32u, s->ncb - 32u * t);
+    bulk = bxc >= 12 && (reinterpret_cast<uintptr_t>(s->px) & 15) == 0;
+    return bulk ? load_subtile<true>(s->px, pitch, bxc, p, n, lane, pix, bar)
+                : load_subtile<false>(s->px, pitch, bxc, p, n, lane, pix, bar);
+  };
+
+  if (lane == 0) {
+    mbar_init(bar);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    slots[0].image = slots[1].image = ~0u;
+  }
+  if (threadIdx.x == 0) *next = 0;
+  if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
+    const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
+    const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
+    ctab[lane] = make_uint4(f >> 1 == 0 ? one : 0u, f >> 1 == 1 ? one : 0u, f >> 1 == 2 ? one : 0u, f >> 1 == 3 ? one : 0u);
+  }
+  fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
+  __syncthreads();
+  if (warp >= act) return;
+
+  int esc = 0, nties = 0;
+  bool fail = false, lost = false, bulk = false;
+  uint32_t phase = 0, t, end, tn, endn;
+  PlanSlot *s = slots, *sn = slots + 1;
+  PixAt at{};
+  claim(a, act, next, s, s, c_acc.n, warp, lane, t, end);
+  if (t < end) at = load(s, t, bulk);
+  while (t < end && !lost) {
+    claim(a, act, next, sn, s, c_acc.n, warp, lane, tn, endn);
+    const int k = K >= 0 ? K : s->k, npub = 63 - k;
+    const int G = s->acc;
+    uint8_t* const privst = stage + kWCb * 2 * npub;
+    const uint64_t pitch = 3ull * s->width;
+    int acc = 0;
+    for (; t < end; ++t) {
+      const uint32_t n = min(32u, s->ncb - 32u * t);
+      if (bulk) {
+        if (!__all_sync(0xffffffffu, mbar_wait(bar, phase))) {   // gave up: nothing more is written
+          lost = true;
+          break;
+        }
+        phase ^= 1u;
+      } else {
+        cp_async_wait_all();
+      }
+      __syncwarp();
+      const uint32_t c = at.c;
+      float2 P[8][4];
+      const float V = transform_rows(area + kWPix + at.even, area + kWPix + at.odd, c, P);
+      __syncwarp();                        // the pixel buffer is read: the next subtile's load starts
+      if (t + 1 < end)
+        at = load(s, t + 1, bulk);
+      else if (tn < endn)
+        at = load(sn, tn, bulk);
+      bulk_wait_read_all();                // the staging area may be written again
+      __syncwarp();
+      int16_t* const pub_cb = reinterpret_cast<int16_t*>(stage) + lane * npub;
+      int16_t* const priv_cb = reinterpret_cast<int16_t*>(privst) + (acc * kWCb + lane) * (k + 1);
+      uint32_t mlo, mhi;
+      stage_columns(P, V, k, (uint32_t)lane < n, pub_cb, priv_cb, mlo, mhi);
+      decide_ties(s->px, pitch, s->bx_count, 32u * t, c, k, mlo, mhi, pub_cb, priv_cb, ctab, lane, nties, esc, fail);
+      fence_proxy_async();                 // staged coefficients, before the bulk store
+      __syncwarp();
+      if (lane == 0) store_run(s->pub + (uint64_t)t * (64u * npub), stage, (int)n * 2 * npub);
+      ++acc;
+      if (acc == G || t + 1 == end) {
+        const uint32_t ta = t + 1 - acc;
+        const int bytes = ((acc - 1) * 32 + (int)n) * 2 * (k + 1);
+        ctr_plan(privst, (bytes + 15) >> 4, (uint64_t)ta * (uint32_t)(4 * (k + 1)), s, wins, lane);
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) store_run(s->priv + (uint64_t)ta * (64u * (k + 1)), privst, bytes);
+        acc = 0;
+      }
+    }
+    PlanSlot* const x = s;
+    s = sn;
+    sn = x;
+    t = tn;
+    end = endn;
+  }
+  if (lost) mbar_wait(bar, phase);         // a copy still in flight
+  bulk_wait_all();
+  if (lane == 0 && a.counters) {
+    if (nties) atomicAdd(&a.counters[0], (unsigned long long)nties);
+    if (esc) atomicAdd(&a.counters[1], (unsigned long long)esc);
+    if (fail || lost) atomicAdd(&a.counters[2], 1ull);
+  }
+}
+
 template <int K, bool BULK>
 static cudaError_t launch_w(const TileArgs& a, cudaStream_t s, int sms) {
   static bool attr[kMaxAttrDevices];
@@ -473,6 +644,35 @@ static cudaError_t launch_w(const TileArgs& a, cudaStream_t s, int sms) {
   b.aes_pair = acc_tiles(a.k);
   if (grid > 0) protect_warp_kernel<K, BULK><<<grid, kWarps * 32, kWEnd, s>>>(b);
   return cudaGetLastError();
+}
+
+// per_sm: a quarter of the CTA's warps each (1 .. 3; else all)
+template <int K>
+static cudaError_t launch_plan(const TileArgs& a, cudaStream_t s, int sms, int per_sm) {
+  static bool attr[kMaxAttrDevices];
+  static bool window_ok[kMaxAttrDevices];
+  int dev = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxAttrDevices) return cudaErrorInvalidDevice;
+  if (!window_ok[dev]) {
+    if ((e = smem_window_start_ok(protect_plan_kernel<K>, (uint32_t)kPLow)) != cudaSuccess) return e;
+    window_ok[dev] = true;
+  }
+  e = smem_attr_once(protect_plan_kernel<K>, kPEnd, attr);
+  if (e != cudaSuccess) return e;
+  TileArgs b = a;
+  b.groups = per_sm >= 1 && per_sm < 4 ? per_sm * kWarps / 4 : kWarps;
+  const int grid = a.total_tiles < sms ? a.total_tiles : sms;
+  if (grid > 0) protect_plan_kernel<K><<<grid, kWarps * 32, kPEnd, s>>>(b);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_protect_plan(const TileArgs& a, cudaStream_t s, int sms, int per_sm) {
+  if (!a.images || a.pack || a.plain_private) return cudaErrorInvalidValue;
+  if (a.k == 0) return launch_plan<0>(a, s, sms, per_sm);
+  if (a.k == 5) return launch_plan<5>(a, s, sms, per_sm);
+  return launch_plan<-1>(a, s, sms, per_sm);
 }
 
 cudaError_t launch_protect_warp(const TileArgs& a, cudaStream_t s, int sms) {

@@ -645,11 +645,7 @@ cudaError_t launch_restore(const TileArgs& a, cudaStream_t s, int sms, int per_s
                                       : launch_k<-1, false, 11>(a, s, sms, per_sm);
     return a.k == 5 ? launch_k<5, false, 8>(a, s, sms, per_sm) : launch_k<-1, false, 8>(a, s, sms, per_sm);
   }
-  if (a.images) {
-    if (a.k == 0) return launch_k<0, true>(a, s, sms, per_sm);
-    if (a.k == 5) return launch_k<5, true>(a, s, sms, per_sm);
-    return launch_k<-1, true>(a, s, sms, per_sm);
-  }
+  if (a.images) return launch_restore_plan(a, s, sms, per_sm);
   return launch_restore_warp(a, s, sms);
 }
 

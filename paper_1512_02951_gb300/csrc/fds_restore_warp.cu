@@ -133,6 +133,122 @@ __device__ __forceinline__ int round_warp_inv(const int16_t* pub, const int16_t*
   return r;
 }
 
+// The coefficients of a lane's channel-block (z = 0 .. k at priv_cb, the rest at pub_cb) to
+// floats, two columns at a time through the column butterflies; returns sum |F|
+template <bool PUBIMG>
+__device__ __forceinline__ float gather_columns(const int16_t* pub_cb, const int16_t* priv_cb, int k, float2 (&G2)[8][4]) {
+  float l1 = 0.0f;  // sum |F|, exact (integers below 2^24)
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {        // two columns: gathered and transformed
+    float2 col[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int z0 = zigzag_of(u, 2 * j), z1 = zigzag_of(u, 2 * j + 1);
+      const int q0 = z0 <= k ? (PUBIMG ? (z0 == 0 ? 1024 : 0) : priv_cb[z0]) : pub_cb[z0 - k - 1];
+      const int q1 = z1 <= k ? (PUBIMG ? 0 : priv_cb[z1]) : pub_cb[z1 - k - 1];
+      col[u] = add2(make_float2(__int_as_float(kMagicBits + q0), __int_as_float(kMagicBits + q1)),
+                    make_float2(-kMagic, -kMagic));
+      l1 += fabsf(col[u].x);
+      l1 += fabsf(col[u].y);
+    }
+    idct8_2(col);
+#pragma unroll
+    for (int y = 0; y < 8; ++y) G2[y][j] = col[y];
+    if (j < 3) asm volatile("" ::: "memory");   // the next columns' loads stay behind
+  }
+  return l1;
+}
+
+// Row butterflies, rounding and clamping; bytes into the pixel buffer at out; bit 8 y + x of
+// mhi:mlo marks a value within the error guard of a half-integer (none where the lane is not live)
+__device__ __forceinline__ void emit_rows(const float2 (&G2)[8][4], float l1, bool live, uint8_t* out, uint32_t& mlo,
+                                          uint32_t& mhi) {
+  const float thr = live ? 0.5f - l1 * kGuardInvScale : 1.0f;
+  mlo = mhi = 0;
+#pragma unroll
+  for (int y = 0; y < 8; ++y) {
+    float row[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      row[2 * j] = G2[y][j].x;
+      row[2 * j + 1] = G2[y][j].y;
+    }
+    idct8(row);
+    float2 r[4];
+    float big = 0.0f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 pc = make_float2(fminf(fmaxf(row[2 * j], 0.0f), 255.0f), fminf(fmaxf(row[2 * j + 1], 0.0f), 255.0f));
+      const float2 yv = add2(pc, make_float2(kMagic, kMagic));
+      r[j] = sub2(pc, add2(yv, make_float2(-kMagic, -kMagic)));
+      big = fmaxf(fmaxf(big, fabsf(r[j].x)), fabsf(r[j].y));
+      out[y * kRPitch + 6 * j] = (uint8_t)__float_as_uint(yv.x);
+      out[y * kRPitch + 6 * j + 3] = (uint8_t)__float_as_uint(yv.y);
+    }
+    if (__any_sync(0xffffffffu, big > thr)) {   // rare: a near tie in this row
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int l = 0; l < 2; ++l)
+          if (fabsf(l ? r[j].y : r[j].x) > thr) {
+            if (8 * y + 2 * j + l < 32)
+              mlo |= 1u << (8 * y + 2 * j + l);
+            else
+              mhi |= 1u << (8 * y + 2 * j + l - 32);
+          }
+    }
+  }
+}
+
+// The marked values of a subtile, one after another, each decided by the whole warp and written
+// by its lane (priv_cb, out: the lane's own; pub_g: the subtile's public coefficients in global
+// memory)
+template <bool PUBIMG>
+__device__ __forceinline__ void decide_pixels(uint32_t mlo, uint32_t mhi, const int16_t* pub_g, const int16_t* priv_cb, int k,
+                                              const uint4* ctab, const uint8_t* uv, int lane, WarpSlot* slot, uint8_t* out) {
+  // near ties, one after another, decided by the whole warp
+  for (uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0); who; who &= who - 1) {
+    const int src = __ffs(who) - 1;
+    uint64_t mask = (uint64_t)__shfl_sync(0xffffffffu, mhi, src) << 32 | __shfl_sync(0xffffffffu, mlo, src);
+    const int16_t* pub_s = pub_g + (uint64_t)src * (63 - k);
+    const int16_t* priv_s = priv_cb + (src - lane) * (k + 1);
+    if (lane == 0) slot->ties += __popcll(mask);
+    for (; mask; mask &= mask - 1) {
+      const int pos = __ffsll((long long)mask) - 1;
+      const int p = round_warp_inv<PUBIMG>(pub_s, priv_s, k, pos, ctab, uv, lane, slot);
+      if (lane == src) out[(pos >> 3) * kRPitch + 3 * (pos & 7)] = (uint8_t)(p < 0 ? 0 : (p > 255 ? 255 : p));
+    }
+  }
+}
+
+// The pixel buffer of a subtile of n channel-blocks to the image; at: the lane's place in it
+__device__ __forceinline__ void store_pixels(uint8_t* img, uint64_t pitch, const CbPos& at, uint32_t c0, int n, int lane,
+                                             const uint8_t* pix) {
+  // whole blocks: lane's 8-byte piece c of its block in 8 rows; a block shared with the next
+  // or previous subtile: its channels' bytes
+  uint8_t* const blk = img + ((uint64_t)at.by * (8 * pitch) + 24ull * at.bx);
+  const int b0l = lane - (int)at.c;
+  const bool whole = b0l >= 0 && b0l + 2 < n;
+  if (whole) {
+    uint8_t* dst = blk + 8 * at.c;
+    const uint8_t* src = pix + 8 * (c0 + lane);
+#pragma unroll
+    for (int y = 0; y < 8; ++y) {
+      *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(src + y * kRPitch);
+      dst += pitch;
+    }
+  }
+  for (uint32_t who = __ballot_sync(0xffffffffu, !whole && lane < n); who; who &= who - 1) {
+    const int src = __ffs(who) - 1;
+    const uint32_t sc = __shfl_sync(0xffffffffu, at.c, src);
+    uint8_t* const sb = reinterpret_cast<uint8_t*>(__shfl_sync(0xffffffffu, (unsigned long long)blk, src));
+    const uint8_t* sp = pix + 8 * (c0 + src - sc) + sc;
+    const int x3 = 3 * (lane & 7), y0 = lane >> 3;
+    sb[y0 * pitch + x3 + sc] = sp[y0 * kRPitch + x3];
+    sb[(y0 + 4) * pitch + x3 + sc] = sp[(y0 + 4) * kRPitch + x3];
+  }
+}
+
 template <int K, bool PUBIMG>
 __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __grid_constant__ TileArgs a) {
   extern __shared__ __align__(128) uint8_t smem_cta[];
@@ -202,13 +318,27 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
               ((cnt - 1) * 32 + nof(t + cnt - 1)) * 2 * (k + 1), lane, bars + 1 + half);
   };
 
-  if (threadIdx.x == 0) *next = sfree;
   if (lane == 0) {
     mbar_init(bars);
     mbar_init(bars + 1);
     mbar_init(bars + 2);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // the warp's first run (without the shared counter) starts loading before the tables are filled
+  int cnt = 0, cnt_n = 0, half = 0;
+  uint32_t run = s1, run_n = s1;
+  __syncwarp();
+  if (warp < act) {
+    if (own)
+      run = claim(cnt);
+    else
+      run = s0 + warp, cnt = 1;
+    if (run < s1) {
+      load_pub(run);
+      if (!PUBIMG) load_priv(run, cnt, 0);
+    }
+  }
+  if (threadIdx.x == 0) *next = own ? sfree : s0 + act;
   if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
     const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
     const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
@@ -231,16 +361,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
   }
   bool lost = false;
   uint32_t ph = 0;                         // phases: bit 0 public, bits 1 and 2 the private buffers
-  int cnt = 0, cnt_n = 0, half = 0;
-  uint32_t run = s1, run_n = s1;
-  if (warp < act) {
-    run = claim(cnt);
-    if (run < s1) {
-      load_pub(run);
-      if (!PUBIMG) load_priv(run, cnt, 0);
-    }
-  }
-
   while (run < s1) {
     run_n = claim(cnt_n);
     if (!PUBIMG) {
@@ -299,25 +419,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
       const int16_t* pub_cb = reinterpret_cast<const int16_t*>(pubst) + lane * npub;
       const int16_t* priv_cb = reinterpret_cast<const int16_t*>(privst + half * priv_half) + (ti * kWCb + lane) * (k + 1);
       float2 G2[8][4];
-      float l1 = 0.0f;  // sum |F|, exact (integers below 2^24)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {        // two columns: gathered and transformed
-        float2 col[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int z0 = zigzag_of(u, 2 * j), z1 = zigzag_of(u, 2 * j + 1);
-          const int q0 = z0 <= k ? (PUBIMG ? (z0 == 0 ? 1024 : 0) : priv_cb[z0]) : pub_cb[z0 - k - 1];
-          const int q1 = z1 <= k ? (PUBIMG ? 0 : priv_cb[z1]) : pub_cb[z1 - k - 1];
-          col[u] = add2(make_float2(__int_as_float(kMagicBits + q0), __int_as_float(kMagicBits + q1)),
-                        make_float2(-kMagic, -kMagic));
-          l1 += fabsf(col[u].x);
-          l1 += fabsf(col[u].y);
-        }
-        idct8_2(col);
-#pragma unroll
-        for (int y = 0; y < 8; ++y) G2[y][j] = col[y];
-        if (j < 3) asm volatile("" ::: "memory");   // the next columns' loads stay behind
-      }
+      const float l1 = gather_columns<PUBIMG>(pub_cb, priv_cb, k, G2);
       __syncwarp();                        // the public part is read: the next one starts loading
       {
         const uint32_t tn = ti + 1 < cnt ? t + 1 : run_n;
@@ -325,81 +427,13 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
       }
       const uint32_t c0 = __shfl_sync(0xffffffffu, at.c, 0);
       uint8_t* const out = pix + 8 * (c0 + lane - at.c) + at.c;
-      const float thr = lane < n ? 0.5f - l1 * kGuardInvScale : 1.0f;
-      uint32_t mlo = 0, mhi = 0;
-#pragma unroll
-      for (int y = 0; y < 8; ++y) {
-        float row[8];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          row[2 * j] = G2[y][j].x;
-          row[2 * j + 1] = G2[y][j].y;
-        }
-        idct8(row);
-        float2 r[4];
-        float big = 0.0f;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float2 pc = make_float2(fminf(fmaxf(row[2 * j], 0.0f), 255.0f), fminf(fmaxf(row[2 * j + 1], 0.0f), 255.0f));
-          const float2 yv = add2(pc, make_float2(kMagic, kMagic));
-          r[j] = sub2(pc, add2(yv, make_float2(-kMagic, -kMagic)));
-          big = fmaxf(fmaxf(big, fabsf(r[j].x)), fabsf(r[j].y));
-          out[y * kRPitch + 6 * j] = (uint8_t)__float_as_uint(yv.x);
-          out[y * kRPitch + 6 * j + 3] = (uint8_t)__float_as_uint(yv.y);
-        }
-        if (__any_sync(0xffffffffu, big > thr)) {   // rare: a near tie in this row
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int l = 0; l < 2; ++l)
-              if (fabsf(l ? r[j].y : r[j].x) > thr) {
-                if (8 * y + 2 * j + l < 32)
-                  mlo |= 1u << (8 * y + 2 * j + l);
-                else
-                  mhi |= 1u << (8 * y + 2 * j + l - 32);
-              }
-        }
-      }
-      // near ties, one after another, decided by the whole warp
-      for (uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0); who; who &= who - 1) {
-        const int src = __ffs(who) - 1;
-        uint64_t mask = (uint64_t)__shfl_sync(0xffffffffu, mhi, src) << 32 | __shfl_sync(0xffffffffu, mlo, src);
-        const int16_t* pub_s = a.pub_in + (uint64_t)(32u * t + src) * npub;
-        const int16_t* priv_s = priv_cb + (src - lane) * (k + 1);
-        if (lane == 0) slot->ties += __popcll(mask);
-        for (; mask; mask &= mask - 1) {
-          const int pos = __ffsll((long long)mask) - 1;
-          const int p = round_warp_inv<PUBIMG>(pub_s, priv_s, k, pos, ctab, uv, lane, slot);
-          if (lane == src) out[(pos >> 3) * kRPitch + 3 * (pos & 7)] = (uint8_t)(p < 0 ? 0 : (p > 255 ? 255 : p));
-        }
-      }
+      uint32_t mlo, mhi;
+      emit_rows(G2, l1, lane < n, out, mlo, mhi);
+      decide_pixels<PUBIMG>(mlo, mhi, a.pub_in + (uint64_t)(32u * t) * npub, priv_cb, k, ctab, uv, lane, slot, out);
       if (!PUBIMG && !twice) fence_proxy_async();
       __syncwarp();                        // the pixel rows are complete
       if (!PUBIMG && !twice && ti + 1 == cnt && run_n < s1) load_priv(run_n, cnt_n, 0);
-      // whole blocks: lane's 8-byte piece c of its block in 8 rows; a block shared with the next
-      // or previous subtile: its channels' bytes
-      const uint64_t pitch = 3ull * (uint64_t)a.width;
-      uint8_t* const blk = a.pixels_out + ((uint64_t)at.by * (8 * pitch) + 24ull * at.bx);
-      const int b0l = lane - (int)at.c;
-      const bool whole = b0l >= 0 && b0l + 2 < n;
-      if (whole) {
-        uint8_t* dst = blk + 8 * at.c;
-        const uint8_t* src = pix + 8 * (c0 + lane);
-#pragma unroll
-        for (int y = 0; y < 8; ++y) {
-          *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(src + y * kRPitch);
-          dst += pitch;
-        }
-      }
-      for (uint32_t who = __ballot_sync(0xffffffffu, !whole && lane < n); who; who &= who - 1) {
-        const int src = __ffs(who) - 1;
-        const uint32_t sc = __shfl_sync(0xffffffffu, at.c, src);
-        uint8_t* const sb = reinterpret_cast<uint8_t*>(__shfl_sync(0xffffffffu, (unsigned long long)blk, src));
-        const uint8_t* sp = pix + 8 * (c0 + src - sc) + sc;
-        const int x3 = 3 * (lane & 7), y0 = lane >> 3;
-        sb[y0 * pitch + x3 + sc] = sp[y0 * kRPitch + x3];
-        sb[(y0 + 4) * pitch + x3 + sc] = sp[(y0 + 4) * kRPitch + x3];
-      }
+      store_pixels(a.pixels_out, 3ull * (uint64_t)a.width, at, c0, n, lane, pix);
       __syncwarp();                        // the pixel buffer may be written again
     }
     if (lost) break;
@@ -410,6 +444,186 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
   if (lost) {                              // copies still in flight
     mbar_wait(bars, ph & 1u);
     if (!PUBIMG && twice && run_n < s1) mbar_wait(bars + 1 + (half ^ 1), (ph >> (1 + (half ^ 1))) & 1u);
+  }
+  if (lane == 0 && a.counters) {
+    if (slot->ties) atomicAdd(&a.counters[0], (unsigned long long)slot->ties);
+    if (slot->esc) atomicAdd(&a.counters[1], (unsigned long long)slot->esc);
+    if (slot->fail || lost) atomicAdd(&a.counters[2], 1ull);
+  }
+}
+
+// ---- batches ---------------------------------------------------------------------------------
+
+constexpr int kQSlot = (kRSlot + 32 + 7) & ~7;    // two PlanSlots after the single-image area
+constexpr int kQWins = kQSlot + 2 * (int)sizeof(PlanSlot);   // the warp's two windows
+constexpr int kQArea = (kQWins + 40 + 31) & ~31;
+constexpr int kQBelow = ((int)kTpairWin - 1024) / kQArea;
+constexpr int kQLow = (int)kTpairWin - kQBelow * kQArea;
+constexpr int kQAbove = kWarps > kQBelow ? kWarps - kQBelow : 0;
+constexpr int kQTail = (int)kTpairWin + kTpairBytes + kQAbove * kQArea;   // counter, folded c(m), (u, v) by zigzag
+constexpr int kQEnd = kQTail + 16 + 512 + 64;
+static_assert(kQEnd <= 227 * 1024, "restore (batches) shared memory");
+
+// by k: run_tiles (at most a tile), and 16 where two runs fit
+struct RunTable {
+  uint8_t n[64];
+};
+constexpr RunTable make_run_table() {
+  RunTable t{};
+  for (int k = 0; k < 64; ++k)
+    t.n[k] = (uint8_t)((run_tiles(k) < kTileSubs ? run_tiles(k) : kTileSubs) | (run_twice(k) ? 16 : 0));
+  return t;
+}
+static __constant__ RunTable c_run = make_run_table();
+
+// Restore of a batch (the tiles as in protect_plan_kernel).  Where the next run is of an image
+// with another k, its parts lie elsewhere in the buffers and are loaded only when the run before
+// is done.
+template <int K>
+__global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __grid_constant__ TileArgs a) {
+  extern __shared__ __align__(128) uint8_t smem_cta[];
+  const uint32_t win0 = smem_u32(smem_cta);
+  if (win0 > (uint32_t)kQLow) {   // see the launcher
+    if (threadIdx.x == 0 && a.counters) atomicAdd(&a.counters[2], 1ull);
+    return;
+  }
+  const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+  uint8_t* area = smem_cta + ((warp < kQBelow ? (uint32_t)(kQLow + warp * kQArea)
+                                              : kTpairWin + kTpairBytes + (uint32_t)(warp - kQBelow) * kQArea) -
+                              win0);
+  uint8_t* const pix = area + kRPix;
+  uint8_t* const frag = area + kRFrag;
+  uint64_t* const bars = reinterpret_cast<uint64_t*>(area + kRBar);
+  WarpSlot* const slot = reinterpret_cast<WarpSlot*>(area + kRSlot);
+  PlanSlot* const slots = reinterpret_cast<PlanSlot*>(area + kQSlot);
+  uint32_t* const wins = reinterpret_cast<uint32_t*>(area + kQWins);
+  uint32_t* const next = reinterpret_cast<uint32_t*>(smem_cta + (kQTail - win0));
+  uint4* const ctab = reinterpret_cast<uint4*>(next + 4);
+  uint8_t* const uv = reinterpret_cast<uint8_t*>(ctab + 32);
+  const int act = a.groups;
+  PlanClaim claim(a, act);
+  auto nof = [&](const PlanSlot* s, uint32_t t) { return (int)min(32u, s->ncb - 32u * t); };
+  auto load_pub = [&](const PlanSlot* s, uint32_t t) {
+    const int npub = 63 - (K >= 0 ? K : s->k);
+    load_part(frag, s->pub + (uint64_t)t * (64u * npub), nof(s, t) * 2 * npub, lane, bars);
+  };
+  auto load_priv = [&](const PlanSlot* s, uint32_t t, int cnt, int half) {
+    const int k = K >= 0 ? K : s->k;
+    load_part(frag + kWCb * 2 * (63 - k) + half * (s->acc & 15) * 64 * (k + 1), s->priv + (uint64_t)t * (64u * (k + 1)),
+              ((cnt - 1) * 32 + nof(s, t + cnt - 1)) * 2 * (k + 1), lane, bars + 1 + half);
+  };
+
+  if (lane == 0) {
+    mbar_init(bars);
+    mbar_init(bars + 1);
+    mbar_init(bars + 2);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    slots[0].image = slots[1].image = ~0u;
+    slot->ties = slot->esc = slot->fail = 0;
+  }
+  if (threadIdx.x == 0) *next = 0;
+  if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
+    const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
+    const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
+    ctab[lane] = make_uint4(f >> 1 == 0 ? one : 0u, f >> 1 == 1 ? one : 0u, f >> 1 == 2 ? one : 0u, f >> 1 == 3 ? one : 0u);
+  }
+  if (threadIdx.x < 64) uv[zigzag_of((int)threadIdx.x >> 3, (int)threadIdx.x & 7)] = (uint8_t)threadIdx.x;
+  fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
+  __syncthreads();
+  if (warp >= act) return;
+
+  bool lost = false;
+  uint32_t ph = 0;                         // phases: bit 0 public, bits 1 and 2 the private buffers
+  PlanSlot *s = slots, *sx = slots + 1;    // the run's image; the other slot
+  uint32_t r, end;                         // the run's first subtile, the end of what was claimed
+  int half = 0;
+  claim(a, act, next, s, s, c_run.n, warp, lane, r, end);
+  if (r < end) {
+    load_priv(s, r, min(s->acc & 15, (int)(end - r)), 0);
+    load_pub(s, r);
+  }
+  while (r < end && !lost) {
+    const int k = K >= 0 ? K : s->k, npub = 63 - k;
+    const int G = s->acc & 15, cnt = min(G, (int)(end - r));
+    const bool twice = s->acc & 16;
+    // the next run: of the same claim, or of a new one
+    PlanSlot* n = s;
+    uint32_t rn = r + cnt, endn = end;
+    if (rn >= end) {
+      n = sx;
+      claim(a, act, next, n, s, c_run.n, warp, lane, rn, endn);
+    }
+    const bool have = rn < endn, pipe = have && (K >= 0 || n->k == k);
+    const int cntn = have ? min(n->acc & 15, (int)(endn - rn)) : 0;
+    uint8_t* const privst = frag + kWCb * 2 * npub + half * G * 64 * (k + 1);
+    if (twice && pipe) {
+      fence_proxy_async();                 // the buffer was decrypted in place
+      __syncwarp();
+      load_priv(n, rn, cntn, half ^ 1);
+    }
+    if (!__all_sync(0xffffffffu, mbar_wait(bars + 1 + half, (ph >> (1 + half)) & 1u))) {
+      lost = true;
+      break;
+    }
+    ph ^= 2u << half;
+    __syncwarp();
+    ctr_plan(privst, (((cnt - 1) * 32 + nof(s, r + cnt - 1)) * 2 * (k + 1) + 15) >> 4, (uint64_t)r * (uint32_t)(4 * (k + 1)),
+             s, wins, lane);
+    __syncwarp();
+#pragma unroll 1
+    for (int ti = 0; ti < cnt; ++ti) {
+      const uint32_t t = r + ti;
+      const int m = nof(s, t);
+      CbPos at;
+      {
+        const uint32_t cb = 32u * t + lane, b = cb / 3, bxc = s->bx_count;
+        at.c = cb - 3 * b;
+        at.by = b / bxc;
+        at.bx = b - at.by * bxc;
+      }
+      if (!__all_sync(0xffffffffu, mbar_wait(bars, ph & 1u))) {   // gave up: nothing more is written
+        lost = true;
+        break;
+      }
+      ph ^= 1u;
+      __syncwarp();
+      const int16_t* pub_cb = reinterpret_cast<const int16_t*>(frag) + lane * npub;
+      const int16_t* priv_cb = reinterpret_cast<const int16_t*>(privst) + (ti * kWCb + lane) * (k + 1);
+      float2 G2[8][4];
+      const float l1 = gather_columns<false>(pub_cb, priv_cb, k, G2);
+      __syncwarp();                        // the public part is read: the next one starts loading
+      if (ti + 1 < cnt)
+        load_pub(s, t + 1);
+      else if (pipe)
+        load_pub(n, rn);
+      const uint32_t c0 = __shfl_sync(0xffffffffu, at.c, 0);
+      uint8_t* const out = pix + 8 * (c0 + lane - at.c) + at.c;
+      uint32_t mlo, mhi;
+      emit_rows(G2, l1, lane < m, out, mlo, mhi);
+      decide_pixels<false>(mlo, mhi, reinterpret_cast<const int16_t*>(s->pub) + (uint64_t)(32u * t) * npub, priv_cb, k, ctab, uv,
+                           lane, slot, out);
+      if (ti + 1 == cnt && have && !(twice && pipe)) fence_proxy_async();
+      __syncwarp();                        // the pixel rows are complete
+      if (ti + 1 == cnt && have && !(twice && pipe)) {
+        if (!pipe) load_pub(n, rn);
+        load_priv(n, rn, cntn, 0);
+      }
+      store_pixels(s->px, 3ull * s->width, at, c0, m, lane, pix);
+      __syncwarp();                        // the pixel buffer may be written again
+    }
+    if (lost) break;
+    half = twice && pipe ? half ^ 1 : 0;
+    if (n != s) {
+      sx = s;
+      s = n;
+    }
+    r = rn;
+    end = endn;
+  }
+  if (lost) {                              // copies still in flight
+    mbar_wait(bars, ph & 1u);
+    mbar_wait(bars + 1, (ph >> 1) & 1u);
+    mbar_wait(bars + 2, (ph >> 2) & 1u);
   }
   if (lane == 0 && a.counters) {
     if (slot->ties) atomicAdd(&a.counters[0], (unsigned long long)slot->ties);
@@ -441,6 +655,35 @@ static cudaError_t launch_w(const TileArgs& a, cudaStream_t s, int sms) {
   b.aes_pair = run_tiles(a.k) | (run_twice(a.k) ? 16 : 0);
   if (grid > 0) restore_warp_kernel<K, PUBIMG><<<grid, kWarps * 32, kREnd, s>>>(b);
   return cudaGetLastError();
+}
+
+// per_sm: half of the CTA's warps (1; else all)
+template <int K>
+static cudaError_t launch_plan(const TileArgs& a, cudaStream_t s, int sms, int per_sm) {
+  static bool attr[kMaxAttrDevices];
+  static bool window_ok[kMaxAttrDevices];
+  int dev = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxAttrDevices) return cudaErrorInvalidDevice;
+  if (!window_ok[dev]) {
+    if ((e = smem_window_start_ok(restore_plan_kernel<K>, (uint32_t)kQLow)) != cudaSuccess) return e;
+    window_ok[dev] = true;
+  }
+  e = smem_attr_once(restore_plan_kernel<K>, kQEnd, attr);
+  if (e != cudaSuccess) return e;
+  TileArgs b = a;
+  b.groups = per_sm == 1 ? kWarps / 2 : kWarps;
+  const int grid = a.total_tiles < sms ? a.total_tiles : sms;
+  if (grid > 0) restore_plan_kernel<K><<<grid, kWarps * 32, kQEnd, s>>>(b);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_restore_plan(const TileArgs& a, cudaStream_t s, int sms, int per_sm) {
+  if (!a.images || a.pack || a.plain_private || a.public_image) return cudaErrorInvalidValue;
+  if (a.k == 0) return launch_plan<0>(a, s, sms, per_sm);
+  if (a.k == 5) return launch_plan<5>(a, s, sms, per_sm);
+  return launch_plan<-1>(a, s, sms, per_sm);
 }
 
 cudaError_t launch_restore_warp(const TileArgs& a, cudaStream_t s, int sms) {

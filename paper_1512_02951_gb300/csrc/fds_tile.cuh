@@ -137,8 +137,11 @@ cudaError_t launch_protect(const TileArgs& a, cudaStream_t s, bool debug, int sm
 cudaError_t launch_restore(const TileArgs& a, cudaStream_t s, int sms, int per_sm = 0);
 // protect of one image in int16 storage, one subtile of 32 channel-blocks per warp
 cudaError_t launch_protect_warp(const TileArgs& a, cudaStream_t s, int sms);
+// protect of a batch, likewise; k as in launch_protect
+cudaError_t launch_protect_plan(const TileArgs& a, cudaStream_t s, int sms, int per_sm);
 // restore (or the public-image form) of one image in int16 storage, likewise
 cudaError_t launch_restore_warp(const TileArgs& a, cudaStream_t s, int sms);
+cudaError_t launch_restore_plan(const TileArgs& a, cudaStream_t s, int sms, int per_sm);
 // restore with the inverse transform on tensor cores (one image, int16 storage)
 cudaError_t launch_restore_tc(const TileArgs& a, cudaStream_t s, int sms);
 // tensor-core protect of one image (form 0: BF16 three limbs, 1: TF32 two limbs); tiles of

@@ -96,4 +96,155 @@ __device__ __forceinline__ void put_window(const TileArgs& a, uint64_t q, int sl
   }
 }
 
+// ---- batches: what a warp knows about the image of a tile it works on (shared memory; two per
+// warp, the tile's and the next one's)
+struct PlanSlot {
+  uint8_t* px;                    // the image's pixels, public and private fragments
+  uint8_t* pub;
+  uint8_t* priv;
+  uint64_t iv_hi, iv_lo, wbase;   // wbase: first counter window of the warp's two, ~0 if none
+  uint32_t width, bx_count, ncb, image;
+  int32_t k, acc;                 // acc: subtiles between two AES phases
+  uint32_t rk[44];
+};
+static_assert(sizeof(PlanSlot) % 8 == 0, "PlanSlot");
+constexpr int kTileSubs = kTileCb / kWCb;         // subtiles of a 64-block tile
+
+// The image of tile g into slot s (the whole warp; acc_of: subtiles between two AES phases by k);
+// hint: a slot whose image it often is; returns the tile's index in the image
+__device__ __forceinline__ int plan_slot(const TileArgs& a, int g, PlanSlot* s, const PlanSlot* hint, const uint8_t* acc_of,
+                                         int lane) {
+  uint32_t im = hint->image;
+  if (!(im < (uint32_t)a.n_images && __ldg(a.tile_start + im) <= g && g < __ldg(a.tile_start + im + 1))) {
+    int lo = 0, hi = a.n_images;                 // tile_start[lo] <= g < tile_start[hi]
+    while (hi - lo > 1) {
+      const int step = (hi - lo + 31) >> 5, p = min(lo + step * lane, hi);
+      const uint32_t le = __ballot_sync(0xffffffffu, __ldg(a.tile_start + p) <= g);
+      lo += step * (__popc(le) - 1);
+      hi = min(lo + step, hi);
+    }
+    im = (uint32_t)lo;
+  }
+  const int local = g - __ldg(a.tile_start + im);
+  const bool other = s->image != im;
+  __syncwarp();
+  if (other) {
+    const BatchImage& b = a.images[im];
+    const int slot = b.key_slot;
+    for (int i = lane; i < 44; i += 32) s->rk[i] = __ldg(a.round_keys + 44 * slot + i);
+    if (lane == 0) {
+      s->px = const_cast<uint8_t*>(a.pixels_in ? a.pixels_in : a.pixels_out) + b.pixel_offset;
+      s->pub = reinterpret_cast<uint8_t*>(a.pub_in ? const_cast<int16_t*>(a.pub_in) : a.pub_out) + b.public_offset;
+      s->priv = (a.priv_in ? const_cast<uint8_t*>(a.priv_in) : a.priv_out) + b.private_offset;
+      s->iv_hi = b.iv_hi;
+      s->iv_lo = b.iv_lo;
+      s->wbase = ~0ull - 1;
+      s->width = (uint32_t)b.width;
+      s->bx_count = (uint32_t)b.width >> 3;
+      s->ncb = 3u * ((uint32_t)b.width >> 3) * ((uint32_t)b.height >> 3);
+      s->image = im;
+      s->k = b.k;
+      s->acc = acc_of[b.k];
+    }
+  } else if (lane == 0) {
+    s->wbase = ~0ull - 1;         // the windows may have been the other slot's
+  }
+  __syncwarp();
+  return local;
+}
+
+// The next run of subtiles of one image for a warp: [t, end), none left where t == end.  A CTA's
+// tiles are [g0, g1), taken by its warps one by one from `next`, the last ones (from g0 + whole on)
+// subtile by subtile; or (a.dispenser) every warp takes tiles from one counter.
+struct PlanClaim {
+  int g0, g1, whole;
+  bool first;
+
+  __device__ __forceinline__ PlanClaim(const TileArgs& a, int act) {
+    g0 = (int)((int64_t)a.total_tiles * blockIdx.x / gridDim.x);
+    g1 = (int)((int64_t)a.total_tiles * (blockIdx.x + 1) / gridDim.x);
+    whole = g1 - g0 - min(g1 - g0, (2 * act + kTileSubs - 1) / kTileSubs);
+    first = true;
+  }
+  __device__ __forceinline__ void operator()(const TileArgs& a, int act, uint32_t* next, PlanSlot* s, const PlanSlot* hint,
+                                             const uint8_t* acc_of, int warp, int lane, uint32_t& t, uint32_t& end) {
+    for (;;) {
+      uint32_t u = 0;
+      if (lane == 0) {
+        if (a.dispenser == nullptr)
+          u = atomicAdd(next, 1u);
+        else if (first)
+          u = blockIdx.x * act + warp;
+        else
+          u = atomicAdd(a.dispenser, 1u) + gridDim.x * act;
+      }
+      u = __shfl_sync(0xffffffffu, u, 0);
+      first = false;
+      int g, sub = -1;
+      if (a.dispenser != nullptr) {
+        if (u >= (uint32_t)a.total_tiles) break;
+        g = (int)u;
+      } else {
+        const int v = (int)u - whole;
+        g = g0 + (v < 0 ? (int)u : whole + v / kTileSubs);
+        if (v >= 0) sub = v % kTileSubs;
+        if (g >= g1) break;
+      }
+      const int local = plan_slot(a, g, s, hint, acc_of, lane);
+      t = (uint32_t)local * kTileSubs;
+      end = min(t + kTileSubs, (s->ncb + 31u) >> 5);
+      if (sub < 0) return;
+      t += sub;
+      if (t < end) {
+        end = t + 1;
+        return;
+      }
+    }
+    t = end = 0;
+  }
+};
+
+// AES-128-CTR over nblk keystream blocks at buf, the first being block `first` of the slot's
+// image: through the warp's two counter windows (wins) where it has them or where more than two
+// rounds of blocks pay for their constants
+__device__ __forceinline__ void ctr_plan(uint8_t* buf, int nblk, uint64_t first, PlanSlot* s, uint32_t* wins, int lane) {
+  const PairLanes lc = pair_lanes();
+  const uint64_t b0 = (s->iv_lo & 255u) + first;               // from the IV's window
+  uint64_t wbase = s->wbase;
+  bool use = (b0 >> 8) >= wbase && ((b0 + nblk - 1) >> 8) <= wbase + 1;
+  if (!use && nblk > 64) {
+    wbase = b0 >> 8;
+    uint32_t w[5];
+    aes_window(s->iv_hi, s->iv_lo, wbase + (lane & 1), s->rk, lc, w);
+    __syncwarp();
+    if (lane < 2) {
+#pragma unroll
+      for (int i = 0; i < 5; ++i) wins[5 * lane + i] = w[i];
+    }
+    if (lane == 0) s->wbase = wbase;
+    __syncwarp();
+    use = true;
+  }
+#pragma unroll 1
+  for (int i = lane; i < nblk; i += 32) {
+    uint32_t ks[4];
+    if (use) {
+      const uint64_t b = b0 + i;
+      const uint32_t* src = wins + ((b >> 8) != wbase ? 5 : 0);
+      const uint32_t w[5] = {src[0], src[1], src[2], src[3], src[4]};
+      aes_from_window(w, (uint32_t)b & 255u, s->rk, lc, ks);
+    } else {
+      ctr_block(s->iv_hi, s->iv_lo, first + i, ks);
+      aes128_encrypt_pair(ks, s->rk, lc);
+    }
+    uint4* p = reinterpret_cast<uint4*>(buf + 16 * i);
+    uint4 d = *p;
+    d.x ^= ks[0];
+    d.y ^= ks[1];
+    d.z ^= ks[2];
+    d.w ^= ks[3];
+    *p = d;
+  }
+}
+
 }  // namespace fds
