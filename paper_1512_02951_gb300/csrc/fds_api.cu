@@ -1059,11 +1059,9 @@ int fds_image_stats(const uint8_t* image, int32_t width, int32_t height, uint64_
   int rc = ensure_init(&dev);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = cudaMemsetAsync(histogram_out, 0, 3 * 256 * sizeof(uint64_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(pair_sums_out, 0, 3 * 3 * 6 * sizeof(int64_t), s);
-  if (e != cudaSuccess) return cuda_fail(e, "clearing the statistics");
-  e = launch_image_stats(image, width, height, reinterpret_cast<unsigned long long*>(histogram_out),
-                         reinterpret_cast<long long*>(pair_sums_out), s, g_tables[dev].sms);
+  const cudaError_t e = launch_image_stats(image, width, height, reinterpret_cast<unsigned long long*>(histogram_out),
+                                           reinterpret_cast<long long*>(pair_sums_out), s, g_tables[dev].sms,
+                                           g_tables[dev].counters);
   return e == cudaSuccess ? FDS_OK : cuda_fail(e, "statistics launch");
 }
 

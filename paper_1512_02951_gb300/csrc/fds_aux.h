@@ -29,10 +29,10 @@ inline cudaError_t smem_window_start_ok(Kernel kernel, uint32_t max_start) {
 cudaError_t launch_aes_full(const uint8_t* in, uint8_t* out, uint64_t bytes, uint64_t iv_hi, uint64_t iv_lo,
                             const uint32_t rk[44], const uint32_t* T, cudaStream_t s, int sms,
                             unsigned long long* counters);
-// histogram and adjacent-pair sums of an H x W x 3 image (hist [3][256], sums [3][3][6],
-// both zero on entry)
+// histogram and adjacent-pair sums of an H x W x 3 image (hist [3][256], sums [3][3][6]; both
+// are cleared first); counters as in launch_aes_full
 cudaError_t launch_image_stats(const uint8_t* img, int width, int height, unsigned long long* hist, long long* sums,
-                               cudaStream_t s, int sms);
+                               cudaStream_t s, int sms, unsigned long long* counters);
 // strong level: out = in XOR (per channel-block SHA-512 of its Part 1 plaintext, [ncb][k+1]
 // int16); the constants are uploaded once per device by upload_sha512_constants
 cudaError_t launch_strong_mask(const uint8_t* plain, const uint8_t* in, uint8_t* out, int width, int height, int k,
