@@ -169,6 +169,8 @@ def lib_path() -> str:
 def load(build_if_missing: bool = False) -> ctypes.CDLL:
     """Load libfds.so (the CUDA library).  Raises if it is not built: there is no fallback."""
     global _lib
+    if _lib is not None:          # set once, complete, under the lock
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib

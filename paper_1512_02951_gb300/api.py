@@ -19,7 +19,9 @@ from . import _lib
 
 
 def _stream_ptr(device: torch.device) -> int:
-    return torch.cuda.current_stream(device).cuda_stream
+    # the current stream's handle without a Stream object around it
+    i = device.index
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if i is None else i)
 
 
 def _check_key(b: bytes, what: str) -> bytes:
