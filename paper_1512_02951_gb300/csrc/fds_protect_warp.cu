@@ -155,6 +155,10 @@ __device__ __forceinline__ void ctr_warp(const TileArgs& a, uint8_t* buf, const 
     aes_from_window(w, (uint32_t)b & 255u, a.rk, lc, s);
     uint4* p = reinterpret_cast<uint4*>(buf + 16 * i);
     uint4 d = *p;
+    if (a.plain_out) {
+      const uint64_t at = 16 * ((uint64_t)list[j] * nb + (i - j * nb));
+      if (at < 6ull * (uint32_t)a.nblocks * (nb >> 2)) *reinterpret_cast<uint4*>(a.plain_out + at) = d;
+    }
     d.x ^= s[0];
     d.y ^= s[1];
     d.z ^= s[2];

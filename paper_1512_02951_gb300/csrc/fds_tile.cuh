@@ -107,6 +107,8 @@ struct TileArgs {
   int32_t aes_pair;
   // protect: tile groups that work in each CTA (1 .. the kernel's groups; 0 = all of them)
   int32_t groups;
+  // strong level (protect of one image): Part 1 is also left here in plaintext
+  uint8_t* plain_out;
   // warp form: block row of block b = (b * bx_magic) >> bx_shift
   uint32_t bx_magic;
   int32_t bx_shift;
