@@ -109,14 +109,6 @@ __device__ __forceinline__ float dct8_row_bytes_w(const float (&X)[8], float (&x
   return pass_weight(s, d);
 }
 
-// dct8<true, true> of an exact-integer column that also returns its error weight
-__device__ __forceinline__ float dct8_rat_w(float (&x)[8]) {
-  const float s[4] = {x[0] + x[7], x[1] + x[6], x[2] + x[5], x[3] + x[4]};
-  const float d[4] = {x[0] - x[7], x[1] - x[6], x[2] - x[5], x[3] - x[4]};
-  dct8_sd<true, true>(s, d, x);
-  return pass_weight(s, d);
-}
-
 // ---- the same butterflies on pairs of independent columns (packed f32x2 arithmetic); every
 // lane performs exactly the scalar operations, so the results are bit-identical
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -154,7 +146,7 @@ __device__ __forceinline__ void dct8_2(float2 (&x)[8]) {
   dct8_sd2<RAT_UNSCALED, IRR_LAMBDA>(s, d, x);
 }
 
-// dct8_rat_w on two exact-integer columns at once; returns the sum of both error weights
+// dct8<true, true> on two exact-integer columns at once; returns the sum of their error weights
 __device__ __forceinline__ float dct8_rat_w2(float2 (&x)[8]) {
   const float2 s[4] = {add2(x[0], x[7]), add2(x[1], x[6]), add2(x[2], x[5]), add2(x[3], x[4])};
   const float2 d[4] = {sub2(x[0], x[7]), sub2(x[1], x[6]), sub2(x[2], x[5]), sub2(x[3], x[4])};
@@ -341,48 +333,6 @@ __device__ __forceinline__ void aes128_encrypt_rep(uint32_t (&s)[4], const uint3
           __byte_perm(l2(s1), 0u, 0x4144u) | __byte_perm(l3(s2), 0u, 0x1444u)) ^ rk[43];
 }
 
-// The same on M independent blocks at once, their rounds interleaved: the M lookups chains
-// overlap, so one warp keeps the table pipe busy where a single block per thread would wait
-// out each round's load latency.
-template <int M, int SH = 7>
-__device__ __forceinline__ void aes128_encrypt_rep_n(uint32_t (&s)[M][4], const uint32_t* rk, uint32_t Tl) {
-  auto l0 = [&](uint32_t w) { return trep_at<SH>(Tl, w, 0x4440u); };
-  auto l1 = [&](uint32_t w) { return trep_at<SH>(Tl, w, 0x4441u); };
-  auto l2 = [&](uint32_t w) { return trep_at<SH>(Tl, w, 0x4442u); };
-  auto l3 = [&](uint32_t w) { return trep_at<SH>(Tl, w, 0x4443u); };
-  auto r8 = [](uint32_t x) { return __byte_perm(x, x, 0x2103u); };
-  auto r16 = [](uint32_t x) { return __byte_perm(x, x, 0x1032u); };
-  auto r24 = [](uint32_t x) { return __byte_perm(x, x, 0x0321u); };
-#pragma unroll
-  for (int m = 0; m < M; ++m)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) s[m][c] ^= rk[c];
-#pragma unroll 1
-  for (int r = 1; r < 10; ++r) {
-    const uint32_t k0 = rk[4 * r], k1 = rk[4 * r + 1], k2 = rk[4 * r + 2], k3 = rk[4 * r + 3];
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      const uint32_t s0 = s[m][0], s1 = s[m][1], s2 = s[m][2], s3 = s[m][3];
-      s[m][0] = l0(s0) ^ r8(l1(s1)) ^ r16(l2(s2)) ^ r24(l3(s3)) ^ k0;
-      s[m][1] = l0(s1) ^ r8(l1(s2)) ^ r16(l2(s3)) ^ r24(l3(s0)) ^ k1;
-      s[m][2] = l0(s2) ^ r8(l1(s3)) ^ r16(l2(s0)) ^ r24(l3(s1)) ^ k2;
-      s[m][3] = l0(s3) ^ r8(l1(s0)) ^ r16(l2(s1)) ^ r24(l3(s2)) ^ k3;
-    }
-  }
-#pragma unroll
-  for (int m = 0; m < M; ++m) {
-    const uint32_t s0 = s[m][0], s1 = s[m][1], s2 = s[m][2], s3 = s[m][3];
-    s[m][0] = (__byte_perm(l0(s0), 0u, 0x4441u) | __byte_perm(l1(s1), 0u, 0x4414u) |
-               __byte_perm(l2(s2), 0u, 0x4144u) | __byte_perm(l3(s3), 0u, 0x1444u)) ^ rk[40];
-    s[m][1] = (__byte_perm(l0(s1), 0u, 0x4441u) | __byte_perm(l1(s2), 0u, 0x4414u) |
-               __byte_perm(l2(s3), 0u, 0x4144u) | __byte_perm(l3(s0), 0u, 0x1444u)) ^ rk[41];
-    s[m][2] = (__byte_perm(l0(s2), 0u, 0x4441u) | __byte_perm(l1(s3), 0u, 0x4414u) |
-               __byte_perm(l2(s0), 0u, 0x4144u) | __byte_perm(l3(s1), 0u, 0x1444u)) ^ rk[42];
-    s[m][3] = (__byte_perm(l0(s3), 0u, 0x4441u) | __byte_perm(l1(s0), 0u, 0x4414u) |
-               __byte_perm(l2(s1), 0u, 0x4144u) | __byte_perm(l3(s2), 0u, 0x1444u)) ^ rk[43];
-  }
-}
-
 // AES-128 with the pair table: T0 and T2 = rotl(T0, 16), each replicated per lane, in one
 // 64 KB table that starts at shared-window address kTpairWin (a multiple of 64 KB).  Entry x
 // of table j (0: T0, 1: T2), copy L, is the word at window address kTpairWin + 256 x + 128 j +
@@ -451,45 +401,6 @@ __device__ __forceinline__ void aes128_encrypt_pair(uint32_t (&s)[4], const uint
   s[1] = last(s1, s2, s3, s0) ^ rk[41];
   s[2] = last(s2, s3, s0, s1) ^ rk[42];
   s[3] = last(s3, s0, s1, s2) ^ rk[43];
-}
-
-// aes128_encrypt on M independent blocks, their rounds interleaved (the same four shared
-// T-tables): a thread with M blocks overlaps their table-lookup latencies.
-template <int M>
-__device__ __forceinline__ void aes128_encrypt_n(uint32_t (&s)[M][4], const uint32_t* rk, const uint32_t* T) {
-  const char* Tc = reinterpret_cast<const char*>(T);
-  auto t0 = [&](uint32_t w) { return *reinterpret_cast<const uint32_t*>(Tc + ((w << 2) & 0x3fcu)); };
-  auto t1 = [&](uint32_t w) { return *reinterpret_cast<const uint32_t*>(Tc + 1024 + ((w >> 6) & 0x3fcu)); };
-  auto t2 = [&](uint32_t w) { return *reinterpret_cast<const uint32_t*>(Tc + 2048 + ((w >> 14) & 0x3fcu)); };
-  auto t3 = [&](uint32_t w) { return *reinterpret_cast<const uint32_t*>(Tc + 3072 + ((w >> 22) & 0x3fcu)); };
-#pragma unroll
-  for (int m = 0; m < M; ++m)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) s[m][c] ^= rk[c];
-#pragma unroll 1
-  for (int r = 1; r < 10; ++r) {
-    const uint32_t k0 = rk[4 * r], k1 = rk[4 * r + 1], k2 = rk[4 * r + 2], k3 = rk[4 * r + 3];
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      const uint32_t s0 = s[m][0], s1 = s[m][1], s2 = s[m][2], s3 = s[m][3];
-      s[m][0] = t0(s0) ^ t1(s1) ^ t2(s2) ^ t3(s3) ^ k0;
-      s[m][1] = t0(s1) ^ t1(s2) ^ t2(s3) ^ t3(s0) ^ k1;
-      s[m][2] = t0(s2) ^ t1(s3) ^ t2(s0) ^ t3(s1) ^ k2;
-      s[m][3] = t0(s3) ^ t1(s0) ^ t2(s1) ^ t3(s2) ^ k3;
-    }
-  }
-#pragma unroll
-  for (int m = 0; m < M; ++m) {
-    const uint32_t s0 = s[m][0], s1 = s[m][1], s2 = s[m][2], s3 = s[m][3];
-    s[m][0] = (__byte_perm(t0(s0), 0u, 0x4441u) | __byte_perm(t0(s1 >> 8), 0u, 0x4414u) |
-               __byte_perm(t0(s2 >> 16), 0u, 0x4144u) | __byte_perm(t0(s3 >> 24), 0u, 0x1444u)) ^ rk[40];
-    s[m][1] = (__byte_perm(t0(s1), 0u, 0x4441u) | __byte_perm(t0(s2 >> 8), 0u, 0x4414u) |
-               __byte_perm(t0(s3 >> 16), 0u, 0x4144u) | __byte_perm(t0(s0 >> 24), 0u, 0x1444u)) ^ rk[41];
-    s[m][2] = (__byte_perm(t0(s2), 0u, 0x4441u) | __byte_perm(t0(s3 >> 8), 0u, 0x4414u) |
-               __byte_perm(t0(s0 >> 16), 0u, 0x4144u) | __byte_perm(t0(s1 >> 24), 0u, 0x1444u)) ^ rk[42];
-    s[m][3] = (__byte_perm(t0(s3), 0u, 0x4441u) | __byte_perm(t0(s0 >> 8), 0u, 0x4414u) |
-               __byte_perm(t0(s1 >> 16), 0u, 0x4144u) | __byte_perm(t0(s2 >> 24), 0u, 0x1444u)) ^ rk[43];
-  }
 }
 
 // Counter block IV + n (128-bit big-endian addition) as four state columns.

@@ -334,7 +334,201 @@ __device__ __forceinline__ void decide_ties(const uint8_t* img, uint64_t pitch, 
   }
 }
 
-template <int K, bool BULK>
+// ---- packed storage (Sect. 6.4.3, Table 5): after a subtile's ties are decided its staged
+// coefficients are packed, the public part in place and out at once, the private parts of a few
+// subtiles side by side until they are encrypted.  The packing itself is the cost (11 bits: 61.6 M
+// warp instructions for 4096 x 4096, k = 5, against 41.8 M for int16): 80 us a launch, 104 us in
+// the grouped form, 101 us before private words were built per channel-block and fields were
+// placed by multiply-adds.
+
+// field code of AC value v in W bits: sign-magnitude; 8-bit storage saturates the magnitude, in 11
+// bits none is too large (|AC| <= 255 sum |basis| / 2 <= 1020)
+template <int W>
+__device__ __forceinline__ uint32_t ac_code(int v) {
+  const int s = v >> 31;
+  int mag = (v ^ s) - s;
+  if (W < 11) mag = min(mag, (1 << (W - 1)) - 1);
+  // a zero has no sign: s is 0 there
+  return ((uint32_t)s & (1u << (W - 1))) | (uint32_t)mag;
+}
+// w |= c << b for a field that does not overlap what w holds: a multiply-add, off the ALU
+__device__ __forceinline__ uint32_t put_bits(uint32_t w, uint32_t c, int b) { return c * (1u << b) + w; }
+
+// bytes of a full subtile's packed public and private part (multiples of 4, so that a subtile's
+// part of either stream starts on a word of it)
+template <int W>
+__device__ __forceinline__ uint32_t pack_pub_bytes(int k) {
+  return 4u * (uint32_t)((63 - k) * W);
+}
+template <int W>
+__host__ __device__ constexpr uint32_t pack_priv_bytes(int k) {
+  return 4u * (uint32_t)(kDcBits + k * W);
+}
+// packed private parts encrypted together: as many as leave the fewest lanes idle in the rounds of
+// 32 keystream blocks (a run of n parts overlaps at most 16-byte blocks of its bytes and one more),
+// as far as the area behind the int16 coefficients holds them; 0: none, packed in place
+constexpr int kPackAcc = kWStageBytes - kWCb * 128;
+template <int W>
+__host__ __device__ constexpr int pack_acc_tiles(int k) {
+  const int per = (int)pack_priv_bytes<W>(k);
+  int best = 0, bn = 0, bp = 1;
+  for (int g = 1; g <= 8 && g * per <= kPackAcc; ++g) {
+    const int n = g * per, p = (n / 16 + 1 + 31) / 32;
+    if (!best || n * bp > bn * p) {
+      best = g;
+      bn = n;
+      bp = p;
+    }
+  }
+  return best;
+}
+
+// Pack the staged int16 public coefficients of n channel-blocks in place: fields f (int16 at
+// pub + f) in groups of 32; group g fills words [W g, W g + W).  Each round reads its inputs into
+// registers before it writes, and the words it writes lie below what later rounds read (32 fields
+// are 64 bytes as int16, at most 44 packed).
+template <int W>
+__device__ __forceinline__ void pack_public(int16_t* pub, int n, int npub, int lane) {
+  const int nf = n * npub, ngroups = (nf + 31) >> 5;
+  uint32_t* const pubw = reinterpret_cast<uint32_t*>(pub);
+#pragma unroll 1
+  for (int r0 = 0; r0 < ngroups; r0 += 32) {
+    const int g = r0 + lane;
+    uint32_t pw[W];
+#pragma unroll
+    for (int j = 0; j < W; ++j) pw[j] = 0;
+    if (g < ngroups) {
+      const int f0 = 32 * g;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        // fields past the last one are zero padding (the area behind them is readable)
+        const uint4 x = reinterpret_cast<const uint4*>(pub + f0)[q];
+        const uint32_t u[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+          const int i = 8 * q + m;
+          int v = (int)(u[m >> 1] << (m & 1 ? 0 : 16)) >> 16;
+          if (f0 + i >= nf) v = 0;
+          const uint32_t c = ac_code<W>(v);
+          const int b = W * i;
+          pw[b >> 5] = put_bits(pw[b >> 5], c, b & 31);
+          if ((b & 31) + W > 32) pw[(b >> 5) + 1] |= c >> (32 - (b & 31));
+        }
+      }
+    }
+    __syncwarp();
+    if (g < ngroups) {
+#pragma unroll
+      for (int j = 0; j < W; ++j) pubw[W * g + j] = pw[j];
+    }
+    __syncwarp();
+  }
+}
+
+// Pack the staged int16 private coefficients of n channel-blocks to dst (their own place, or the
+// area behind them): word j gathers the fields overlapping bits [32 j, 32 j + 32); a channel-block
+// takes 11 + k W bits.  In place, a round's words lie below what later rounds read (a word holds
+// at least 2.9 fields, which took 5.8 bytes).
+template <int W>
+__device__ __forceinline__ void pack_private(const int16_t* priv, uint32_t* dst, int n, int k, int lane) {
+  const int period = kDcBits + k * W, pbits = n * period, nwords = (pbits + 31) >> 5;
+#pragma unroll 1
+  for (int r0 = 0; r0 < nwords; r0 += 32) {
+    const int g = r0 + lane;
+    uint32_t vw = 0;
+    if (g < nwords) {
+      const int bit = 32 * g, end = min(bit + 32, pbits);
+      int cb = bit / period;
+      const int r = bit - cb * period;
+      int z = r < kDcBits ? 0 : 1 + (r - kDcBits) / W;
+      int pos = cb * period + (z == 0 ? 0 : kDcBits + (z - 1) * W);
+      while (pos < end) {
+        const int v = priv[cb * (k + 1) + z];
+        const uint32_t c = z == 0 ? ((uint32_t)v & 0x7ffu) : ac_code<W>(v);
+        const int sh = pos - bit;   // in (-11, 32)
+        vw |= sh >= 0 ? c << sh : c >> (-sh);
+        pos += z == 0 ? kDcBits : W;
+        if (++z > k) {
+          z = 0;
+          ++cb;
+        }
+      }
+    }
+    __syncwarp();
+    if (g < nwords) dst[g] = vw;
+    __syncwarp();
+  }
+}
+
+// The same for a k known here, to an area of its own: a lane's channel-block as words, shifted to
+// its place and merged in (pack_private took a third of the packing's instructions at k = 5)
+template <int K, int W>
+__device__ __forceinline__ void pack_private_k(const int16_t* priv, uint32_t* dst, int n, int lane) {
+  constexpr int kPeriod = kDcBits + K * W, kWords = (kPeriod + 31) / 32;
+#pragma unroll 1
+  for (int i = lane; i < kPeriod; i += 32) dst[i] = 0;       // 32 channel-blocks: kPeriod words
+  uint32_t w[kWords + 1];
+#pragma unroll
+  for (int i = 0; i <= kWords; ++i) w[i] = 0;
+#pragma unroll
+  for (int z = 0; z <= K; ++z) {
+    const int v = priv[lane * (K + 1) + z];
+    const uint32_t c = z == 0 ? ((uint32_t)v & 0x7ffu) : ac_code<W>(v);
+    const int b = z == 0 ? 0 : kDcBits + (z - 1) * W, fw = z == 0 ? kDcBits : W;
+    w[b >> 5] = put_bits(w[b >> 5], c, b & 31);
+    if ((b & 31) + fw > 32) w[(b >> 5) + 1] |= c >> (32 - (b & 31));
+  }
+  __syncwarp();
+  if (lane < n) {
+    const int at = lane * kPeriod, sh = at & 31;
+    uint32_t* const q = dst + (at >> 5);
+#pragma unroll
+    for (int i = 0; i <= kWords; ++i) {
+      const uint32_t x = __funnelshift_l(i > 0 ? w[i - 1] : 0u, w[i], sh);   // w[kWords] holds no bits
+      if (x) atomicOr(q + i, x);
+    }
+  }
+  __syncwarp();
+}
+
+// AES-128-CTR over the packed bytes [off, off + bytes) of the private stream at w (off a multiple
+// of 4): a lane per keystream block they overlap; a block that two warps' parts share is generated
+// by both, each XORing its own words
+__device__ __forceinline__ void ctr_packed(const TileArgs& a, uint32_t* w, uint64_t off, int bytes, int lane) {
+  const PairLanes lc = pair_lanes();
+  const uint64_t b0 = off >> 4;
+  const int nblk = (int)(((off + (uint64_t)bytes + 15) >> 4) - b0);
+  const int nw = (bytes + 3) >> 2, skew = (int)((off & 15) >> 2);
+#pragma unroll 1
+  for (int i = lane; i < nblk; i += 32) {
+    uint32_t s[4];
+    ctr_block(a.iv_hi, a.iv_lo, b0 + i, s);
+    aes128_encrypt_pair(s, a.rk, lc);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const int wi = 4 * i + m - skew;
+      if (wi >= 0 && wi < nw) w[wi] ^= s[m];
+    }
+  }
+}
+
+// packed bytes to a stream by the whole warp, as wide as the destination is aligned
+__device__ __forceinline__ void store_packed(uint8_t* dst, const uint8_t* src, int bytes, int lane) {
+  const uintptr_t al = reinterpret_cast<uintptr_t>(dst);
+  if ((al & 7) == 0) {
+    for (int i = lane; i < (bytes >> 3); i += 32) reinterpret_cast<uint2*>(dst)[i] = reinterpret_cast<const uint2*>(src)[i];
+    if (lane < (bytes & 7)) dst[(bytes & ~7) + lane] = src[(bytes & ~7) + lane];
+  } else if ((al & 3) == 0) {
+    for (int i = lane; i < (bytes >> 2); i += 32)
+      reinterpret_cast<uint32_t*>(dst)[i] = reinterpret_cast<const uint32_t*>(src)[i];
+    if (lane < (bytes & 3)) dst[(bytes & ~3) + lane] = src[(bytes & ~3) + lane];
+  } else {
+    for (int i = lane; i < bytes; i += 32) dst[i] = src[i];
+  }
+}
+
+// PACK: 0 = int16 fragments; 11 or 8 = packed streams
+template <int K, bool BULK, int PACK = 0>
 __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __grid_constant__ TileArgs a) {
   extern __shared__ __align__(128) uint8_t smem_cta[];
   const uint32_t win0 = smem_u32(smem_cta);
@@ -366,7 +560,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
   const uint32_t iv8 = (uint32_t)a.iv_lo & 255u;
   uint64_t wbase = (iv8 + (uint64_t)s0 * nb) >> 8;
   const uint64_t wlast = (iv8 + (uint64_t)s1 * nb - 1) >> 8;
-  const bool dynamic = wlast - wbase < kWins;
+  const bool dynamic = PACK == 0 && wlast - wbase < kWins;
   uint32_t t = s1, tend = s1;
   if (warp < act) {
     t = dynamic ? s0 + warp : s0 + (uint32_t)((uint64_t)(s1 - s0) * warp / act);
@@ -389,7 +583,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
   }
   fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
   __syncthreads();
-  if (!a.plain_private) {
+  if (PACK == 0 && !a.plain_private) {
     if (dynamic) {
       const int i = (int)threadIdx.x;
       if ((uint32_t)(i & ~31) <= wlast - wbase) put_window(a, wbase + i, (uint32_t)i <= wlast - wbase ? i : -1, wins);
@@ -435,10 +629,38 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
     bulk_wait_read_all();                  // the staging area may be written again
     __syncwarp();
     int16_t* pub_cb = pubst + lane * npub;
-    int16_t* priv_cb = reinterpret_cast<int16_t*>(privst) + (acc * kWCb + lane) * (k + 1);
+    int16_t* priv_cb = reinterpret_cast<int16_t*>(privst) + ((PACK ? 0 : acc * kWCb) + lane) * (k + 1);
     uint32_t mlo, mhi;
     stage_columns(P, V, k, (uint32_t)lane < n, pub_cb, priv_cb, mlo, mhi);
     decide_ties(a.pixels_in, pitch, (uint32_t)a.bx_count, 32u * t, c, k, mlo, mhi, pub_cb, priv_cb, ctab, lane, nties, esc, fail);
+    if constexpr (PACK != 0) {
+      constexpr int kPW = PACK ? PACK : 8;
+      __syncwarp();                        // every staged coefficient is final
+      pack_public<kPW>(pubst, (int)n, npub, lane);
+      store_packed(reinterpret_cast<uint8_t*>(a.pub_out) + (uint64_t)t * pack_pub_bytes<kPW>(k), stage,
+                   ((int)n * npub * kPW + 7) >> 3, lane);
+      const uint32_t per = pack_priv_bytes<kPW>(k);
+      const int GP = K >= 0 ? pack_acc_tiles<kPW>(K >= 0 ? K : 0) : a.aes_pair;
+      uint8_t* const pst = GP ? stage + kWCb * 128 : privst;
+      if constexpr (K >= 0 && pack_acc_tiles<kPW>(K >= 0 ? K : 0) > 0)
+        pack_private_k<K, kPW>(reinterpret_cast<const int16_t*>(privst), reinterpret_cast<uint32_t*>(pst + acc * per), (int)n,
+                               lane);
+      else
+        pack_private<kPW>(reinterpret_cast<const int16_t*>(privst), reinterpret_cast<uint32_t*>(pst + acc * per), (int)n, k,
+                          lane);
+      ++acc;
+      if (acc >= GP || tn >= tend) {
+        const uint64_t off = (uint64_t)(t + 1 - acc) * per;
+        const int bytes = (acc - 1) * (int)per + (((int)n * (kDcBits + k * kPW) + 7) >> 3);
+        ctr_packed(a, reinterpret_cast<uint32_t*>(pst), off, bytes, lane);
+        __syncwarp();
+        store_packed(a.priv_out + off, pst, bytes, lane);
+        acc = 0;
+      }
+      __syncwarp();                        // the staging area may be written again
+      t = tn;
+      continue;
+    }
     fence_proxy_async();                   // staged coefficients, before the bulk store
     __syncwarp();
     if (lane == 0) store_run(reinterpret_cast<uint8_t*>(a.pub_out) + (uint64_t)t * (64u * npub), stage, (int)n * 2 * npub);
@@ -625,7 +847,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
   }
 }
 
-template <int K, bool BULK>
+template <int K, bool BULK, int PACK = 0>
 static cudaError_t launch_w(const TileArgs& a, cudaStream_t s, int sms) {
   static bool attr[kMaxAttrDevices];
   static bool window_ok[kMaxAttrDevices];
@@ -634,10 +856,10 @@ static cudaError_t launch_w(const TileArgs& a, cudaStream_t s, int sms) {
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxAttrDevices) return cudaErrorInvalidDevice;
   if (!window_ok[dev]) {
-    if ((e = smem_window_start_ok(protect_warp_kernel<K, BULK>, (uint32_t)kWLow)) != cudaSuccess) return e;
+    if ((e = smem_window_start_ok(protect_warp_kernel<K, BULK, PACK>, (uint32_t)kWLow)) != cudaSuccess) return e;
     window_ok[dev] = true;
   }
-  e = smem_attr_once(protect_warp_kernel<K, BULK>, kWEnd, attr);
+  e = smem_attr_once(protect_warp_kernel<K, BULK, PACK>, kWEnd, attr);
   if (e != cudaSuccess) return e;
   TileArgs b = a;
   const long long nsub = (3ll * a.nblocks + 31) / 32;
@@ -645,8 +867,8 @@ static cudaError_t launch_w(const TileArgs& a, cudaStream_t s, int sms) {
   const long long per = (nsub + grid - 1) / (grid ? grid : 1);
   b.groups = (int)(per < kWarps ? per : kWarps);
   bx_division(b);
-  b.aes_pair = acc_tiles(a.k);
-  if (grid > 0) protect_warp_kernel<K, BULK><<<grid, kWarps * 32, kWEnd, s>>>(b);
+  b.aes_pair = PACK == 11 ? pack_acc_tiles<11>(a.k) : (PACK == 8 ? pack_acc_tiles<8>(a.k) : acc_tiles(a.k));
+  if (grid > 0) protect_warp_kernel<K, BULK, PACK><<<grid, kWarps * 32, kWEnd, s>>>(b);
   return cudaGetLastError();
 }
 
@@ -680,10 +902,15 @@ cudaError_t launch_protect_plan(const TileArgs& a, cudaStream_t s, int sms, int 
 }
 
 cudaError_t launch_protect_warp(const TileArgs& a, cudaStream_t s, int sms) {
-  if (a.images || a.pack || a.k < 0 || a.k > 63) return cudaErrorInvalidValue;
+  if (a.images || a.k < 0 || a.k > 63 || (a.pack && a.pack != 11 && a.pack != 8)) return cudaErrorInvalidValue;
   // bulk copies of whole row runs need 16-byte aligned pixels and subtiles of at most two block
   // rows
-  if (a.bx_count >= 12 && ((uintptr_t)a.pixels_in & 15) == 0) {
+  const bool bulk = a.bx_count >= 12 && ((uintptr_t)a.pixels_in & 15) == 0;
+  if (a.pack == 11) return !bulk ? launch_w<-1, false, 11>(a, s, sms)
+                                 : (a.k == 5 ? launch_w<5, true, 11>(a, s, sms) : launch_w<-1, true, 11>(a, s, sms));
+  if (a.pack == 8) return !bulk ? launch_w<-1, false, 8>(a, s, sms)
+                                : (a.k == 5 ? launch_w<5, true, 8>(a, s, sms) : launch_w<-1, true, 8>(a, s, sms));
+  if (bulk) {
     if (a.k == 0) return launch_w<0, true>(a, s, sms);
     if (a.k == 5) return launch_w<5, true>(a, s, sms);
     return launch_w<-1, true>(a, s, sms);

@@ -1,11 +1,10 @@
 // Fused restore kernel (defragmentation, Sect. 3.2, Fig. 3; inverse of Sect. 6.3.1) in its tiled
-// form, for batches, packed storage and the tensor-core inverse (one image in int16 storage and
-// the public-image form: fds_restore_warp.cu): CTR
-// decryption of the confidential fragment, merge with the public fragment by zigzag
-// position, inverse 8x8 DCT, round half away from zero (exact), clamp to [0, 255].
+// form, for packed storage and the tensor-core inverse (int16 storage, batches and the public-image
+// form: fds_restore_warp.cu): CTR decryption of the confidential fragment, merge with the public
+// fragment by zigzag position, inverse 8x8 DCT, round half away from zero (exact), clamp to
+// [0, 255].
 //
-// Persistent CTAs over a tile schedule (one image, or every tile of a batch of images in one
-// launch); per tile (see fds_tile.cuh for the decomposition):
+// Persistent CTAs over the image's tiles, b, b + gridDim.x, ..; per tile (see fds_tile.cuh):
 //   A. the tile's fragments are in shared memory, already decrypted; the next tile's start
 //      loading (one bulk copy per fragment range, or cp.async pieces)
 //   1. per channel-block: column then row float32 inverse butterflies (the column pass and
@@ -247,39 +246,32 @@ __device__ __forceinline__ void wait_fragments(const TileSlot* sl, uint64_t* bar
   }
 }
 
-// CTR decryption of the private range of slot sl's tile, in staging area st; REP: Ts is the
-// lane-replicated table, else the four T-tables
-template <bool REP>
-__device__ __forceinline__ void decrypt_fragments(const TileSlot* sl, const uint32_t* rk, uint8_t* st,
-                                                  const uint32_t* Ts, bool aes_pair = false) {
+// CTR decryption of the private range of slot sl's tile, in staging area st (int16 storage)
+__device__ __forceinline__ void decrypt_fragments(const TileSlot* sl, const uint32_t* rk, uint8_t* st, const uint32_t* Trep) {
   const int k = sl->k;
-  const int bytes = sl->nb * 6 * (k + 1);
   const uint64_t first = ((uint64_t)sl->local * kTileBlocks * 6ull * (uint64_t)(k + 1)) >> 4;
-  if constexpr (REP)
-    ctr_tile_rep(st + kTileCb * 2 * (63 - k), bytes, first, sl, rk, Ts, aes_pair, (int)threadIdx.x);
-  else
-    ctr_tile(st + kTileCb * 2 * (63 - k), bytes, first, sl, rk, Ts, aes_pair, (int)threadIdx.x);
+  ctr_tile_rep(st + kTileCb * 2 * (63 - k), sl->nb * 6 * (k + 1), first, sl, rk, Trep, (int)threadIdx.x);
 }
 
-// BATCH: tiles of many images (round keys from the slot); else one image (round keys read
-// from the kernel parameters, which AES then takes as constant-bank operands)
+// one image (round keys read from the kernel parameters, which AES then takes as constant-bank
+// operands)
 // TC: the inverse transform as tcgen05 MMAs (one image, int16 storage; a.tc_b = the inverse
 // basis table); a tile holding a coefficient of magnitude 2048 or more takes the float32
 // butterflies instead.
-template <int K, bool BATCH, int PACK = 0, bool TC = false>
+template <int K, int PACK = 0, bool TC = false>
 __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel(const __grid_constant__ TileArgs a) {
-  static_assert(!TC || (!BATCH && PACK == 0), "tensor-core inverse: one image, int16 storage");
+  static_assert(TC != (PACK != 0), "packed streams, or the tensor-core inverse of int16 storage");
   extern __shared__ __align__(128) uint8_t smem[];
   // AES tables: T0 replicated per lane (one image, int16 storage, private fragment decrypted),
   // else the four T-tables
-  constexpr bool REP = !BATCH && PACK == 0;
+  constexpr bool REP = PACK == 0;
   __shared__ __align__(16) uint32_t T4[REP ? 4 : 1024];
   uint32_t* Ts = REP ? reinterpret_cast<uint32_t*>(smem + kSmemTrep) : T4;
   uint32_t* queue = reinterpret_cast<uint32_t*>(smem + kSmemQueue);
   // misc: [0] queue size, [1] queued total, [2] escalations, [3] failures, [4..5] schedule
   int* misc = reinterpret_cast<int*>(smem + kSmemMisc);
   const int t = threadIdx.x;
-  const int ntiles = a.images ? a.total_tiles : (a.nblocks + kTileBlocks - 1) / kTileBlocks;
+  const int ntiles = (a.nblocks + kTileBlocks - 1) / kTileBlocks;
   if ((int)blockIdx.x >= ntiles) return;
   auto slot = [&](int i) { return reinterpret_cast<TileSlot*>(smem + kSmemSlot + i * kSlotBytes); };
   auto stage = [&](int i) { return smem + kSmemCoef + i * kCoefBytes; };
@@ -292,8 +284,8 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
   if (t < 4) misc[t] = 0;
   if (t == 0) {
     misc[6] = 0;                         // TC: a tensor-core wait gave up
-    misc[4] = next_tile(a, 0, blockIdx.x, gridDim.x);
-    misc[5] = next_tile(a, 1, blockIdx.x, gridDim.x);
+    misc[4] = blockIdx.x;
+    misc[5] = blockIdx.x + gridDim.x;
   }
   if (t < kTileBlocks) fill_slot(a, blockIdx.x, slot(0), t);
   __syncthreads();
@@ -335,7 +327,7 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
     wait_fragments(slot(0), bars, phase[0], lost);
     __syncthreads();
     if (!a.plain_private)
-      decrypt_fragments<REP>(slot(0), BATCH ? slot(0)->rk : a.rk, stage(0), Ts, BATCH && a.aes_pair);
+      decrypt_fragments(slot(0), a.rk, stage(0), Ts);
   }
   int esc = 0;
   bool fail = false;
@@ -362,7 +354,7 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
       asm volatile("cp.async.bulk.wait_group.read 1;\n" ::: "memory");
     }
     __syncthreads();                                                       // A
-    if (t == 0) misc[4 + buf] = nxt < ntiles ? next_tile(a, it + 2, blockIdx.x, gridDim.x) : ntiles;
+    if (t == 0) misc[4 + buf] = nxt < ntiles ? (int)(blockIdx.x + (it + 2) * gridDim.x) : ntiles;
     if (nxt < ntiles) {
       if constexpr (PACK != 0)
         load_packed<PACK>(slot((it + 1) % 3), land, bars + (buf ^ 1));
@@ -565,8 +557,7 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
         unpack_tile<PACK>(slot((it + 1) % 3), land, stage(buf ^ 1));
       }
     } else if (nxt < ntiles && !a.plain_private) {
-      decrypt_fragments<REP>(slot((it + 1) % 3), BATCH ? slot((it + 1) % 3)->rk : a.rk, stage(buf ^ 1), Ts,
-                        BATCH && a.aes_pair);
+      decrypt_fragments(slot((it + 1) % 3), a.rk, stage(buf ^ 1), Ts);
     }
     fence_proxy_async();                                  // pixel writes before the bulk stores
     const bool skip = __syncthreads_or(cur_lost != 0);                     // C
@@ -578,7 +569,7 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
       // tile's blocks are contiguous and 16-byte aligned in every row, else 8-byte stores
       const uint64_t w3 = (uint64_t)sl->width * 3ull;
       uint8_t* row0 = sl->px_out + sl->blk[0];
-      if (sl->px_flags & kPxOut16) {
+      if (sl->px_out16) {
         if (t == 0) {
 #pragma unroll 1
           for (int y = 0; y < 8; ++y) bulk_store(row0 + y * w3, pix + y * kRowBytes, (uint32_t)(nb * 24));
@@ -612,18 +603,18 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
   }
 }
 
-template <int K, bool BATCH, int PACK = 0, bool TC = false>
+template <int K, int PACK = 0, bool TC = false>
 static cudaError_t launch_k(const TileArgs& a, cudaStream_t s, int sms, int per_sm) {
   static bool attr[kMaxAttrDevices];
   static int resident[kMaxAttrDevices];
-  constexpr int smem = TC ? kSmemBytesTc : (PACK ? kSmemBytesPacked : (BATCH ? kSmemBytes : kSmemBytesRep));
-  cudaError_t e = smem_attr_once(restore_kernel<K, BATCH, PACK, TC>, smem, attr);
+  constexpr int smem = TC ? kSmemBytesTc : (PACK ? kSmemBytesPacked : kSmemBytesRep);
+  cudaError_t e = smem_attr_once(restore_kernel<K, PACK, TC>, smem, attr);
   if (e != cudaSuccess) return e;
   const int ntiles = total_tiles(a);
-  const int r = resident_ctas(restore_kernel<K, BATCH, PACK, TC>, kThreads, smem, resident);
+  const int r = resident_ctas(restore_kernel<K, PACK, TC>, kThreads, smem, resident);
   const int cap = (per_sm >= 1 && per_sm < r ? per_sm : r) * sms;
   const int grid = ntiles < cap ? ntiles : cap;
-  if (grid > 0) restore_kernel<K, BATCH, PACK, TC><<<grid, kThreads, smem, s>>>(a);
+  if (grid > 0) restore_kernel<K, PACK, TC><<<grid, kThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -631,9 +622,9 @@ static cudaError_t launch_k(const TileArgs& a, cudaStream_t s, int sms, int per_
 // one CTA per SM (the operands and TMEM take what a second CTA would need)
 cudaError_t launch_restore_tc(const TileArgs& a, cudaStream_t s, int sms) {
   if (a.images || a.k < 0 || a.public_image || a.pack || a.plain_private || !a.tc_b) return cudaErrorInvalidValue;
-  if (a.k == 0) return launch_k<0, false, 0, true>(a, s, sms, 1);
-  if (a.k == 5) return launch_k<5, false, 0, true>(a, s, sms, 1);
-  return launch_k<-1, false, 0, true>(a, s, sms, 1);
+  if (a.k == 0) return launch_k<0, 0, true>(a, s, sms, 1);
+  if (a.k == 5) return launch_k<5, 0, true>(a, s, sms, 1);
+  return launch_k<-1, 0, true>(a, s, sms, 1);
 }
 
 // k is uniform over the launch when a.k >= 0; a.k < 0 (batches of mixed k) reads k per tile;
@@ -641,9 +632,9 @@ cudaError_t launch_restore_tc(const TileArgs& a, cudaStream_t s, int sms) {
 cudaError_t launch_restore(const TileArgs& a, cudaStream_t s, int sms, int per_sm) {
   if (a.pack) {   // one image, packed streams in pub_in / priv_in
     if (a.images || a.k < 0 || a.public_image || (a.pack != 11 && a.pack != 8)) return cudaErrorInvalidValue;
-    if (a.pack == 11) return a.k == 5 ? launch_k<5, false, 11>(a, s, sms, per_sm)
-                                      : launch_k<-1, false, 11>(a, s, sms, per_sm);
-    return a.k == 5 ? launch_k<5, false, 8>(a, s, sms, per_sm) : launch_k<-1, false, 8>(a, s, sms, per_sm);
+    if (a.pack == 11) return a.k == 5 ? launch_k<5, 11>(a, s, sms, per_sm)
+                                      : launch_k<-1, 11>(a, s, sms, per_sm);
+    return a.k == 5 ? launch_k<5, 8>(a, s, sms, per_sm) : launch_k<-1, 8>(a, s, sms, per_sm);
   }
   if (a.images) return launch_restore_plan(a, s, sms, per_sm);
   return launch_restore_warp(a, s, sms);

@@ -134,16 +134,6 @@ __device__ __forceinline__ void sha256_rounds(uint32_t (&v)[8], uint32_t (&w)[16
   v[7] = hh;
 }
 
-// one SHA-256 compression of the 16 big-endian words w into state h
-__device__ __forceinline__ void sha256_compress(uint32_t (&h)[8], uint32_t (&w)[16]) {
-  uint32_t v[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = h[i];
-  sha256_rounds<0>(v, w);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) h[i] += v[i];
-}
-
 // this translation unit's copy of the constants, to the current device
 static cudaError_t upload_sha_tables() {
   uint64_t k[80], h0[8];

@@ -1,14 +1,11 @@
-// Tile machinery shared by the fused protect and restore kernels.
+// What the fused kernels share: their arguments, copies and barriers, and the tiles of the kernels
+// that work on 64 blocks at a time (packed restore, the tensor-core forms; the plans' schedules
+// count in them too).
 //
-// Work decomposition: a tile is 64 consecutive 8x8 pixel blocks (row-major over an image's
-// block grid); one thread per channel-block (cb = 3 * block + channel, 192 threads per CTA).
-// A tile's public and private outputs are contiguous, 16-byte aligned byte ranges
-// (64 blocks x 3 channels x 2(63-k) or 2(k+1) bytes), so a tile stages them in shared memory
-// and moves them with 16-byte (or bulk) copies; the tile's private range is a whole number of
-// AES blocks, so CTR needs nothing from neighbouring tiles.
-//
-// The kernels are persistent: each CTA walks tiles blockIdx.x, blockIdx.x + gridDim.x, ...
-// and prefetches the next tile's input with cp.async while it transforms the current one.
+// A tile is 64 consecutive 8x8 pixel blocks (row-major over an image's block grid), 192
+// channel-blocks (cb = 3 * block + channel).  Its public and private parts are contiguous,
+// 16-byte aligned byte ranges (64 blocks x 3 channels x 2(63-k) or 2(k+1) bytes), the private one a
+// whole number of AES blocks, so CTR needs nothing from neighbouring tiles.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -103,9 +100,10 @@ struct TileArgs {
   int32_t pack;
   // restore in the public-image form (one image): private positions zero, DC 1024
   int32_t public_image;
-  // AES lane schedule of the batched form: nonzero = two keystream blocks per thread
+  // warp forms of one image: subtiles whose private parts go through AES together (filled in by
+  // the launcher).  A plan's AES lane schedule arrives here too; its kernels have only one.
   int32_t aes_pair;
-  // protect: tile groups that work in each CTA (1 .. the kernel's groups; 0 = all of them)
+  // warp forms: working warps of each CTA (filled in by the launcher)
   int32_t groups;
   // strong level (protect of one image): Part 1 is also left here in plaintext
   uint8_t* plain_out;
@@ -114,30 +112,26 @@ struct TileArgs {
   int32_t bx_shift;
 };
 
-// What a CTA knows about the tile it is working on (shared memory, filled one tile ahead).
+// What a CTA of the tiled restore knows about the tile it is working on (shared memory, filled one
+// tile ahead).
 struct TileSlot {
   uint64_t blk[kTileBlocks];      // byte offset of each block's top-left pixel in the image
-  uint32_t rk[44];                // the image's AES-128 round keys
-  const uint8_t* px_in;           // the image's pixels, public and private fragments
-  uint8_t* px_out;
+  uint8_t* px_out;                // the image's pixels, public and private fragments
   const uint8_t* pub_in;
-  uint8_t* pub_out;
   const uint8_t* priv_in;
-  uint8_t* priv_out;
   uint64_t iv_hi, iv_lo;
   int32_t width, k, local, nb;    // local = tile index inside the image; nb = its blocks
-  // the tile's 8 pixel rows are contiguous runs of nb * 24 bytes in the image, 16-byte aligned
-  // (kPxIn16: in px_in, a whole tile; kPxOut16: in px_out)
-  int32_t px_flags;
+  // nonzero: the tile's 8 pixel rows are contiguous runs of nb * 24 bytes in the image, 16-byte
+  // aligned
+  int32_t px_out16;
 };
-constexpr int32_t kPxIn16 = 1, kPxOut16 = 2;
 
-// launchers (one translation unit each); `sms` = number of SMs of the device, `per_sm` =
-// tile groups per SM to launch, at most the kernel's residency (protect: 3 groups of one CTA
-// for one image, 4 CTAs for batches; restore: 2 CTAs); 0 = that residency
+// launchers (one translation unit each); `sms` = number of SMs of the device; `per_sm` counts
+// quarters (protect of a batch, 1 .. 4) or halves (its restore, 1 .. 2) of a CTA's sixteen warps,
+// or CTAs (packed restore, 1 .. 2); 0 = all
 cudaError_t launch_protect(const TileArgs& a, cudaStream_t s, bool debug, int sms, int per_sm = 0);
 cudaError_t launch_restore(const TileArgs& a, cudaStream_t s, int sms, int per_sm = 0);
-// protect of one image in int16 storage, one subtile of 32 channel-blocks per warp
+// protect of one image (int16 or packed storage), one subtile of 32 channel-blocks per warp
 cudaError_t launch_protect_warp(const TileArgs& a, cudaStream_t s, int sms);
 // protect of a batch, likewise; k as in launch_protect
 cudaError_t launch_protect_plan(const TileArgs& a, cudaStream_t s, int sms, int per_sm);
@@ -183,12 +177,6 @@ inline int resident_ctas(Kernel kernel, int threads, int bytes, int (&cache)[kMa
 
 inline int total_tiles(const TileArgs& a) {
   return a.images ? a.total_tiles : (a.nblocks + kTileBlocks - 1) / kTileBlocks;
-}
-
-// barrier of one 192-thread tile group of a CTA (named barrier `id`, never 0: that is the
-// CTA-wide __syncthreads)
-__device__ __forceinline__ void group_sync(int id) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kThreads) : "memory");
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -266,70 +254,29 @@ __device__ __forceinline__ uint64_t block_offset(int width, int gb) {
   return (uint64_t)by * 8ull * (uint64_t)width * 3ull + (uint64_t)bx * 24ull;
 }
 
-// Fill slot s for global tile g.  Called by threads t = 0 .. kTileBlocks-1 of the tile group
-// (each writes its own fields); the caller publishes the slot with a barrier.
+// Fill slot s for tile g of the image.  Called by threads t = 0 .. kTileBlocks-1 (each writes its
+// own fields); the caller publishes the slot with a barrier.
 __device__ __forceinline__ void fill_slot(const TileArgs& a, int g, TileSlot* s, int t) {
-  int width, nblocks, k, local;
-  uint64_t iv_hi, iv_lo, pxo = 0, puo = 0, pro = 0;
-  const uint32_t* rk;
-  if (a.images == nullptr) {
-    width = a.width, nblocks = a.nblocks, k = a.k, local = g;
-    iv_hi = a.iv_hi, iv_lo = a.iv_lo;
-    rk = a.rk;
-  } else {
-    int lo = 0, hi = a.n_images;                 // tile_start[lo] <= g < tile_start[hi]
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (__ldg(a.tile_start + mid) <= g)
-        lo = mid;
-      else
-        hi = mid;
-    }
-    const BatchImage& im = a.images[lo];
-    width = im.width, k = im.k, local = g - __ldg(a.tile_start + lo);
-    nblocks = (im.width >> 3) * (im.height >> 3);
-    iv_hi = im.iv_hi, iv_lo = im.iv_lo;
-    pxo = im.pixel_offset, puo = im.public_offset, pro = im.private_offset;
-    rk = a.round_keys + 44 * im.key_slot;
-  }
-  const int nb = min(kTileBlocks, nblocks - local * kTileBlocks);
+  const int nb = min(kTileBlocks, a.nblocks - g * kTileBlocks);
   if (t == 0) {
-    s->px_in = a.pixels_in + pxo;
-    s->px_out = a.pixels_out + pxo;
-    s->pub_in = reinterpret_cast<const uint8_t*>(a.pub_in) + puo;
-    s->pub_out = reinterpret_cast<uint8_t*>(a.pub_out) + puo;
-    s->priv_in = a.priv_in + pro;
-    s->priv_out = a.priv_out + pro;
-    s->iv_hi = iv_hi;
-    s->iv_lo = iv_lo;
-    s->width = width;
-    s->k = k;
-    s->local = local;
+    s->px_out = a.pixels_out;
+    s->pub_in = reinterpret_cast<const uint8_t*>(a.pub_in);
+    s->priv_in = a.priv_in;
+    s->iv_hi = a.iv_hi;
+    s->iv_lo = a.iv_lo;
+    s->width = a.width;
+    s->k = a.k;
+    s->local = g;
     s->nb = nb;
-    const int bxc = width >> 3;
-    const uint64_t w3 = 3ull * (uint64_t)width, b0 = block_offset(width, local * kTileBlocks);
-    const bool rows = (local * kTileBlocks) % bxc + nb <= bxc && ((nb * 24) & 15) == 0 && (w3 & 15) == 0;
-    int32_t f = 0;
-    if (rows && nb == kTileBlocks && (reinterpret_cast<uintptr_t>(a.pixels_in + pxo + b0) & 15) == 0) f |= kPxIn16;
-    if (rows && (reinterpret_cast<uintptr_t>(a.pixels_out + pxo + b0) & 15) == 0) f |= kPxOut16;
-    s->px_flags = f;
+    const int bxc = a.width >> 3;
+    const uint64_t w3 = 3ull * (uint64_t)a.width, b0 = block_offset(a.width, g * kTileBlocks);
+    const bool rows = (g * kTileBlocks) % bxc + nb <= bxc && ((nb * 24) & 15) == 0 && (w3 & 15) == 0;
+    s->px_out16 = rows && (reinterpret_cast<uintptr_t>(a.pixels_out + b0) & 15) == 0;
   }
-  if (t < 44) s->rk[t] = rk[t];
-  if (t < nb) s->blk[t] = block_offset(width, local * kTileBlocks + t);
-}
-
-// Tile schedule of a persistent tile group (vb = its index among the launch's vgrid groups;
-// a group is a CTA, or one of the CTA's independent 192-thread groups): the i-th tile is
-// vb + i * vgrid (static), or for i >= 1 the value of an atomic counter plus vgrid (dynamic,
-// a.dispenser non-null; the counter must be zero at launch).  Called by one thread.
-__device__ __forceinline__ int next_tile(const TileArgs& a, int i, int vb, int vgrid) {
-  if (a.dispenser == nullptr || i == 0) return vb + i * vgrid;
-  return (int)atomicAdd(a.dispenser, 1u) + vgrid;
+  if (t < nb) s->blk[t] = block_offset(a.width, g * kTileBlocks + t);
 }
 
 // column pairs of the packed column pass: (0, 4), (1, 2), (3, 5), (6, 7)
-__host__ __device__ constexpr int pair_of(int v) { return (v == 0 || v == 4) ? 0 : (v < 3 ? 1 : ((v == 3 || v == 5) ? 2 : 3)); }
-__host__ __device__ constexpr int pair_lane(int v) { return (v == 4 || v == 2 || v == 5 || v == 7) ? 1 : 0; }
 __host__ __device__ constexpr int pair_col(int j, int l) {
   return j == 0 ? (l ? 4 : 0) : (j == 1 ? (l ? 2 : 1) : (j == 2 ? (l ? 5 : 3) : (l ? 7 : 6)));
 }
@@ -347,90 +294,18 @@ __device__ __forceinline__ void load_row_shifted(const uint8_t* tile, int y, int
 }
 
 // AES-128-CTR over `bytes` bytes of a 16-byte aligned staging area whose first byte is byte
-// 16 * first_block of the image's private message.
-// The IV comes from the tile's slot; rk are the 44 round keys.  aes_pair: each thread takes
-// two keystream blocks, i and i + kThreads, encrypted interleaved (the lane schedule the
-// batched form's autotuner can choose), instead of one.
-__device__ __forceinline__ void ctr_tile(uint8_t* st, int bytes, uint64_t first_block,
-                                         const TileSlot* sl, const uint32_t* rk, const uint32_t* Ts,
-                                         bool aes_pair, int t) {
-  const int nblk = (bytes + 15) >> 4;
-  if (aes_pair) {
-    for (int i = t; i < nblk; i += 2 * kThreads) {
-      const bool two = i + kThreads < nblk;
-      uint32_t s[2][4];
-      ctr_block(sl->iv_hi, sl->iv_lo, first_block + i, s[0]);
-      ctr_block(sl->iv_hi, sl->iv_lo, first_block + i + kThreads, s[1]);
-      aes128_encrypt_n<2>(s, rk, Ts);
-#pragma unroll
-      for (int m = 0; m < 2; ++m) {
-        if (m == 1 && !two) break;
-        uint4* p = reinterpret_cast<uint4*>(st + 16 * (i + m * kThreads));
-        uint4 d = *p;
-        d.x ^= s[m][0];
-        d.y ^= s[m][1];
-        d.z ^= s[m][2];
-        d.w ^= s[m][3];
-        *p = d;
-      }
-    }
-    return;
-  }
-  for (int i = t; i < nblk; i += kThreads) {
-    uint32_t s[4];
-    ctr_block(sl->iv_hi, sl->iv_lo, first_block + i, s);
-    aes128_encrypt(s, rk, Ts);
-    uint4* p = reinterpret_cast<uint4*>(st + 16 * i);
-    uint4 d = *p;
-    d.x ^= s[0];
-    d.y ^= s[1];
-    d.z ^= s[2];
-    d.w ^= s[3];
-    *p = d;
-  }
-}
-
-// ctr_tile with a replicated T0 table (2^(SH-2) copies at Trep, entry x of copy c at word
-// 2^(SH-2) x + c; SH = 7: every lookup of a warp hits 32 distinct banks).  aes_pair as in
-// ctr_tile; t = the thread's index in its 192-thread tile group.
+// 16 * first_block of the image's private message.  The IV comes from the tile's slot; rk are the
+// 44 round keys; Trep: T0 replicated 2^(SH-2) times (entry x of copy c at word 2^(SH-2) x + c;
+// SH = 7: every lookup of a warp hits 32 distinct banks); t = the thread's index.
 template <int SH = 7>
 __device__ __forceinline__ void ctr_tile_rep(uint8_t* st, int bytes, uint64_t first_block, const TileSlot* sl,
-                                             const uint32_t* rk, const uint32_t* Trep, bool aes_pair, int t) {
+                                             const uint32_t* rk, const uint32_t* Trep, int t) {
   const int nblk = (bytes + 15) >> 4;
   const uint32_t Tl = smem_u32(Trep) + 4u * (t & ((1 << (SH - 2)) - 1));
-  const int step = aes_pair ? 2 * kThreads : kThreads;
-  for (int i = t; i < nblk; i += step) {
-    const int m_n = aes_pair && i + kThreads < nblk ? 2 : 1;
-    uint32_t s[2][4];
-    ctr_block(sl->iv_hi, sl->iv_lo, first_block + i, s[0]);
-    if (aes_pair) {
-      ctr_block(sl->iv_hi, sl->iv_lo, first_block + i + kThreads, s[1]);
-      aes128_encrypt_rep_n<2, SH>(s, rk, Tl);
-    } else {
-      aes128_encrypt_rep<SH>(s[0], rk, Tl);
-    }
-    for (int m = 0; m < m_n; ++m) {
-      uint4* p = reinterpret_cast<uint4*>(st + 16 * (i + m * kThreads));
-      uint4 d = *p;
-      d.x ^= s[m][0];
-      d.y ^= s[m][1];
-      d.z ^= s[m][2];
-      d.w ^= s[m][3];
-      *p = d;
-    }
-  }
-}
-
-// ctr_tile with the pair table (window address kTpairWin, see aes128_encrypt_pair), one
-// keystream block per thread; t = the thread's index in its 192-thread tile group.
-__device__ __forceinline__ void ctr_tile_pair(uint8_t* st, int bytes, uint64_t first_block, const TileSlot* sl,
-                                              const uint32_t* rk, int t) {
-  const int nblk = (bytes + 15) >> 4;
-  const PairLanes lc = pair_lanes();
   for (int i = t; i < nblk; i += kThreads) {
     uint32_t s[4];
     ctr_block(sl->iv_hi, sl->iv_lo, first_block + i, s);
-    aes128_encrypt_pair(s, rk, lc);
+    aes128_encrypt_rep<SH>(s, rk, Tl);
     uint4* p = reinterpret_cast<uint4*>(st + 16 * i);
     uint4 d = *p;
     d.x ^= s[0];
@@ -458,27 +333,16 @@ __device__ __forceinline__ void packed_extent(const TileSlot* sl, bool priv, uin
 // AES-128-CTR over the tile's packed private part (words at w, stream bytes [off, off +
 // bytes), off a multiple of 4): one thread per keystream block the part overlaps; a block
 // that straddles two tiles is generated by both, each XORing its own words
-// SH = 0: the four T-tables at Ts; SH = kTabPair: the pair table (Ts unused); else a
-// replicated T0 as in ctr_tile_rep
-constexpr int kTabPair = -1;
-template <int SH = 0>
-__device__ __forceinline__ void ctr_tile_packed(uint32_t* w, uint64_t off, int bytes, const TileSlot* sl,
-                                                const uint32_t* rk, const uint32_t* Ts, int t) {
+__device__ __forceinline__ void ctr_tile_packed(uint32_t* w, uint64_t off, int bytes, const TileSlot* sl, const uint32_t* rk,
+                                                const uint32_t* Ts, int t) {
   const uint64_t b0 = off >> 4;
   const int nblk = (int)(((off + (uint64_t)bytes + 15) >> 4) - b0);
   const int nw = (bytes + 3) >> 2;
   const int skew = (int)((off & 15) >> 2);
-  const uint32_t Tl = SH > 0 ? smem_u32(Ts) + 4u * (t & ((1 << (SH > 2 ? SH - 2 : 0)) - 1)) : 0u;
-  const PairLanes lc = pair_lanes();
   for (int i = t; i < nblk; i += kThreads) {
     uint32_t s[4];
     ctr_block(sl->iv_hi, sl->iv_lo, b0 + i, s);
-    if constexpr (SH == kTabPair)
-      aes128_encrypt_pair(s, rk, lc);
-    else if constexpr (SH != 0)
-      aes128_encrypt_rep<SH>(s, rk, Tl);
-    else
-      aes128_encrypt(s, rk, Ts);
+    aes128_encrypt(s, rk, Ts);
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       const int wi = 4 * i + m - skew;
