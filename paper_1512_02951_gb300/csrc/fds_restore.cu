@@ -1,32 +1,24 @@
-// Fused restore kernel (defragmentation, Sect. 3.2, Fig. 3; inverse of Sect. 6.3.1) in its tiled
-// form, for packed storage and the tensor-core inverse (int16 storage, batches and the public-image
-// form: fds_restore_warp.cu): CTR decryption of the confidential fragment, merge with the public
-// fragment by zigzag position, inverse 8x8 DCT, round half away from zero (exact), clamp to
+// Restore of one image with the inverse transform on tensor cores, and the dispatch of restore (its
+// float32 forms: fds_restore_warp.cu): CTR decryption of the confidential fragment, merge with the
+// public fragment by zigzag position, inverse 8x8 DCT, round half away from zero (exact), clamp to
 // [0, 255].
 //
 // Persistent CTAs over the image's tiles, b, b + gridDim.x, ..; per tile (see fds_tile.cuh):
 //   A. the tile's fragments are in shared memory, already decrypted; the next tile's start
 //      loading (one bulk copy per fragment range, or cp.async pieces)
-//   1. per channel-block: column then row float32 inverse butterflies (the column pass and
-//      the rounding on pairs with packed f32x2 instructions, bit-identical per lane), round +
-//      clamp, bytes into the interleaved pixel tile; values within the float32 error guard of
-//      a half-integer are queued
+//   1. the coefficients as the MMAs' f16 operand, the accumulators back from TMEM (or, per
+//      channel-block, float32 inverse butterflies, columns then rows); round + clamp, bytes into
+//      the interleaved pixel tile; values within the error guard of a half-integer are queued
 //   B. 2. queued pixels are re-decided exactly (integer coordinates in Z[cos(pi/16)]) by the
 //      last threads while the first ones decrypt the next tile's private range in place
 //      (AES-128-CTR)
 //   C. 3. the pixel tile goes to global memory: one bulk (TMA engine) store per pixel row when
 //      the tile's rows are contiguous and 16-byte aligned, else 8-byte stores.  The pixel tile
 //      is double-buffered so the bulk stores overlap the next tile.
-//
-// Packed storage (PACK = 11 or 8 bits per AC field, Sect. 6.4.3): the tile's part of the two
-// packed streams lands in a separate shared-memory area (bulk copies when 16-byte aligned,
-// else 8-byte cp.async pieces), its private bytes are decrypted there and both parts are
-// unpacked into the int16 staging area, all one tile ahead, before the transform reads it.
 #include "fds_mma.cuh"
 
 namespace fds {
 
-constexpr int kRCtasPerSm = 2;
 constexpr int kSmemCoef = 0;                                 // 2 fragment staging areas
 constexpr int kSmemPix = kSmemCoef + 2 * kCoefBytes;         // 2 pixel tiles
 constexpr int kSmemQueue = kSmemPix + 2 * kPixBytes;
@@ -35,11 +27,6 @@ constexpr int kSlotBytes = (sizeof(TileSlot) + 15) & ~15;
 constexpr int kSmemBar = kSmemSlot + 3 * kSlotBytes;         // 2 mbarriers (staging areas)
 constexpr int kSmemMisc = kSmemBar + 16;
 constexpr int kSmemBytes = kSmemMisc + 32;
-// packed storage: one landing area for a tile's packed public and private parts, 24 (63 w + 11)
-// bytes at most (w = 11) plus 16 for aligning the private part
-constexpr int kLandBytes = 24 * (63 * 11 + 11) + 32;
-constexpr int kSmemLand = kSmemBytes;
-constexpr int kSmemBytesPacked = kSmemLand + kLandBytes;
 // one image in int16 storage: the lane-replicated AES table (32 KB; conflict-free lookups)
 // after the rest (measured: 88.7 -> 86.7 us on 4096 x 4096 at k = 5; the batched form, whose
 // tiles mostly carry little keystream, was slower with it, 2.96 -> 3.11 ms on 2000 images)
@@ -58,132 +45,6 @@ constexpr uint32_t kTcInvIdesc = idesc_f16(192, false);
 // below S 2^-24, and refuses otherwise; 2^-22 covers the roundings of the guard itself)
 constexpr float kTcInvGuardS = 1.0f / 16777216.0f;
 constexpr float kTcInvGuard0 = 1.0f / 4194304.0f;
-
-// ---- packed storage: land, decrypt, unpack one tile
-template <int W>
-__device__ __forceinline__ int land_private_offset(int k) {
-  return ((24 * (63 - k) * W) + 15) & ~15;
-}
-// true if both packed parts of slot sl's tile arrive as one bulk copy each
-template <int W>
-__device__ __forceinline__ bool packed_bulk(const TileSlot* sl) {
-  uint64_t po, vo;
-  int pb, vb;
-  packed_extent<W>(sl, false, po, pb);
-  packed_extent<W>(sl, true, vo, vb);
-  return ((reinterpret_cast<uintptr_t>(sl->pub_in + po) | reinterpret_cast<uintptr_t>(sl->priv_in + vo) |
-           (uintptr_t)pb | (uintptr_t)vb) & 15) == 0;
-}
-// the packed parts of slot sl's tile into the landing area (all threads; thread 0 issues the
-// bulk copies); the streams are 8-byte aligned, so are the tiles' offsets
-template <int W>
-__device__ __forceinline__ void load_packed(const TileSlot* sl, uint8_t* land, uint64_t* bar) {
-  const int t = threadIdx.x;
-  uint64_t po, vo;
-  int pb, vb;
-  packed_extent<W>(sl, false, po, pb);
-  packed_extent<W>(sl, true, vo, vb);
-  const uint8_t* psrc = sl->pub_in + po;
-  const uint8_t* vsrc = sl->priv_in + vo;
-  uint8_t* vdst = land + land_private_offset<W>(sl->k);
-  if (packed_bulk<W>(sl)) {
-    if (t == 0) {
-      mbar_expect_tx(bar, (uint32_t)(pb + vb));
-      if (pb) bulk_load(land, psrc, (uint32_t)pb, bar);
-      if (vb) bulk_load(vdst, vsrc, (uint32_t)vb, bar);
-    }
-    return;
-  }
-  const int p8 = pb >> 3, v8 = vb >> 3;
-  for (int i = t; i < p8 + v8; i += kThreads) {
-    if (i < p8)
-      cp_async8(land + 8 * i, psrc + 8 * i);
-    else
-      cp_async8(vdst + 8 * (i - p8), vsrc + 8 * (i - p8));
-  }
-  if (t < (pb & 7)) land[(pb & ~7) + t] = psrc[(pb & ~7) + t];
-  if (t < (vb & 7)) vdst[(vb & ~7) + t] = vsrc[(vb & ~7) + t];
-  cp_async_commit();
-}
-template <int W>
-__device__ __forceinline__ void wait_packed(const TileSlot* sl, uint64_t* bar, uint32_t& phase, int& lost) {
-  if (packed_bulk<W>(sl)) {
-    if (!mbar_wait(bar, phase)) ++lost;
-    phase ^= 1u;
-  } else {
-    cp_async_wait_all();
-  }
-}
-// AES-128-CTR over the landed private part (all threads; a barrier must follow)
-template <int W>
-__device__ __forceinline__ void decrypt_packed(const TileSlot* sl, uint8_t* land, const uint32_t* rk,
-                                               const uint32_t* Ts) {
-  uint64_t vo;
-  int vb;
-  packed_extent<W>(sl, true, vo, vb);
-  ctr_tile_packed(reinterpret_cast<uint32_t*>(land + land_private_offset<W>(sl->k)), vo, vb, sl, rk, Ts,
-                  (int)threadIdx.x);
-}
-// the landed (decrypted) parts -> int16 staging st, public [cb][63 - k], private [cb][k + 1]
-// (all threads): a public thread unpacks 32 fields (W words), a private thread one
-// channel-block (11 + k W bits)
-template <int W>
-__device__ __forceinline__ void unpack_tile(const TileSlot* sl, const uint8_t* land, uint8_t* st) {
-  const int t = threadIdx.x;
-  const int k = sl->k, nb = sl->nb, npub = 63 - k;
-  const int nf = 3 * nb * npub, ngroups = (nf + 31) >> 5;
-  const uint32_t* pw = reinterpret_cast<const uint32_t*>(land);
-  int16_t* pub16 = reinterpret_cast<int16_t*>(st);
-  for (int g = t; g < ngroups; g += kThreads) {
-    uint32_t word[W];
-#pragma unroll
-    for (int j = 0; j < W; ++j) word[j] = pw[W * g + j];
-    int v[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const int b = W * i;
-      uint32_t c = word[b >> 5] >> (b & 31);
-      if ((b & 31) + W > 32) c |= word[(b >> 5) + 1] << (32 - (b & 31));
-      const int mag = (int)(c & ((1u << (W - 1)) - 1u));
-      v[i] = (c >> (W - 1)) & 1u ? -mag : mag;
-    }
-    const int f0 = 32 * g;
-    if (f0 + 32 <= nf) {
-      uint4* dst = reinterpret_cast<uint4*>(pub16 + f0);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        uint32_t u[4];
-#pragma unroll
-        for (int m = 0; m < 4; ++m)
-          u[m] = ((uint32_t)v[8 * q + 2 * m] & 0xffffu) | ((uint32_t)v[8 * q + 2 * m + 1] << 16);
-        dst[q] = make_uint4(u[0], u[1], u[2], u[3]);
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 32; ++i)
-        if (f0 + i < nf) pub16[f0 + i] = (int16_t)v[i];
-    }
-  }
-  if (t < 3 * nb) {
-    const uint32_t* vw = reinterpret_cast<const uint32_t*>(land + land_private_offset<W>(k));
-    int16_t* dst = reinterpret_cast<int16_t*>(st + kTileCb * 2 * npub) + t * (k + 1);
-    int pos = t * (kDcBits + k * W);
-    for (int z = 0; z <= k; ++z) {
-      const int fw = z == 0 ? kDcBits : W;
-      const int sh = pos & 31;
-      uint32_t c = vw[pos >> 5] >> sh;
-      if (sh + fw > 32) c |= vw[(pos >> 5) + 1] << (32 - sh);
-      c &= (1u << fw) - 1u;
-      if (z == 0) {
-        dst[0] = (int16_t)c;
-      } else {
-        const int mag = (int)(c & ((1u << (W - 1)) - 1u));
-        dst[z] = (int16_t)((c >> (W - 1)) & 1u ? -mag : mag);
-      }
-      pos += fw;
-    }
-  }
-}
 
 // gather the 64 int16 coefficients of tile channel-block cb in zigzag order, two per word
 __device__ __forceinline__ void gather_coefs(const int16_t* pubst, const int16_t* privst, int cb,
@@ -253,20 +114,13 @@ __device__ __forceinline__ void decrypt_fragments(const TileSlot* sl, const uint
   ctr_tile_rep(st + kTileCb * 2 * (63 - k), sl->nb * 6 * (k + 1), first, sl, rk, Trep, (int)threadIdx.x);
 }
 
-// one image (round keys read from the kernel parameters, which AES then takes as constant-bank
-// operands)
-// TC: the inverse transform as tcgen05 MMAs (one image, int16 storage; a.tc_b = the inverse
-// basis table); a tile holding a coefficient of magnitude 2048 or more takes the float32
-// butterflies instead.
-template <int K, int PACK = 0, bool TC = false>
-__global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel(const __grid_constant__ TileArgs a) {
-  static_assert(TC != (PACK != 0), "packed streams, or the tensor-core inverse of int16 storage");
+// The inverse transform as tcgen05 MMAs (one image, int16 storage; a.tc_b = the inverse basis
+// table); a tile holding a coefficient of magnitude 2048 or more takes the float32 butterflies
+// instead.  Round keys are read from the kernel parameters.
+template <int K>
+__global__ void __launch_bounds__(kThreads, 1) restore_tc_kernel(const __grid_constant__ TileArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
-  // AES tables: T0 replicated per lane (one image, int16 storage, private fragment decrypted),
-  // else the four T-tables
-  constexpr bool REP = PACK == 0;
-  __shared__ __align__(16) uint32_t T4[REP ? 4 : 1024];
-  uint32_t* Ts = REP ? reinterpret_cast<uint32_t*>(smem + kSmemTrep) : T4;
+  uint32_t* Ts = reinterpret_cast<uint32_t*>(smem + kSmemTrep);   // T0 replicated per lane
   uint32_t* queue = reinterpret_cast<uint32_t*>(smem + kSmemQueue);
   // misc: [0] queue size, [1] queued total, [2] escalations, [3] failures, [4..5] schedule
   int* misc = reinterpret_cast<int*>(smem + kSmemMisc);
@@ -276,11 +130,7 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
   auto slot = [&](int i) { return reinterpret_cast<TileSlot*>(smem + kSmemSlot + i * kSlotBytes); };
   auto stage = [&](int i) { return smem + kSmemCoef + i * kCoefBytes; };
 
-  if constexpr (REP) {
-    for (int i = t; i < kTrepWords; i += kThreads) Ts[i] = __ldg(a.T + (i >> 5));
-  } else {
-    for (int i = t; i < 1024; i += kThreads) Ts[i] = a.T[i];
-  }
+  for (int i = t; i < kTrepWords; i += kThreads) Ts[i] = __ldg(a.T + (i >> 5));
   if (t < 4) misc[t] = 0;
   if (t == 0) {
     misc[6] = 0;                         // TC: a tensor-core wait gave up
@@ -293,14 +143,13 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
   uint32_t phase[2] = {0u, 0u};
   int lost = 0;
   // TC: operands, MMA barrier, TMEM (kTcCols columns rounded up to 512)
-  uint8_t* const tcbase = TC ? reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem + kSmemBytesRep) + 1023) &
-                                                          ~(uintptr_t)1023)
-                             : nullptr;
+  uint8_t* const tcbase =
+      reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem + kSmemBytesRep) + 1023) & ~(uintptr_t)1023);
   uint8_t* const tA = tcbase;
-  uint8_t* const tB = TC ? tcbase + kTcA : nullptr;
-  uint64_t* const tbar = TC ? reinterpret_cast<uint64_t*>(tcbase + kTcA + kMmaInvBytes) : nullptr;
-  uint32_t* const tslot = TC ? reinterpret_cast<uint32_t*>(tcbase + kTcA + kMmaInvBytes + 8) : nullptr;
-  if constexpr (TC) {
+  uint8_t* const tB = tcbase + kTcA;
+  uint64_t* const tbar = reinterpret_cast<uint64_t*>(tcbase + kTcA + kMmaInvBytes);
+  uint32_t* const tslot = reinterpret_cast<uint32_t*>(tcbase + kTcA + kMmaInvBytes + 8);
+  {
     for (int i = t; i < kMmaInvBytes / 16; i += kThreads) reinterpret_cast<uint4*>(tB)[i] = a.tc_b[i];
     for (int i = t; i < 64 * 128 / 16; i += kThreads)    // A rows 192..255 (never a channel-block)
       reinterpret_cast<uint4*>(tA + 192 * 128)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -310,32 +159,21 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
   if (t == 0) {
     mbar_init(bars);
     mbar_init(bars + 1);
-    if constexpr (TC) mbar_init(tbar);
+    mbar_init(tbar);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  uint8_t* land = smem + kSmemLand;   // PACK only
-  if constexpr (PACK != 0) {
-    load_packed<PACK>(slot(0), land, bars);
-    wait_packed<PACK>(slot(0), bars, phase[0], lost);
-    __syncthreads();
-    decrypt_packed<PACK>(slot(0), land, a.rk, Ts);
-    __syncthreads();
-    unpack_tile<PACK>(slot(0), land, stage(0));
-  } else {
-    load_fragments(slot(0), stage(0), bars);
-    wait_fragments(slot(0), bars, phase[0], lost);
-    __syncthreads();
-    if (!a.plain_private)
-      decrypt_fragments(slot(0), a.rk, stage(0), Ts);
-  }
+  load_fragments(slot(0), stage(0), bars);
+  wait_fragments(slot(0), bars, phase[0], lost);
+  __syncthreads();
+  decrypt_fragments(slot(0), a.rk, stage(0), Ts);
   int esc = 0;
   bool fail = false;
   // a fragment load that did not complete in time leaves its tile's pixels unwritten (the
   // failure counter records it): cur_lost for the tile being transformed, lost counts them all
   int cur_lost = lost;
   uint32_t tmem = 0, tphase = 0;
-  if constexpr (TC) {
+  {
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -356,10 +194,7 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
     __syncthreads();                                                       // A
     if (t == 0) misc[4 + buf] = nxt < ntiles ? (int)(blockIdx.x + (it + 2) * gridDim.x) : ntiles;
     if (nxt < ntiles) {
-      if constexpr (PACK != 0)
-        load_packed<PACK>(slot((it + 1) % 3), land, bars + (buf ^ 1));
-      else
-        load_fragments(slot((it + 1) % 3), stage(buf ^ 1), bars + (buf ^ 1));
+      load_fragments(slot((it + 1) % 3), stage(buf ^ 1), bars + (buf ^ 1));
     }
     const int k = K >= 0 ? K : sl->k;
     const int npub = 63 - k;
@@ -391,7 +226,7 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
       }
     };
     bool tc_done = false;
-    if constexpr (TC) {
+    {
       // A row t: the channel-block's 64 coefficients in zigzag order (the K order of the
       // basis table), as f16 -- exact for |q| < 2048; S = sum |q| sizes the guard
       int S = 0;
@@ -527,10 +362,7 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
     }
     const int lost_before_next = lost;
     if (nxt < ntiles) {
-      if constexpr (PACK != 0)
-        wait_packed<PACK>(slot((it + 1) % 3), bars + (buf ^ 1), phase[buf ^ 1], lost);
-      else
-        wait_fragments(slot((it + 1) % 3), bars + (buf ^ 1), phase[buf ^ 1], lost);
+      wait_fragments(slot((it + 1) % 3), bars + (buf ^ 1), phase[buf ^ 1], lost);
     }
     __syncthreads();                                                       // B
     {
@@ -550,15 +382,7 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
       }
       if (t == 0) misc[1] += misc[0];
     }
-    if constexpr (PACK != 0) {
-      if (nxt < ntiles) {
-        decrypt_packed<PACK>(slot((it + 1) % 3), land, a.rk, Ts);
-        __syncthreads();                                                   // B2
-        unpack_tile<PACK>(slot((it + 1) % 3), land, stage(buf ^ 1));
-      }
-    } else if (nxt < ntiles && !a.plain_private) {
-      decrypt_fragments(slot((it + 1) % 3), a.rk, stage(buf ^ 1), Ts);
-    }
+    if (nxt < ntiles) decrypt_fragments(slot((it + 1) % 3), a.rk, stage(buf ^ 1), Ts);
     fence_proxy_async();                                  // pixel writes before the bulk stores
     const bool skip = __syncthreads_or(cur_lost != 0);                     // C
     cur_lost = lost - lost_before_next;                   // the next tile's fragments
@@ -589,9 +413,9 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
   }
   if (esc) atomicAdd(&misc[2], esc);
   if (fail || lost) atomicAdd(&misc[3], 1);
-  if constexpr (TC) tc_fence_before_sync();
+  tc_fence_before_sync();
   __syncthreads();
-  if constexpr (TC) {
+  {
     tc_fence_after_sync();
     if (t < 32) tmem_dealloc<512>(tmem);
   }
@@ -603,18 +427,14 @@ __global__ void __launch_bounds__(kThreads, TC ? 1 : kRCtasPerSm) restore_kernel
   }
 }
 
-template <int K, int PACK = 0, bool TC = false>
-static cudaError_t launch_k(const TileArgs& a, cudaStream_t s, int sms, int per_sm) {
+template <int K>
+static cudaError_t launch_k(const TileArgs& a, cudaStream_t s, int sms) {
   static bool attr[kMaxAttrDevices];
-  static int resident[kMaxAttrDevices];
-  constexpr int smem = TC ? kSmemBytesTc : (PACK ? kSmemBytesPacked : kSmemBytesRep);
-  cudaError_t e = smem_attr_once(restore_kernel<K, PACK, TC>, smem, attr);
+  cudaError_t e = smem_attr_once(restore_tc_kernel<K>, kSmemBytesTc, attr);
   if (e != cudaSuccess) return e;
   const int ntiles = total_tiles(a);
-  const int r = resident_ctas(restore_kernel<K, PACK, TC>, kThreads, smem, resident);
-  const int cap = (per_sm >= 1 && per_sm < r ? per_sm : r) * sms;
-  const int grid = ntiles < cap ? ntiles : cap;
-  if (grid > 0) restore_kernel<K, PACK, TC><<<grid, kThreads, smem, s>>>(a);
+  const int grid = ntiles < sms ? ntiles : sms;
+  if (grid > 0) restore_tc_kernel<K><<<grid, kThreads, kSmemBytesTc, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -622,22 +442,14 @@ static cudaError_t launch_k(const TileArgs& a, cudaStream_t s, int sms, int per_
 // one CTA per SM (the operands and TMEM take what a second CTA would need)
 cudaError_t launch_restore_tc(const TileArgs& a, cudaStream_t s, int sms) {
   if (a.images || a.k < 0 || a.public_image || a.pack || a.plain_private || !a.tc_b) return cudaErrorInvalidValue;
-  if (a.k == 0) return launch_k<0, 0, true>(a, s, sms, 1);
-  if (a.k == 5) return launch_k<5, 0, true>(a, s, sms, 1);
-  return launch_k<-1, 0, true>(a, s, sms, 1);
+  if (a.k == 0) return launch_k<0>(a, s, sms);
+  if (a.k == 5) return launch_k<5>(a, s, sms);
+  return launch_k<-1>(a, s, sms);
 }
 
-// k is uniform over the launch when a.k >= 0; a.k < 0 (batches of mixed k) reads k per tile;
-// one image in int16 storage, and the public-image form, go to the warp form
+// k is uniform over the launch when a.k >= 0; a.k < 0 (batches of mixed k) reads k per tile
 cudaError_t launch_restore(const TileArgs& a, cudaStream_t s, int sms, int per_sm) {
-  if (a.pack) {   // one image, packed streams in pub_in / priv_in
-    if (a.images || a.k < 0 || a.public_image || (a.pack != 11 && a.pack != 8)) return cudaErrorInvalidValue;
-    if (a.pack == 11) return a.k == 5 ? launch_k<5, 11>(a, s, sms, per_sm)
-                                      : launch_k<-1, 11>(a, s, sms, per_sm);
-    return a.k == 5 ? launch_k<5, 8>(a, s, sms, per_sm) : launch_k<-1, 8>(a, s, sms, per_sm);
-  }
-  if (a.images) return launch_restore_plan(a, s, sms, per_sm);
-  return launch_restore_warp(a, s, sms);
+  return a.images ? launch_restore_plan(a, s, sms, per_sm) : launch_restore_warp(a, s, sms);
 }
 
 }  // namespace fds

@@ -84,7 +84,7 @@ static_assert(sizeof(WarpSlot) == 32, "WarpSlot");
 // int16 coefficients of any value make |n_j| <= 2^22, so the constants carry 40 fraction bits and
 // the error bound is the sum of the |n_j|.
 __device__ __noinline__ int round_far_inv(const int (&n)[9], int* esc, bool* fail) { return exact_round(n, esc, fail); }
-template <bool PUBIMG>
+template <bool PUBIMG, bool STAGED = false>
 __device__ __forceinline__ int round_warp_inv(const int16_t* pub, const int16_t* priv, int k, int pos, const uint4* ctab,
                                               const uint8_t* uv, int lane, WarpSlot* slot) {
   const int y = pos >> 3, x = pos & 7;
@@ -92,7 +92,7 @@ __device__ __forceinline__ int round_warp_inv(const int16_t* pub, const int16_t*
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const int z = 2 * lane + i, t = uv[z], u = t >> 3, v = t & 7;
-    const int q = z <= k ? (PUBIMG ? (z == 0 ? 1024 : 0) : priv[z]) : __ldg(pub + z - k - 1);
+    const int q = z <= k ? (PUBIMG ? (z == 0 ? 1024 : 0) : priv[z]) : (STAGED ? pub[z - k - 1] : __ldg(pub + z - k - 1));
     const int a = u ? (2 * y + 1) * u : 4, b = v ? (2 * x + 1) * v : 4;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -202,8 +202,8 @@ __device__ __forceinline__ void emit_rows(const float2 (&G2)[8][4], float l1, bo
 
 // The marked values of a subtile, one after another, each decided by the whole warp and written
 // by its lane (priv_cb, out: the lane's own; pub_g: the subtile's public coefficients in global
-// memory)
-template <bool PUBIMG>
+// memory, or STAGED in shared memory)
+template <bool PUBIMG, bool STAGED = false>
 __device__ __forceinline__ void decide_pixels(uint32_t mlo, uint32_t mhi, const int16_t* pub_g, const int16_t* priv_cb, int k,
                                               const uint4* ctab, const uint8_t* uv, int lane, WarpSlot* slot, uint8_t* out) {
   // near ties, one after another, decided by the whole warp
@@ -215,7 +215,7 @@ __device__ __forceinline__ void decide_pixels(uint32_t mlo, uint32_t mhi, const 
     if (lane == 0) slot->ties += __popcll(mask);
     for (; mask; mask &= mask - 1) {
       const int pos = __ffsll((long long)mask) - 1;
-      const int p = round_warp_inv<PUBIMG>(pub_s, priv_s, k, pos, ctab, uv, lane, slot);
+      const int p = round_warp_inv<PUBIMG, STAGED>(pub_s, priv_s, k, pos, ctab, uv, lane, slot);
       if (lane == src) out[(pos >> 3) * kRPitch + 3 * (pos & 7)] = (uint8_t)(p < 0 ? 0 : (p > 255 ? 255 : p));
     }
   }
@@ -450,6 +450,279 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
     if (slot->esc) atomicAdd(&a.counters[1], (unsigned long long)slot->esc);
     if (slot->fail || lost) atomicAdd(&a.counters[2], 1ull);
   }
+}
+
+// ---- packed storage (Sect. 6.4.3) ----------------------------------------------------------------
+
+// A subtile's packed parts land as they lie in the streams (4-byte granular: widened to 16-byte
+// boundaries for a bulk copy), the private ones of a run of subtiles at a time, and are unpacked
+// into an int16 staging area, which the transform and the exact decisions read; a landing area is
+// free, and loads again, as soon as it is unpacked.
+constexpr int kUPix = 0;
+constexpr int kUStage = kUPix + 8 * kRPitch;      // int16 coefficients of a subtile
+constexpr int kULand = kUStage + kWCb * 128;      // public landing, private landing
+constexpr int kULandBytes = 3632;
+constexpr int kUBar = kULand + kULandBytes;
+constexpr int kUSlot = kUBar + 16;                // mbarriers: public, private
+constexpr int kUArea = (kUSlot + 32 + 31) & ~31;
+constexpr int kUBelow = ((int)kTpairWin - 1024) / kUArea;
+constexpr int kULow = (int)kTpairWin - kUBelow * kUArea;
+constexpr int kUAbove = kWarps > kUBelow ? kWarps - kUBelow : 0;
+constexpr int kUTail = (int)kTpairWin + kTpairBytes + kUAbove * kUArea;   // folded c(m), (u, v) by zigzag
+constexpr int kUEnd = kUTail + 512 + 64;
+static_assert(kUEnd <= 227 * 1024 && kUSlot % 8 == 0, "packed restore shared memory");
+
+template <int W>
+__host__ __device__ constexpr int land_pub_bytes(int k) { return (4 * (63 - k) * W + 31) & ~15; }   // + 12 of skew
+template <int W>
+__host__ __device__ constexpr int run_tiles_packed(int k) {
+  const int per = 4 * (kDcBits + k * W);
+  int best = 1, bn = per, bp = (per / 16 + 2 + 31) / 32;
+  for (int g = 2; g <= 8 && land_pub_bytes<W>(k) + g * per + 28 <= kULandBytes; ++g) {
+    const int n = g * per, p = (n / 16 + 2 + 31) / 32;
+    if (n * bp > bn * p) {
+      best = g;
+      bn = n;
+      bp = p;
+    }
+  }
+  return best;
+}
+
+// bytes [off, off + bytes) of a stream of `total` bytes (off a multiple of 4, the stream 8-byte
+// aligned) to the 16-byte aligned dst, whose first byte stands for the 16-byte boundary at or below
+// the first one; returns the distance from there.  Where the widened copy would leave the stream,
+// the lanes copy words and bytes.
+__device__ __forceinline__ uint32_t land_stream(uint8_t* dst, const uint8_t* stream, uint64_t total, uint64_t off, int bytes,
+                                                int lane, uint64_t* bar) {
+  const uint8_t* src = stream + off;
+  const uint32_t skew = (uint32_t)(reinterpret_cast<uintptr_t>(src) & 15);
+  const uint32_t wide = (skew + (uint32_t)bytes + 15u) & ~15u;
+  if (off >= skew && off - skew + wide <= total) {
+    if (lane == 0) {
+      mbar_expect_tx(bar, wide);
+      if (wide) bulk_load(dst, src - skew, wide, bar);
+    }
+  } else {
+    for (int i = lane; i < (bytes >> 2); i += 32)
+      reinterpret_cast<uint32_t*>(dst + skew)[i] = __ldg(reinterpret_cast<const uint32_t*>(src) + i);
+    if (lane < (bytes & 3)) dst[skew + (bytes & ~3) + lane] = src[(bytes & ~3) + lane];
+    __syncwarp();
+    if (lane == 0) mbar_expect_tx(bar, 0u);
+  }
+  return skew;
+}
+
+// sign-magnitude code of W bits -> value
+template <int W>
+__device__ __forceinline__ int ac_value(uint32_t c) {
+  const int mag = (int)(c & ((1u << (W - 1)) - 1u));
+  return (c >> (W - 1)) & 1u ? -mag : mag;
+}
+
+// n channel-blocks' packed public fields (words at w) -> int16 at pub, 32 fields (W words) a lane
+// and round
+template <int W>
+__device__ __forceinline__ void unpack_public(const uint32_t* w, int16_t* pub, int n, int npub, int lane) {
+  const int ngroups = (n * npub + 31) >> 5;
+#pragma unroll 1
+  for (int g = lane; g < ngroups; g += 32) {
+    uint32_t word[W];
+#pragma unroll
+    for (int j = 0; j < W; ++j) word[j] = w[W * g + j];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      uint32_t u[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        uint32_t v[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int b = W * (8 * q + 2 * m + h);
+          const uint32_t c = (b & 31) + W > 32 ? __funnelshift_r(word[b >> 5], word[(b >> 5) + 1], b & 31) : word[b >> 5] >> (b & 31);
+          v[h] = (uint32_t)ac_value<W>(c);
+        }
+        u[m] = __byte_perm(v[0], v[1], 0x5410u);
+      }
+      reinterpret_cast<uint4*>(pub + 32 * g)[q] = make_uint4(u[0], u[1], u[2], u[3]);   // past the last field: not read
+    }
+  }
+}
+
+// a lane's channel-block cb of a landed private run (words at w) -> its k + 1 int16 at dst
+template <int W>
+__device__ __forceinline__ void unpack_private(const uint32_t* w, int16_t* dst, int cb, int k) {
+  int pos = cb * (kDcBits + k * W);
+  dst[0] = (int16_t)(__funnelshift_r(w[pos >> 5], w[(pos >> 5) + 1], pos & 31) & ((1u << kDcBits) - 1u));
+  pos += kDcBits;
+#pragma unroll 1
+  for (int z = 1; z <= k; ++z, pos += W)
+    dst[z] = (int16_t)ac_value<W>(__funnelshift_r(w[pos >> 5], w[(pos >> 5) + 1], pos & 31));
+}
+
+template <int K, int W>
+__global__ void __launch_bounds__(kWarps * 32, 1) restore_packed_kernel(const __grid_constant__ TileArgs a) {
+  extern __shared__ __align__(128) uint8_t smem_cta[];
+  const uint32_t win0 = smem_u32(smem_cta);
+  if (win0 > (uint32_t)kULow) {   // see the launcher
+    if (threadIdx.x == 0 && a.counters) atomicAdd(&a.counters[2], 1ull);
+    return;
+  }
+  const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+  uint8_t* area = smem_cta + ((warp < kUBelow ? (uint32_t)(kULow + warp * kUArea)
+                                              : kTpairWin + kTpairBytes + (uint32_t)(warp - kUBelow) * kUArea) -
+                              win0);
+  uint8_t* const pix = area + kUPix;
+  uint64_t* const bars = reinterpret_cast<uint64_t*>(area + kUBar);
+  WarpSlot* const slot = reinterpret_cast<WarpSlot*>(area + kUSlot);
+  uint4* const ctab = reinterpret_cast<uint4*>(smem_cta + (kUTail - win0));
+  uint8_t* const uv = reinterpret_cast<uint8_t*>(ctab + 32);
+  const int k = K >= 0 ? K : a.k;
+  const int npub = 63 - k, period = kDcBits + k * W;
+  const uint32_t pub_per = 4u * (uint32_t)(npub * W), priv_per = 4u * (uint32_t)period;
+  const int G = K >= 0 ? run_tiles_packed<W>(K >= 0 ? K : 0) : a.aes_pair;
+  uint8_t* const land_pub = area + kULand;
+  uint8_t* const land_priv = land_pub + land_pub_bytes<W>(k);
+  int16_t* const pubst = reinterpret_cast<int16_t*>(area + kUStage);
+  int16_t* const privst = pubst + kWCb * npub;
+  const uint32_t ncb = 3u * (uint32_t)a.nblocks, nsub = (ncb + 31u) >> 5;
+  const uint64_t pub_total = ((uint64_t)ncb * (uint32_t)(npub * W) + 7) >> 3, priv_total = ((uint64_t)ncb * (uint32_t)period + 7) >> 3;
+  const int act = a.groups;       // working warps of each CTA, each with a run of the subtiles
+  const uint32_t id = blockIdx.x * act + warp, nw = gridDim.x * act;
+  const uint32_t t0 = warp < act ? (uint32_t)((uint64_t)nsub * id / nw) : 0u;
+  const uint32_t t1 = warp < act ? (uint32_t)((uint64_t)nsub * (id + 1) / nw) : 0u;
+  auto nof = [&](uint32_t t) { return (int)min(32u, ncb - 32u * t); };
+  auto load_pub = [&](uint32_t t) {
+    return land_stream(land_pub, reinterpret_cast<const uint8_t*>(a.pub_in), pub_total, (uint64_t)t * pub_per,
+                       (nof(t) * npub * W + 7) >> 3, lane, bars);
+  };
+  auto load_priv = [&](uint32_t t) {
+    const int cnt = min(G, (int)(t1 - t));
+    return land_stream(land_priv, a.priv_in, priv_total, (uint64_t)t * priv_per,
+                       (cnt - 1) * (int)priv_per + ((nof(t + cnt - 1) * period + 7) >> 3), lane, bars + 1);
+  };
+
+  if (lane == 0) {
+    mbar_init(bars);
+    mbar_init(bars + 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    slot->ties = slot->esc = slot->fail = 0;
+  }
+  __syncwarp();
+  uint32_t skew_pub = 0, skew_priv = 0;
+  if (t0 < t1) {
+    skew_pub = load_pub(t0);
+    skew_priv = load_priv(t0);
+  }
+  if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
+    const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
+    const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
+    ctab[lane] = make_uint4(f >> 1 == 0 ? one : 0u, f >> 1 == 1 ? one : 0u, f >> 1 == 2 ? one : 0u, f >> 1 == 3 ? one : 0u);
+  }
+  if (threadIdx.x < 64) uv[zigzag_of((int)threadIdx.x >> 3, (int)threadIdx.x & 7)] = (uint8_t)threadIdx.x;
+  fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
+  __syncthreads();
+
+  bool lost = false;
+  uint32_t ph = 0, run = t0;               // phases: bit 0 public, bit 1 private; the run's first subtile
+#pragma unroll 1
+  for (uint32_t t = t0; t < t1; ++t) {
+    const int n = nof(t);
+    if (t == run) {                        // a new run: decrypt its private parts where they landed
+      if (!__all_sync(0xffffffffu, mbar_wait(bars + 1, ph >> 1))) {
+        lost = true;
+        break;
+      }
+      ph ^= 2u;
+      __syncwarp();
+      const int cnt = min(G, (int)(t1 - t));
+      const uint64_t off = (uint64_t)t * priv_per;
+      const int nblk = (int)((skew_priv + (cnt - 1) * priv_per + (uint32_t)((nof(t + cnt - 1) * period + 7) >> 3) + 15) >> 4);
+      const PairLanes lc = pair_lanes();
+#pragma unroll 1
+      for (int i = lane; i < nblk; i += 32) {
+        uint32_t ks[4];
+        ctr_block(a.iv_hi, a.iv_lo, (off >> 4) + i, ks);
+        aes128_encrypt_pair(ks, a.rk, lc);
+        uint4* p = reinterpret_cast<uint4*>(land_priv + 16 * i);
+        uint4 d = *p;
+        d.x ^= ks[0];
+        d.y ^= ks[1];
+        d.z ^= ks[2];
+        d.w ^= ks[3];
+        *p = d;
+      }
+      __syncwarp();
+    }
+    if (!__all_sync(0xffffffffu, mbar_wait(bars, ph & 1u))) {   // gave up: nothing more is written
+      lost = true;
+      break;
+    }
+    ph ^= 1u;
+    __syncwarp();
+    unpack_public<W>(reinterpret_cast<const uint32_t*>(land_pub + skew_pub), pubst, n, npub, lane);
+    unpack_private<W>(reinterpret_cast<const uint32_t*>(land_priv + skew_priv), privst + lane * (k + 1),
+                      (int)(t - run) * kWCb + (lane < n ? lane : 0), k);
+    if (t + 1 < t1) {
+      const bool last = t + 1 - run == (uint32_t)G;   // of the run: the next one's private parts load too
+      if (last) fence_proxy_async();       // the landing area was decrypted in place
+      __syncwarp();                        // unpacked: the landing areas are free
+      skew_pub = load_pub(t + 1);
+      if (last) {
+        run = t + 1;
+        skew_priv = load_priv(run);
+      }
+    } else {
+      __syncwarp();
+    }
+    const CbPos at = cb_pos(a, 32u * t + lane);
+    const int16_t* pub_cb = pubst + lane * npub;
+    const int16_t* priv_cb = privst + lane * (k + 1);
+    float2 G2[8][4];
+    const float l1 = gather_columns<false>(pub_cb, priv_cb, k, G2);
+    const uint32_t c0 = __shfl_sync(0xffffffffu, at.c, 0);
+    uint8_t* const out = pix + 8 * (c0 + lane - at.c) + at.c;
+    uint32_t mlo, mhi;
+    emit_rows(G2, l1, lane < n, out, mlo, mhi);
+    decide_pixels<false, true>(mlo, mhi, pubst, priv_cb, k, ctab, uv, lane, slot, out);
+    __syncwarp();                          // the pixel rows are complete
+    store_pixels(a.pixels_out, 3ull * (uint64_t)a.width, at, c0, n, lane, pix);
+    __syncwarp();                          // the staging area and the pixel buffer may be written again
+  }
+  if (lost) {                              // copies still in flight
+    mbar_wait(bars, ph & 1u);
+    mbar_wait(bars + 1, ph >> 1);
+  }
+  if (lane == 0 && a.counters) {
+    if (slot->ties) atomicAdd(&a.counters[0], (unsigned long long)slot->ties);
+    if (slot->esc) atomicAdd(&a.counters[1], (unsigned long long)slot->esc);
+    if (slot->fail || lost) atomicAdd(&a.counters[2], 1ull);
+  }
+}
+
+template <int K, int W>
+static cudaError_t launch_packed(const TileArgs& a, cudaStream_t s, int sms) {
+  static bool attr[kMaxAttrDevices];
+  static bool window_ok[kMaxAttrDevices];
+  int dev = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxAttrDevices) return cudaErrorInvalidDevice;
+  if (!window_ok[dev]) {
+    if ((e = smem_window_start_ok(restore_packed_kernel<K, W>, (uint32_t)kULow)) != cudaSuccess) return e;
+    window_ok[dev] = true;
+  }
+  e = smem_attr_once(restore_packed_kernel<K, W>, kUEnd, attr);
+  if (e != cudaSuccess) return e;
+  TileArgs b = a;
+  const long long nsub = (3ll * a.nblocks + 31) / 32;
+  const int grid = (int)(nsub < sms ? nsub : sms);
+  const long long per = (nsub + grid - 1) / (grid ? grid : 1);
+  b.groups = (int)(per < kWarps ? per : kWarps);
+  bx_division(b);
+  b.aes_pair = run_tiles_packed<W>(a.k);
+  if (grid > 0) restore_packed_kernel<K, W><<<grid, kWarps * 32, kUEnd, s>>>(b);
+  return cudaGetLastError();
 }
 
 // ---- batches ---------------------------------------------------------------------------------
@@ -687,7 +960,13 @@ cudaError_t launch_restore_plan(const TileArgs& a, cudaStream_t s, int sms, int 
 }
 
 cudaError_t launch_restore_warp(const TileArgs& a, cudaStream_t s, int sms) {
-  if (a.images || a.pack || a.k < 0 || a.k > 63) return cudaErrorInvalidValue;
+  if (a.images || a.k < 0 || a.k > 63) return cudaErrorInvalidValue;
+  if (a.pack) {
+    if (a.public_image || a.plain_private) return cudaErrorInvalidValue;
+    if (a.pack == 11) return a.k == 5 ? launch_packed<5, 11>(a, s, sms) : launch_packed<-1, 11>(a, s, sms);
+    if (a.pack == 8) return a.k == 5 ? launch_packed<5, 8>(a, s, sms) : launch_packed<-1, 8>(a, s, sms);
+    return cudaErrorInvalidValue;
+  }
   if (a.public_image) return a.k == 5 ? launch_w<5, true>(a, s, sms) : launch_w<-1, true>(a, s, sms);
   if (a.k == 0) return launch_w<0, false>(a, s, sms);
   if (a.k == 5) return launch_w<5, false>(a, s, sms);

@@ -127,8 +127,8 @@ struct TileSlot {
 };
 
 // launchers (one translation unit each); `sms` = number of SMs of the device; `per_sm` counts
-// quarters (protect of a batch, 1 .. 4) or halves (its restore, 1 .. 2) of a CTA's sixteen warps,
-// or CTAs (packed restore, 1 .. 2); 0 = all
+// quarters (protect of a batch, 1 .. 4) or halves (its restore, 1 .. 2) of a CTA's sixteen warps;
+// 0 = all
 cudaError_t launch_protect(const TileArgs& a, cudaStream_t s, bool debug, int sms, int per_sm = 0);
 cudaError_t launch_restore(const TileArgs& a, cudaStream_t s, int sms, int per_sm = 0);
 // protect of one image (int16 or packed storage), one subtile of 32 channel-blocks per warp
@@ -159,20 +159,6 @@ inline cudaError_t smem_attr_once(Kernel kernel, int bytes, bool (&done)[kMaxAtt
     done[dev] = true;
   }
   return cudaSuccess;
-}
-
-// Resident CTAs per SM of `kernel` at `threads` threads and `bytes` dynamic shared memory on
-// the current device (at least 1), cached per device in `cache` (0 = not yet asked)
-template <typename Kernel>
-inline int resident_ctas(Kernel kernel, int threads, int bytes, int (&cache)[kMaxAttrDevices]) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxAttrDevices) return 1;
-  if (!cache[dev]) {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, bytes) != cudaSuccess || n < 1) n = 1;
-    cache[dev] = n;
-  }
-  return cache[dev];
 }
 
 inline int total_tiles(const TileArgs& a) {
@@ -316,40 +302,7 @@ __device__ __forceinline__ void ctr_tile_rep(uint8_t* st, int bytes, uint64_t fi
   }
 }
 
-// ---- packed storage (Sect. 6.4.3): a full tile's 192 channel-blocks are a multiple of 8,
-// so its part of either bit stream starts on a byte boundary
-constexpr int kDcBits = 11;
-
-// bytes of a tile's packed public / private part and their offsets in the image's streams
-// (a full tile: 24 (63 - k) W and 24 (11 + k W) bytes)
-template <int W>
-__device__ __forceinline__ void packed_extent(const TileSlot* sl, bool priv, uint64_t& off, int& bytes) {
-  const int k = sl->k;
-  const int per_cb = priv ? kDcBits + k * W : (63 - k) * W;   // bits per channel-block
-  off = (uint64_t)sl->local * 24ull * (uint64_t)per_cb;
-  bytes = (3 * sl->nb * per_cb + 7) >> 3;
-}
-
-// AES-128-CTR over the tile's packed private part (words at w, stream bytes [off, off +
-// bytes), off a multiple of 4): one thread per keystream block the part overlaps; a block
-// that straddles two tiles is generated by both, each XORing its own words
-__device__ __forceinline__ void ctr_tile_packed(uint32_t* w, uint64_t off, int bytes, const TileSlot* sl, const uint32_t* rk,
-                                                const uint32_t* Ts, int t) {
-  const uint64_t b0 = off >> 4;
-  const int nblk = (int)(((off + (uint64_t)bytes + 15) >> 4) - b0);
-  const int nw = (bytes + 3) >> 2;
-  const int skew = (int)((off & 15) >> 2);
-  for (int i = t; i < nblk; i += kThreads) {
-    uint32_t s[4];
-    ctr_block(sl->iv_hi, sl->iv_lo, b0 + i, s);
-    aes128_encrypt(s, rk, Ts);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const int wi = 4 * i + m - skew;
-      if (wi >= 0 && wi < nw) w[wi] ^= s[m];
-    }
-  }
-}
+constexpr int kDcBits = 11;   // packed storage (Sect. 6.4.3): bits of the DC field
 
 // Exact integer coordinates of 8 F[u][v] (pos = 8u+v) of channel c of tile block b:
 // n[j] = sum over the 64 pixels of pixel * K_j, with the signed-byte weights K_j of
