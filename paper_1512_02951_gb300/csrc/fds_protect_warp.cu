@@ -767,7 +767,17 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     slots[0].image = slots[1].image = ~0u;
   }
-  if (threadIdx.x == 0) *next = 0;
+  if (threadIdx.x == 0) *next = (uint32_t)act;
+  __syncthreads();                         // a first claim may go on to the counter
+  int esc = 0, nties = 0;
+  bool fail = false, lost = false, bulk = false;
+  uint32_t phase = 0, t = 0, end = 0, tn, endn;
+  PlanSlot *s = slots, *sn = slots + 1;
+  PixAt at{};
+  if (warp < act) {                        // the first run starts loading before the tables are filled
+    claim(a, act, next, s, s, c_acc.n, warp, lane, t, end);
+    if (t < end) at = load(s, t, bulk);
+  }
   if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
     const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
     const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
@@ -777,13 +787,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
   __syncthreads();
   if (warp >= act) return;
 
-  int esc = 0, nties = 0;
-  bool fail = false, lost = false, bulk = false;
-  uint32_t phase = 0, t, end, tn, endn;
-  PlanSlot *s = slots, *sn = slots + 1;
-  PixAt at{};
-  claim(a, act, next, s, s, c_acc.n, warp, lane, t, end);
-  if (t < end) at = load(s, t, bulk);
   while (t < end && !lost) {
     claim(a, act, next, sn, s, c_acc.n, warp, lane, tn, endn);
     const int k = K >= 0 ? K : s->k, npub = 63 - k;

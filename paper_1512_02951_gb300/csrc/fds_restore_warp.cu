@@ -794,7 +794,20 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
     slots[0].image = slots[1].image = ~0u;
     slot->ties = slot->esc = slot->fail = 0;
   }
-  if (threadIdx.x == 0) *next = 0;
+  if (threadIdx.x == 0) *next = (uint32_t)act;
+  __syncthreads();                         // a first claim may go on to the counter
+  bool lost = false;
+  uint32_t ph = 0;                         // phases: bit 0 public, bits 1 and 2 the private buffers
+  PlanSlot *s = slots, *sx = slots + 1;    // the run's image; the other slot
+  uint32_t r = 0, end = 0;                 // the run's first subtile, the end of what was claimed
+  int half = 0;
+  if (warp < act) {                        // the first run starts loading before the tables are filled
+    claim(a, act, next, s, s, c_run.n, warp, lane, r, end);
+    if (r < end) {
+      load_priv(s, r, min(s->acc & 15, (int)(end - r)), 0);
+      load_pub(s, r);
+    }
+  }
   if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
     const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
     const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
@@ -805,16 +818,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
   __syncthreads();
   if (warp >= act) return;
 
-  bool lost = false;
-  uint32_t ph = 0;                         // phases: bit 0 public, bits 1 and 2 the private buffers
-  PlanSlot *s = slots, *sx = slots + 1;    // the run's image; the other slot
-  uint32_t r, end;                         // the run's first subtile, the end of what was claimed
-  int half = 0;
-  claim(a, act, next, s, s, c_run.n, warp, lane, r, end);
-  if (r < end) {
-    load_priv(s, r, min(s->acc & 15, (int)(end - r)), 0);
-    load_pub(s, r);
-  }
   while (r < end && !lost) {
     const int k = K >= 0 ? K : s->k, npub = 63 - k;
     const int G = s->acc & 15, cnt = min(G, (int)(end - r));

@@ -154,51 +154,63 @@ __device__ __forceinline__ int plan_slot(const TileArgs& a, int g, PlanSlot* s, 
 }
 
 // The next run of subtiles of one image for a warp: [t, end), none left where t == end.  A CTA's
-// tiles are [g0, g1), taken by its warps one by one from `next`, the last ones (from g0 + whole on)
-// subtile by subtile; or (a.dispenser) every warp takes tiles from one counter.
+// tiles are [g0, g1).  As many as give every warp the same number of whole tiles are handed out
+// whole, the last 2 act subtiles or so one by one, those between in halves, so that the CTA's warps
+// end together: with all but the last whole, 12 tiles a CTA left warps idle for a whole tile (30
+// images of mixed k, protect 56.0 -> 49.3 us, restore 61.8 -> 56.5).  A warp's first run is its own,
+// so that it starts loading before the CTA's tables are filled; the others come from `next`, which
+// starts at act and is set before any claim (a first run may be an empty one).  Or (a.dispenser)
+// every warp takes tiles from one counter.
 struct PlanClaim {
-  int g0, g1, whole;
+  int g0, g1, whole, halves;
   bool first;
 
   __device__ __forceinline__ PlanClaim(const TileArgs& a, int act) {
     g0 = (int)((int64_t)a.total_tiles * blockIdx.x / gridDim.x);
     g1 = (int)((int64_t)a.total_tiles * (blockIdx.x + 1) / gridDim.x);
-    whole = g1 - g0 - min(g1 - g0, (2 * act + kTileSubs - 1) / kTileSubs);
+    const int rest = max(0, g1 - g0 - (2 * act + kTileSubs - 1) / kTileSubs);
+    whole = rest / act * act;
+    halves = rest - whole;
     first = true;
   }
   __device__ __forceinline__ void operator()(const TileArgs& a, int act, uint32_t* next, PlanSlot* s, const PlanSlot* hint,
                                              const uint8_t* acc_of, int warp, int lane, uint32_t& t, uint32_t& end) {
     for (;;) {
       uint32_t u = 0;
-      if (lane == 0) {
-        if (a.dispenser == nullptr)
+      if (a.dispenser == nullptr) {
+        if (first)
+          u = (uint32_t)warp;
+        else if (lane == 0)
           u = atomicAdd(next, 1u);
-        else if (first)
-          u = blockIdx.x * act + warp;
-        else
-          u = atomicAdd(a.dispenser, 1u) + gridDim.x * act;
+      } else if (first) {
+        u = blockIdx.x * act + warp;
+      } else if (lane == 0) {
+        u = atomicAdd(a.dispenser, 1u) + gridDim.x * act;
       }
       u = __shfl_sync(0xffffffffu, u, 0);
       first = false;
-      int g, sub = -1;
+      int g = (int)u, sub = 0, len = kTileSubs;
       if (a.dispenser != nullptr) {
         if (u >= (uint32_t)a.total_tiles) break;
-        g = (int)u;
       } else {
-        const int v = (int)u - whole;
-        g = g0 + (v < 0 ? (int)u : whole + v / kTileSubs);
-        if (v >= 0) sub = v % kTileSubs;
+        int v = (int)u - whole;
+        if (v >= 2 * halves) {
+          v -= 2 * halves;
+          g = whole + halves + v / kTileSubs;
+          sub = v % kTileSubs;
+          len = 1;
+        } else if (v >= 0) {
+          g = whole + (v >> 1);
+          len = kTileSubs / 2;
+          sub = v & 1 ? len : 0;
+        }
+        g += g0;
         if (g >= g1) break;
       }
       const int local = plan_slot(a, g, s, hint, acc_of, lane);
-      t = (uint32_t)local * kTileSubs;
-      end = min(t + kTileSubs, (s->ncb + 31u) >> 5);
-      if (sub < 0) return;
-      t += sub;
-      if (t < end) {
-        end = t + 1;
-        return;
-      }
+      t = (uint32_t)(local * kTileSubs + sub);
+      end = min(t + len, (s->ncb + 31u) >> 5);
+      if (t < end) return;
     }
     t = end = 0;
   }
