@@ -926,7 +926,7 @@ static cudaError_t launch_w(const TileArgs& a, cudaStream_t s, int sms) {
   const long long nsub = (3ll * a.nblocks + 31) / 32;
   const int grid = (int)(nsub < sms ? nsub : sms);
   const long long per = (nsub + grid - 1) / (grid ? grid : 1);
-  b.groups = (int)(per < kWarps ? per : kWarps);
+  b.groups = working_warps(per);
   bx_division(b);
   b.aes_pair = run_tiles(a.k) | (run_twice(a.k) ? 16 : 0);
   if (grid > 0) restore_warp_kernel<K, PUBIMG><<<grid, kWarps * 32, kREnd, s>>>(b);

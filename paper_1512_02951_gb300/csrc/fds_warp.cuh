@@ -26,6 +26,14 @@ __device__ __forceinline__ CbPos cb_pos(const TileArgs& a, uint32_t cb) {
   return p;
 }
 
+// Working warps of a CTA for `per` subtiles an SM.  Up to three warps on a scheduler a round takes
+// the latency of one subtile, the fourth makes it longer; so two rounds of twelve take less than
+// one of sixteen and a short one (restore of 4096 x 512, k = 5, 20 subtiles an SM: 18.4 -> 17.6 us)
+inline int working_warps(long long per) {
+  if (per > kWarps && per <= 24) return 12;
+  return (int)(per < kWarps ? per : kWarps);
+}
+
 // block / bx_count as a multiply and a shift, exact for block numbers below 2^31: with l the
 // smallest integer such that bx_count <= 2^l, the multiplier is off by less than 2^l / bx_count
 inline void bx_division(TileArgs& a) {
