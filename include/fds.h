@@ -138,19 +138,18 @@ int fds_plan_reserve(int32_t capacity, fds_plan** plan_out);
  * after it).  Waits only for the previous update's copy to have left the staging area. */
 int fds_plan_update(fds_plan* plan, const fds_image* images, int32_t n, void* stream);
 
-/* The most a plan's schedule may launch per SM: protect runs one CTA per SM holding up to
- * four independent tile groups of 192 threads (its "ctas_per_sm" counts those groups; one
- * image outside a plan runs three, which share one AES table); restore runs up to two CTAs
- * of 192 threads per SM. */
+/* The most a plan's schedule may ask for per SM.  Both directions run one CTA of sixteen warps
+ * per SM, each warp on tiles of its own; "ctas_per_sm" counts the working warps in quarters
+ * (protect) or halves (restore) of the sixteen. */
 #define FDS_PROTECT_MAX_CTAS_PER_SM 4
 #define FDS_RESTORE_MAX_CTAS_PER_SM 2
 
-/* Schedule of the persistent launches, both directions at once.  ctas_per_sm: tile groups
- * (protect) or CTAs (restore) per SM, 0 = the most (protect 4, restore 2), 1 .. 4 (restore
- * takes values above 2 as 0); dynamic: 0 = static round-robin tile assignment, 1 = tiles handed
- * out by an atomic counter; largest_first: 0 = tiles in descriptor order, 1 = images by
- * decreasing size (shared by the directions).  The lane schedule of both directions goes
- * back to one keystream block per thread.  Re-uploads the tile order when it changes and
+/* Schedule of the persistent launches, both directions at once.  ctas_per_sm as above, 0 = the
+ * most (protect 4, restore 2), 1 .. 4 (restore takes values above 2 as 0); dynamic: 0 = a run of
+ * the batch's tiles for each CTA, handed out among its warps, 1 = tiles handed out to every warp
+ * by one atomic counter; largest_first: 0 = tiles in descriptor order, 1 = images by
+ * decreasing size (shared by the directions).  aes_pair of both directions goes
+ * back to 0.  Re-uploads the tile order when it changes and
  * drops captured graphs.  FDS_E_INVALID for ctas_per_sm outside 0 .. 4. */
 int fds_plan_set_schedule(fds_plan* plan, int32_t ctas_per_sm, int32_t dynamic,
                           int32_t largest_first);
@@ -161,10 +160,9 @@ int fds_plan_get_schedule(const fds_plan* plan, int32_t* ctas_per_sm, int32_t* d
                           int32_t* largest_first);
 
 /* Schedule of one direction (0 = protect, 1 = restore): ctas_per_sm 0 .. the direction's
- * FDS_*_MAX_CTAS_PER_SM, dynamic as above, aes_pair: 0 = each thread of a CTA encrypts one
- * 16-byte keystream block of the tile at a time, 1 = two blocks with their AES rounds
- * interleaved (fewer threads, more independent lookups each; it pays only where a tile has
- * more keystream blocks than a CTA has threads, k > 7).  Drops captured graphs.
+ * FDS_*_MAX_CTAS_PER_SM, dynamic as above, aes_pair: 0 or 1, kept
+ * and reported for stored schedules (the kernels have one lane schedule: a keystream block per
+ * lane).  Drops captured graphs.
  * FDS_E_INVALID for a bad direction or value. */
 int fds_plan_set_direction_schedule(fds_plan* plan, int32_t direction, int32_t ctas_per_sm,
                                     int32_t dynamic, int32_t aes_pair);

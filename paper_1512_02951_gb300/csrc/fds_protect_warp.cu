@@ -725,8 +725,9 @@ constexpr AccTable make_acc_table() {
 static __constant__ AccTable c_acc = make_acc_table();
 
 // Protect of a batch: every tile of 64 blocks of every image, six subtiles a tile.  A CTA has a
-// run of the batch's tiles, taken by its warps one by one, the last few subtile by subtile; or
-// (a.dispenser) every warp takes tiles from one counter.
+// run of the batch's tiles, taken by its warps as PlanClaim says; or (a.dispenser) every warp takes
+// tiles from one counter.  Bound by issue, as one image: 1000 images (2.97 GB in and out), k = 0,
+// 1210 -> 797 us (24 warps of 80 registers per SM, which spilled and met at three barriers a tile, before).
 template <int K>
 __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __grid_constant__ TileArgs a) {
   extern __shared__ __align__(128) uint8_t smem_cta[];

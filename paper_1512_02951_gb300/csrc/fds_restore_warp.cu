@@ -1,6 +1,7 @@
 // Fused restore kernel in its warp form (defragmentation, Sect. 3.2, Fig. 3): CTR decryption of
 // the confidential fragment, merge by zigzag position, inverse 8x8 DCT, round half away from zero
-// (exact), clamp to [0, 255], of one image; and the public-image form (Sect. 6.5.1).
+// (exact), clamp to [0, 255], of one image, of packed fragments and of a batch; and the public-image
+// form (Sect. 6.5.1).
 //
 // As in the warp form of protect, each warp works on subtiles of 32 channel-blocks of its own,
 // with no barrier between warps after the AES table is filled.  It is bound by the issue of
@@ -457,7 +458,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
 // A subtile's packed parts land as they lie in the streams (4-byte granular: widened to 16-byte
 // boundaries for a bulk copy), the private ones of a run of subtiles at a time, and are unpacked
 // into an int16 staging area, which the transform and the exact decisions read; a landing area is
-// free, and loads again, as soon as it is unpacked.
+// free, and loads again, as soon as it is unpacked.  Bound by issue: 4096 x 4096, k = 5,
+// 104 -> 76 us (11 and 8 bits).
 constexpr int kUPix = 0;
 constexpr int kUStage = kUPix + 8 * kRPitch;      // int16 coefficients of a subtile
 constexpr int kULand = kUStage + kWCb * 128;      // public landing, private landing
@@ -751,7 +753,8 @@ static __constant__ RunTable c_run = make_run_table();
 
 // Restore of a batch (the tiles as in protect_plan_kernel).  Where the next run is of an image
 // with another k, its parts lie elsewhere in the buffers and are loaded only when the run before
-// is done.
+// is done.  Bound by issue, as one image: 300 images (742 MB in and out), k = 5, 445 -> 306 us (two
+// CTAs per SM, a tile of six warps each, before).
 template <int K>
 __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __grid_constant__ TileArgs a) {
   extern __shared__ __align__(128) uint8_t smem_cta[];
