@@ -19,7 +19,10 @@ from . import _lib
 
 
 def _stream_ptr(device: torch.device) -> int:
-    # the current stream's handle without a Stream object around it
+    # the current stream's handle without a Stream object around it; host tensors are refused here,
+    # as torch.cuda.current_stream refuses their device: the library would take their addresses
+    if device.type != "cuda":
+        raise ValueError(f"expected a CUDA tensor, but got one on {device}")
     i = device.index
     return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if i is None else i)
 
