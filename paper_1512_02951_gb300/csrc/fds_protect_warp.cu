@@ -573,8 +573,13 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
   }
   __syncwarp();
   PixAt at{};
-  uint32_t phase = 0;
-  if (t < tend) at = load_subtile<BULK>(a.pixels_in, pitch, (uint32_t)a.bx_count, cb_pos(a, 32u * t + lane), min(32u, ncb - 32u * t), lane, pix, bar);
+  Loads ld;
+  auto load = [&](uint32_t s) {
+    at = load_subtile<BULK>(a.pixels_in, pitch, (uint32_t)a.bx_count, cb_pos(a, 32u * s + lane), min(32u, ncb - 32u * s), lane,
+                            pix, bar);
+    if (BULK) ld.issued(0);
+  };
+  if (t < tend) load(t);
   if (threadIdx.x == 0) *next = s0 + act;
   if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
     const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
@@ -597,7 +602,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
   constexpr int kG = K >= 0 ? acc_tiles(K >= 0 ? K : 0) : 0;
   const int G = K >= 0 ? kG : a.aes_pair;           // subtiles between two AES phases
   int esc = 0, nties = 0;
-  bool fail = false;
+  bool fail = false, lost = false;         // exact_round failed; a load did not arrive in time
   int acc = 0;
   int16_t* const pubst = reinterpret_cast<int16_t*>(stage);
   uint8_t* const privst = stage + kWCb * 2 * npub;
@@ -610,11 +615,10 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
     }
     const uint32_t n = min(32u, ncb - 32u * t);
     if constexpr (BULK) {
-      if (!__all_sync(0xffffffffu, mbar_wait(bar, phase))) {   // gave up: nothing more is written
-        fail = true;
+      if (!load_wait(ld, bar, 0)) {        // gave up: nothing more is written
+        lost = true;
         break;
       }
-      phase ^= 1u;
     } else {
       cp_async_wait_all();
       __syncwarp();
@@ -625,7 +629,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
     float2 P[8][4];
     const float V = transform_rows(px_even, px_odd, c, P);
     __syncwarp();                          // the pixel buffer is read: the next subtile's load starts
-    if (tn < tend) at = load_subtile<BULK>(a.pixels_in, pitch, (uint32_t)a.bx_count, cb_pos(a, 32u * tn + lane), min(32u, ncb - 32u * tn), lane, pix, bar);
+    if (tn < tend) load(tn);
     bulk_wait_read_all();                  // the staging area may be written again
     __syncwarp();
     int16_t* pub_cb = pubst + lane * npub;
@@ -690,13 +694,13 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
     }
     t = tn;
   }
-  if (BULK && fail) mbar_wait(bar, phase);   // a copy still in flight
+  if (BULK && lost) load_drain(ld, bar, 1);
   bulk_wait_all();
   if (lane == 0) {
     if (a.counters) {
       if (nties) atomicAdd(&a.counters[0], (unsigned long long)nties);
       if (esc) atomicAdd(&a.counters[1], (unsigned long long)esc);
-      if (fail) atomicAdd(&a.counters[2], 1ull);
+      if (fail || lost) atomicAdd(&a.counters[2], 1ull);
     }
   }
 }
@@ -749,6 +753,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
   uint4* const ctab = reinterpret_cast<uint4*>(next + 4);
   const int act = a.groups;
   PlanClaim claim(a, act);
+  Loads ld;
   // subtile t of slot s starts loading; bulk: by bulk copies (they complete on the mbarrier)
   auto load = [&](const PlanSlot* s, uint32_t t, bool& bulk) {
     const uint32_t cb = 32u * t + lane, b = cb / 3, bxc = s->bx_count;
@@ -759,6 +764,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
     const uint64_t pitch = 3ull * s->width;
     const uint32_t n = min(32u, s->ncb - 32u * t);
     bulk = bxc >= 12 && (reinterpret_cast<uintptr_t>(s->px) & 15) == 0;
+    if (bulk) ld.issued(0);
     return bulk ? load_subtile<true>(s->px, pitch, bxc, p, n, lane, pix, bar)
                 : load_subtile<false>(s->px, pitch, bxc, p, n, lane, pix, bar);
   };
@@ -772,7 +778,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
   __syncthreads();                         // a first claim may go on to the counter
   int esc = 0, nties = 0;
   bool fail = false, lost = false, bulk = false;
-  uint32_t phase = 0, t = 0, end = 0, tn, endn;
+  uint32_t t = 0, end = 0, tn, endn;
   PlanSlot *s = slots, *sn = slots + 1;
   PixAt at{};
   if (warp < act) {                        // the first run starts loading before the tables are filled
@@ -798,11 +804,10 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
     for (; t < end; ++t) {
       const uint32_t n = min(32u, s->ncb - 32u * t);
       if (bulk) {
-        if (!__all_sync(0xffffffffu, mbar_wait(bar, phase))) {   // gave up: nothing more is written
+        if (!load_wait(ld, bar, 0)) {      // gave up: nothing more is written
           lost = true;
           break;
         }
-        phase ^= 1u;
       } else {
         cp_async_wait_all();
       }
@@ -842,7 +847,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
     t = tn;
     end = endn;
   }
-  if (lost) mbar_wait(bar, phase);         // a copy still in flight
+  if (lost) load_drain(ld, bar, 1);
   bulk_wait_all();
   if (lane == 0 && a.counters) {
     if (nties) atomicAdd(&a.counters[0], (unsigned long long)nties);

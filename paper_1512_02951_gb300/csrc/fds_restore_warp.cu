@@ -311,12 +311,15 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
     return t & 0x7fffffffu;
   };
   auto nof = [&](uint32_t t) { return (int)min(32u, ncb - 32u * t); };
+  Loads ld;                                // barrier 0: public, 1 and 2: the private buffers
   auto load_pub = [&](uint32_t t) {
     load_part(pubst, reinterpret_cast<const uint8_t*>(a.pub_in) + (uint64_t)t * (64u * npub), nof(t) * 2 * npub, lane, bars);
+    ld.issued(0);
   };
   auto load_priv = [&](uint32_t t, int cnt, int half) {
     load_part(privst + half * priv_half, a.priv_in + (uint64_t)t * (64u * (k + 1)),
               ((cnt - 1) * 32 + nof(t + cnt - 1)) * 2 * (k + 1), lane, bars + 1 + half);
+    ld.issued(1 + half);
   };
 
   if (lane == 0) {
@@ -361,7 +364,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
     __syncwarp();
   }
   bool lost = false;
-  uint32_t ph = 0;                         // phases: bit 0 public, bits 1 and 2 the private buffers
   while (run < s1) {
     run_n = claim(cnt_n);
     if (!PUBIMG) {
@@ -370,12 +372,11 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
         __syncwarp();
         load_priv(run_n, cnt_n, half ^ 1);
       }
-      if (!__all_sync(0xffffffffu, mbar_wait(bars + 1 + half, (ph >> (1 + half)) & 1u))) {
+      if (!load_wait(ld, bars, 1 + half)) {
         lost = true;
         break;
       }
       __syncwarp();
-      ph ^= 2u << half;
       if (cipher) {
         uint8_t* const buf = privst + half * priv_half;
         const uint32_t total = (uint32_t)cnt * nb;
@@ -411,12 +412,11 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
       const uint32_t t = run + ti;
       const int n = nof(t);
       const CbPos at = cb_pos(a, 32u * t + lane);
-      if (!__all_sync(0xffffffffu, mbar_wait(bars, ph & 1u))) {   // gave up: nothing more is written
+      if (!load_wait(ld, bars, 0)) {       // gave up: nothing more is written
         lost = true;
         break;
       }
       __syncwarp();
-      ph ^= 1u;
       const int16_t* pub_cb = reinterpret_cast<const int16_t*>(pubst) + lane * npub;
       const int16_t* priv_cb = reinterpret_cast<const int16_t*>(privst + half * priv_half) + (ti * kWCb + lane) * (k + 1);
       float2 G2[8][4];
@@ -442,10 +442,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
     cnt = cnt_n;
     if (twice) half ^= 1;
   }
-  if (lost) {                              // copies still in flight
-    mbar_wait(bars, ph & 1u);
-    if (!PUBIMG && twice && run_n < s1) mbar_wait(bars + 1 + (half ^ 1), (ph >> (1 + (half ^ 1))) & 1u);
-  }
+  if (lost) load_drain(ld, bars, 3);
   if (lane == 0 && a.counters) {
     if (slot->ties) atomicAdd(&a.counters[0], (unsigned long long)slot->ties);
     if (slot->esc) atomicAdd(&a.counters[1], (unsigned long long)slot->esc);
@@ -594,12 +591,15 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_packed_kernel(const __
   const uint32_t t0 = warp < act ? (uint32_t)((uint64_t)nsub * id / nw) : 0u;
   const uint32_t t1 = warp < act ? (uint32_t)((uint64_t)nsub * (id + 1) / nw) : 0u;
   auto nof = [&](uint32_t t) { return (int)min(32u, ncb - 32u * t); };
+  Loads ld;                                // barrier 0: public, 1: private
   auto load_pub = [&](uint32_t t) {
+    ld.issued(0);
     return land_stream(land_pub, reinterpret_cast<const uint8_t*>(a.pub_in), pub_total, (uint64_t)t * pub_per,
                        (nof(t) * npub * W + 7) >> 3, lane, bars);
   };
   auto load_priv = [&](uint32_t t) {
     const int cnt = min(G, (int)(t1 - t));
+    ld.issued(1);
     return land_stream(land_priv, a.priv_in, priv_total, (uint64_t)t * priv_per,
                        (cnt - 1) * (int)priv_per + ((nof(t + cnt - 1) * period + 7) >> 3), lane, bars + 1);
   };
@@ -626,16 +626,15 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_packed_kernel(const __
   __syncthreads();
 
   bool lost = false;
-  uint32_t ph = 0, run = t0;               // phases: bit 0 public, bit 1 private; the run's first subtile
+  uint32_t run = t0;                       // the run's first subtile
 #pragma unroll 1
   for (uint32_t t = t0; t < t1; ++t) {
     const int n = nof(t);
     if (t == run) {                        // a new run: decrypt its private parts where they landed
-      if (!__all_sync(0xffffffffu, mbar_wait(bars + 1, ph >> 1))) {
+      if (!load_wait(ld, bars, 1)) {
         lost = true;
         break;
       }
-      ph ^= 2u;
       __syncwarp();
       const int cnt = min(G, (int)(t1 - t));
       const uint64_t off = (uint64_t)t * priv_per;
@@ -656,11 +655,10 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_packed_kernel(const __
       }
       __syncwarp();
     }
-    if (!__all_sync(0xffffffffu, mbar_wait(bars, ph & 1u))) {   // gave up: nothing more is written
+    if (!load_wait(ld, bars, 0)) {         // gave up: nothing more is written
       lost = true;
       break;
     }
-    ph ^= 1u;
     __syncwarp();
     unpack_public<W>(reinterpret_cast<const uint32_t*>(land_pub + skew_pub), pubst, n, npub, lane);
     unpack_private<W>(reinterpret_cast<const uint32_t*>(land_priv + skew_priv), privst + lane * (k + 1),
@@ -691,10 +689,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_packed_kernel(const __
     store_pixels(a.pixels_out, 3ull * (uint64_t)a.width, at, c0, n, lane, pix);
     __syncwarp();                          // the staging area and the pixel buffer may be written again
   }
-  if (lost) {                              // copies still in flight
-    mbar_wait(bars, ph & 1u);
-    mbar_wait(bars + 1, ph >> 1);
-  }
+  if (lost) load_drain(ld, bars, 2);
   if (lane == 0 && a.counters) {
     if (slot->ties) atomicAdd(&a.counters[0], (unsigned long long)slot->ties);
     if (slot->esc) atomicAdd(&a.counters[1], (unsigned long long)slot->esc);
@@ -779,12 +774,15 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
   const int act = a.groups;
   PlanClaim claim(a, act);
   auto nof = [&](const PlanSlot* s, uint32_t t) { return (int)min(32u, s->ncb - 32u * t); };
+  Loads ld;                                // barrier 0: public, 1 and 2: the private buffers
   auto load_pub = [&](const PlanSlot* s, uint32_t t) {
     const int npub = 63 - (K >= 0 ? K : s->k);
+    ld.issued(0);
     load_part(frag, s->pub + (uint64_t)t * (64u * npub), nof(s, t) * 2 * npub, lane, bars);
   };
   auto load_priv = [&](const PlanSlot* s, uint32_t t, int cnt, int half) {
     const int k = K >= 0 ? K : s->k;
+    ld.issued(1 + half);
     load_part(frag + kWCb * 2 * (63 - k) + half * (s->acc & 15) * 64 * (k + 1), s->priv + (uint64_t)t * (64u * (k + 1)),
               ((cnt - 1) * 32 + nof(s, t + cnt - 1)) * 2 * (k + 1), lane, bars + 1 + half);
   };
@@ -800,7 +798,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
   if (threadIdx.x == 0) *next = (uint32_t)act;
   __syncthreads();                         // a first claim may go on to the counter
   bool lost = false;
-  uint32_t ph = 0;                         // phases: bit 0 public, bits 1 and 2 the private buffers
   PlanSlot *s = slots, *sx = slots + 1;    // the run's image; the other slot
   uint32_t r = 0, end = 0;                 // the run's first subtile, the end of what was claimed
   int half = 0;
@@ -840,11 +837,10 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
       __syncwarp();
       load_priv(n, rn, cntn, half ^ 1);
     }
-    if (!__all_sync(0xffffffffu, mbar_wait(bars + 1 + half, (ph >> (1 + half)) & 1u))) {
+    if (!load_wait(ld, bars, 1 + half)) {
       lost = true;
       break;
     }
-    ph ^= 2u << half;
     __syncwarp();
     ctr_plan(privst, (((cnt - 1) * 32 + nof(s, r + cnt - 1)) * 2 * (k + 1) + 15) >> 4, (uint64_t)r * (uint32_t)(4 * (k + 1)),
              s, wins, lane);
@@ -860,11 +856,10 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
         at.by = b / bxc;
         at.bx = b - at.by * bxc;
       }
-      if (!__all_sync(0xffffffffu, mbar_wait(bars, ph & 1u))) {   // gave up: nothing more is written
+      if (!load_wait(ld, bars, 0)) {       // gave up: nothing more is written
         lost = true;
         break;
       }
-      ph ^= 1u;
       __syncwarp();
       const int16_t* pub_cb = reinterpret_cast<const int16_t*>(frag) + lane * npub;
       const int16_t* priv_cb = reinterpret_cast<const int16_t*>(privst) + (ti * kWCb + lane) * (k + 1);
@@ -899,11 +894,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
     r = rn;
     end = endn;
   }
-  if (lost) {                              // copies still in flight
-    mbar_wait(bars, ph & 1u);
-    mbar_wait(bars + 1, (ph >> 1) & 1u);
-    mbar_wait(bars + 2, (ph >> 2) & 1u);
-  }
+  if (lost) load_drain(ld, bars, 3);
   if (lane == 0 && a.counters) {
     if (slot->ties) atomicAdd(&a.counters[0], (unsigned long long)slot->ties);
     if (slot->esc) atomicAdd(&a.counters[1], (unsigned long long)slot->esc);

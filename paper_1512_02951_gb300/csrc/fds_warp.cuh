@@ -2,6 +2,7 @@
 // per lane), their place in the image, and AES-128-CTR with the first rounds of neighbouring
 // counter blocks computed once.
 #pragma once
+#include "fds_loads.h"
 #include "fds_tile.cuh"
 
 namespace fds {
@@ -11,6 +12,17 @@ constexpr int kWarps = 16;                        // per CTA, one CTA per SM
 // AES constants of counter windows, 5 words each: of the whole CTA's range where it has at most
 // kWins, else two for each warp
 constexpr int kWins = 64;
+
+// wait for the copy pending on barrier i of the warp's (the whole warp); false: gave up
+__device__ __forceinline__ bool load_wait(Loads& ld, uint64_t* bars, int i) {
+  const bool ok = __all_sync(0xffffffffu, mbar_wait(bars + i, ld.parity(i)));
+  if (ok) ld.arrived(i);
+  return ok;
+}
+// after giving up: the copies still under way
+__device__ __forceinline__ void load_drain(const Loads& ld, uint64_t* bars, int n) {
+  ld.drain(n, [&](int i, uint32_t parity) { mbar_wait(bars + i, parity); });
+}
 
 // One image position of a lane's channel-block: block column, block row, channel
 struct CbPos {
