@@ -815,6 +815,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
       const uint32_t c = at.c;
       float2 P[8][4];
       const float V = transform_rows(area + kWPix + at.even, area + kWPix + at.odd, c, P);
+      // cp.async wrote the buffer through the generic proxy; a bulk copy may write it next
+      if (!bulk) fence_proxy_async();
       __syncwarp();                        // the pixel buffer is read: the next subtile's load starts
       if (t + 1 < end)
         at = load(s, t + 1, bulk);

@@ -61,7 +61,8 @@ __host__ __device__ constexpr int run_tiles(int k) {
 __host__ __device__ constexpr bool run_twice(int k) { return (63 - k) * 64 + 2 * run_tiles(k) * (k + 1) * 64 <= kRFragBytes; }
 
 // bytes of a fragment part to shared memory: a bulk copy completing on bar (lane 0 announces it),
-// and a tail of 2-byte copies
+// and a tail of 2-byte copies (only behind the last, short subtile of an image: where another
+// image's part follows in the buffer, the lanes fence their stores before the next bulk copy)
 __device__ __forceinline__ void load_part(uint8_t* dst, const uint8_t* src, int bytes, int lane, uint64_t* bar) {
   const int b16 = bytes & ~15;
   if (lane == 0) {
@@ -491,13 +492,14 @@ __host__ __device__ constexpr int run_tiles_packed(int k) {
 // bytes [off, off + bytes) of a stream of `total` bytes (off a multiple of 4, the stream 8-byte
 // aligned) to the 16-byte aligned dst, whose first byte stands for the 16-byte boundary at or below
 // the first one; returns the distance from there.  Where the widened copy would leave the stream,
-// the lanes copy words and bytes.
+// the lanes copy words and bytes (by_lanes: fence their stores before the next bulk copy there).
 __device__ __forceinline__ uint32_t land_stream(uint8_t* dst, const uint8_t* stream, uint64_t total, uint64_t off, int bytes,
-                                                int lane, uint64_t* bar) {
+                                                int lane, uint64_t* bar, bool& by_lanes) {
   const uint8_t* src = stream + off;
   const uint32_t skew = (uint32_t)(reinterpret_cast<uintptr_t>(src) & 15);
   const uint32_t wide = (skew + (uint32_t)bytes + 15u) & ~15u;
-  if (off >= skew && off - skew + wide <= total) {
+  by_lanes = off < skew || off - skew + wide > total;
+  if (!by_lanes) {
     if (lane == 0) {
       mbar_expect_tx(bar, wide);
       if (wide) bulk_load(dst, src - skew, wide, bar);
@@ -592,16 +594,18 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_packed_kernel(const __
   const uint32_t t1 = warp < act ? (uint32_t)((uint64_t)nsub * (id + 1) / nw) : 0u;
   auto nof = [&](uint32_t t) { return (int)min(32u, ncb - 32u * t); };
   Loads ld;                                // barrier 0: public, 1: private
+  bool lanes_pub = false;                  // the public part at hand was landed by the lanes
   auto load_pub = [&](uint32_t t) {
     ld.issued(0);
     return land_stream(land_pub, reinterpret_cast<const uint8_t*>(a.pub_in), pub_total, (uint64_t)t * pub_per,
-                       (nof(t) * npub * W + 7) >> 3, lane, bars);
+                       (nof(t) * npub * W + 7) >> 3, lane, bars, lanes_pub);
   };
   auto load_priv = [&](uint32_t t) {
     const int cnt = min(G, (int)(t1 - t));
+    bool by_lanes;                         // fenced below in any case
     ld.issued(1);
     return land_stream(land_priv, a.priv_in, priv_total, (uint64_t)t * priv_per,
-                       (cnt - 1) * (int)priv_per + ((nof(t + cnt - 1) * period + 7) >> 3), lane, bars + 1);
+                       (cnt - 1) * (int)priv_per + ((nof(t + cnt - 1) * period + 7) >> 3), lane, bars + 1, by_lanes);
   };
 
   if (lane == 0) {
@@ -665,7 +669,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_packed_kernel(const __
                       (int)(t - run) * kWCb + (lane < n ? lane : 0), k);
     if (t + 1 < t1) {
       const bool last = t + 1 - run == (uint32_t)G;   // of the run: the next one's private parts load too
-      if (last) fence_proxy_async();       // the landing area was decrypted in place
+      // the private parts were decrypted in place, or the public one landed by the lanes' stores
+      if (last || lanes_pub) fence_proxy_async();
       __syncwarp();                        // unpacked: the landing areas are free
       skew_pub = load_pub(t + 1);
       if (last) {
@@ -865,6 +870,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
       const int16_t* priv_cb = reinterpret_cast<const int16_t*>(privst) + (ti * kWCb + lane) * (k + 1);
       float2 G2[8][4];
       const float l1 = gather_columns<false>(pub_cb, priv_cb, k, G2);
+      if (m < kWCb) fence_proxy_async();   // load_part's tail, before the next image's bulk copy
       __syncwarp();                        // the public part is read: the next one starts loading
       if (ti + 1 < cnt)
         load_pub(s, t + 1);
