@@ -1112,11 +1112,20 @@ int fds_protect_image_strong(const uint8_t* pixels, int32_t width, int32_t heigh
   cudaStream_t s = (cudaStream_t)stream;
   int16_t* s_pub = static_cast<int16_t*>(scratch);
   uint8_t* s_plain = static_cast<uint8_t*>(scratch) + align16u(pub16);
+  // the transform writes the ciphertext while it still reads pixels and writes scratch; a private
+  // buffer inside one of those (or under the public image) is written last, from the plaintext
+  auto apart = [&](const void* p, uint64_t bytes) {
+    const uintptr_t a0 = (uintptr_t)private_out, b0 = (uintptr_t)p;
+    return a0 + priv16 <= b0 || b0 + bytes <= a0;
+  };
+  const uint64_t px = (uint64_t)width * (uint64_t)height * 3ull;
+  const bool direct = apart(pixels, px) && apart(scratch, align16u(pub16) + priv16) && apart(public_image_out, px);
   TileArgs a{};                                  // 1. transform; Part 1 encrypted, and in plaintext
   a.pixels_in = pixels;
   a.pub_out = s_pub;
-  a.priv_out = private_out;
-  a.plain_out = s_plain;
+  a.priv_out = direct ? private_out : s_plain;
+  a.plain_out = direct ? s_plain : nullptr;
+  a.plain_private = !direct;
   fill_geometry(a, width, height, k);
   expand_key(key, a.rk);
   iv_words(iv, &a.iv_hi, &a.iv_lo);
@@ -1127,8 +1136,12 @@ int fds_protect_image_strong(const uint8_t* pixels, int32_t width, int32_t heigh
   b.public_image = 1;
   fill_geometry(b, width, height, k);
   if ((rc = run_restore(b, dev, s))) return rc;
-  const cudaError_t e = launch_strong_mask(s_plain, public_image_out, public_image_out, width, height, k, s);
-  return e == cudaSuccess ? FDS_OK : cuda_fail(e, "mask launch");   // 3. XOR the SHA-512 masks
+  cudaError_t e = launch_strong_mask(s_plain, public_image_out, public_image_out, width, height, k, s);
+  if (e != cudaSuccess) return cuda_fail(e, "mask launch");   // 3. XOR the SHA-512 masks
+  if (!direct)                                   // 4. encrypt Part 1
+    e = launch_aes_full(s_plain, private_out, priv16, a.iv_hi, a.iv_lo, a.rk, g_tables[dev].T, s, g_tables[dev].sms,
+                        g_tables[dev].counters);
+  return e == cudaSuccess ? FDS_OK : cuda_fail(e, "encryption launch");
 }
 
 int fds_restore_image_strong(const uint8_t* public_image_in, const uint8_t* private_in, int32_t width,
