@@ -25,14 +25,15 @@ namespace fds {
 //             coordinate j, 64 signed bytes K_j(u,v,y,x) (16 words, word w = row w/2,
 //             x = 4(w&1) .. +3)
 //  g_cinv     the same for the inverse: for pixel 8y+x and coordinate j, the weight of the
-//             coefficient at zigzag index z = 4t + byte (16 words)
+//             coefficient at zigzag index z = 4t + byte (16 words); behind it the same words by
+//             (t, j, pixel), for 32 lanes with a pixel each
 //  g_counters exact-fallback counters
 //  g_rk       round keys of the registered key slots (FDS_MAX_KEYS x 44 words)
 // where 8 b_u(y) b_v(x) = sum_j K_j(u,v,y,x) cos(j pi/16), cos(0) = 1.
 __device__ __align__(16) uint32_t g_T[1024];
 __device__ __align__(16) uint32_t g_rk[FDS_MAX_KEYS * 44];
 __device__ __align__(16) uint32_t g_cfwd[64 * 128];
-__device__ __align__(16) uint32_t g_cinv[64 * 128];
+__device__ __align__(16) uint32_t g_cinv[2 * 64 * 128];
 __device__ unsigned long long g_counters[3];
 //  g_tcb0/1   tensor-core B operands (basis limbs, BF16 / TF32) in shared-memory byte order
 __device__ __align__(16) uint4 g_tcb0[kTcBBytesBf16 / 16];
@@ -369,7 +370,7 @@ int ensure_init(int* dev_out = nullptr) {
             if (j < 8) K[u][v][y][x][j] = (int8_t)(K[u][v][y][x][j] + sg);
           }
         }
-  static uint32_t hf[64 * 128], hinv[64 * 128];
+  static uint32_t hf[64 * 128], hinv[2 * 64 * 128];
   std::memset(hf, 0, sizeof(hf));
   std::memset(hinv, 0, sizeof(hinv));
   int uz[64], vz[64];
@@ -393,6 +394,9 @@ int ensure_init(int* dev_out = nullptr) {
             const int z = 4 * tw + i;
             hinv[(8 * y + x) * 128 + 16 * j + tw] |= (uint32_t)(uint8_t)K[uz[z]][vz[z]][y][x][j] << (8 * i);
           }
+  for (int pos = 0; pos < 64; ++pos)
+    for (int j = 0; j < 8; ++j)
+      for (int tw = 0; tw < 16; ++tw) hinv[64 * 128 + (8 * tw + j) * 64 + pos] = hinv[pos * 128 + 16 * j + tw];
   if ((e = cudaMemcpyToSymbol(g_cfwd, hf, sizeof(hf))) != cudaSuccess) return cuda_fail(e, "table upload");
   if ((e = cudaMemcpyToSymbol(g_cinv, hinv, sizeof(hinv))) != cudaSuccess) return cuda_fail(e, "table upload");
   init_tables_kernel<<<1, 256>>>();

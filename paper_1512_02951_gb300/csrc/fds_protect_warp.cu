@@ -14,7 +14,7 @@
 //   2. column butterflies by pairs of columns, rounded and written as int16 to the staging area;
 //      a pair of columns in which some lane has a value within the error guard of a
 //      half-integer (one three-input maximum per two values, one vote) marks those values
-//   3. marked values are decided exactly by the whole warp at once (round_warp), in place
+//   3. marked values are decided exactly, four at a time (decide_ties), in place
 //   4. the public part leaves (bulk store); the private parts of several subtiles are collected
 //      until their keystream blocks fill whole warps (k = 5: 24 blocks each, four subtiles fill
 //      three), encrypted, and leave
@@ -40,7 +40,7 @@ constexpr int kWStage = kWPix + kWPixBytes;
 constexpr int kWList = kWStage + kWStageBytes;    // the staged private parts' subtiles
 constexpr int kWBar = kWList + 4 * 8;             // mbarrier of the pixel loads
 constexpr int kWArea = (kWBar + 8 + 31) & ~31;
-constexpr int kWWinBytes = 20 * kWins + 16 + 512; // and the CTA's subtile counter, and c(m) folded
+constexpr int kWWinBytes = 20 * kWins + 16;       // and the CTA's subtile counter
 constexpr int kBelow = ((int)kTpairWin - 1024) / kWArea;    // areas below the pair table
 constexpr int kWLow = (int)kTpairWin - kBelow * kWArea;     // window address of the first
 constexpr int kAbove = kWarps > kBelow ? kWarps - kBelow : 0;
@@ -175,51 +175,6 @@ __device__ __forceinline__ void store_run(uint8_t* dst, const uint8_t* src, int 
     *reinterpret_cast<uint16_t*>(dst + j) = *reinterpret_cast<const uint16_t*>(src + j);
 }
 
-// Exact rounding of coefficient pos of one channel-block by the whole warp (pos and px, the
-// block's first byte of the channel, the same in every lane).  8 F is the sum of p[y][x]
-// (c(a - b) + c(a + b)), a = (2 y + 1) u or 4, b = (2 x + 1) v or 4 (fds_device.cuh).  Each lane
-// takes two pixels; their parts of the coordinates n_j of c(j), j = 0..7, are added as pairs of
-// 16-bit fields (|n_j| <= 2 . 64 . 255 < 2^15), so four warp sums give them all.  The value is
-// then decided in 64-bit fixed point: each c(j) 2^46 is within a unit, so the sum is within
-// sum |n_j| <= 2^15 units.  Nearer than that to a boundary it is a tie if it is rational (about
-// half of all near ties: positions whose u and v are 2 or 6), and else left to exact_round.
-constexpr int kTieFrac = 46;
-__device__ __noinline__ int round_far(const int (&n)[9], int* esc, bool* fail) { return exact_round(n, esc, fail); }
-__device__ __forceinline__ int round_warp(const uint8_t* px, uint64_t pitch, int pos, const uint4* ctab, int lane,
-                                          int& esc, bool& fail) {
-  const int u = pos >> 3, v = pos & 7, y = lane >> 2, x = 2 * (lane & 3);
-  const int a = u ? (2 * y + 1) * u : 4, b = v ? (2 * x + 1) * v : 4, b2 = v ? b + 2 * v : 4;
-  const uint8_t* p = px + y * pitch + 3 * x;
-  const uint32_t p0 = __ldg(p), p1 = __ldg(p + 3);
-  const uint4 A = ctab[(a - b) & 31], B = ctab[(a + b) & 31], C = ctab[(a - b2) & 31], D = ctab[(a + b2) & 31];
-  const uint32_t w[4] = {p0 * (A.x + B.x) + p1 * (C.x + D.x), p0 * (A.y + B.y) + p1 * (C.y + D.y),
-                         p0 * (A.z + B.z) + p1 * (C.z + D.z), p0 * (A.w + B.w) + p1 * (C.w + D.w)};
-  int n[9];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint32_t s = __reduce_add_sync(0xffffffffu, w[i]);
-    n[2 * i] = (int16_t)(s & 0xffffu);
-    n[2 * i + 1] = (int)(s - (uint32_t)n[2 * i]) >> 16;
-  }
-  n[8] = 0;
-  long long d = (long long)(n[0] + 4) << kTieFrac;
-  int any = 0;
-#pragma unroll
-  for (int j = 1; j < 8; ++j) {
-    d += (long long)n[j] * (c_cos_q62[j - 1] >> (62 - kTieFrac));
-    any |= n[j];
-  }
-  // d / 2^49 = F + 1/2
-  const int q = (int)(d >> (kTieFrac + 3));
-  const long long rem = d & ((8ll << kTieFrac) - 1);
-  if (any == 0) return rem == 0 && q <= 0 ? q - 1 : q;      // rational: a tie goes away from zero
-  if (rem > 32768 && rem < (8ll << kTieFrac) - 32768) return q;
-  int e = 0;
-  const int r = round_far(n, &e, &fail);
-  esc += e;
-  return r;
-}
-
 // Row butterflies of a lane's channel-block from its pixel buffer: outputs as pairs of columns
 // (0, 4), (1, 2), (3, 5), (6, 7), so that the column pass runs on two columns per packed f32x2
 // instruction; returns the row passes' error weight
@@ -310,27 +265,80 @@ __device__ __forceinline__ void stage_columns(const float2 (&P)[8][4], float V, 
   }
 }
 
-// The marked values of the subtile whose first channel-block is cb0, one after another, each
-// decided by the whole warp and staged by its lane (c, pub_cb, priv_cb: the lane's own)
-__device__ __forceinline__ void decide_ties(const uint8_t* img, uint64_t pitch, uint32_t bx_count, uint32_t cb0, uint32_t c,
-                                            int k, uint32_t mlo, uint32_t mhi, int16_t* pub_cb, int16_t* priv_cb,
-                                            const uint4* ctab, int lane, int& nties, int& esc,
-                                            bool& fail) {
-  for (uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0); who; who &= who - 1) {
-    const int src = __ffs(who) - 1;
-    uint64_t mask = (uint64_t)__shfl_sync(0xffffffffu, mhi, src) << 32 | __shfl_sync(0xffffffffu, mlo, src);
-    const uint32_t sc = __shfl_sync(0xffffffffu, c, src);
-    const uint32_t b = (cb0 + src) / 3, by = b / bx_count;
-    const uint8_t* blk = img + (uint64_t)by * (8 * pitch) + 24ull * (b - by * bx_count);
-    nties += __popcll(mask);
-    for (; mask; mask &= mask - 1) {
-      const int pos = __ffsll((long long)mask) - 1;
-      int e = 0;
-      const int q = round_warp(blk + sc, pitch, pos, ctab, lane, e, fail);
-      esc += e;
-      const int z = zigzag_of(pos >> 3, pos & 7);
-      if (lane == src) *(z <= k ? priv_cb + z : pub_cb + (z - k - 1)) = (int16_t)q;
+// The marked values of a subtile, decided exactly (take_ties) and staged.  block(): the lane's own
+// block in the image; pub0, priv0: the first lane's place in the staging area; table: a.cfwd, whose
+// row of a position holds eight words a coordinate pair: a lane takes a pixel row and its two words.
+// |n_j| <= 2 . 64 . 255 and so is their sum, so 46 fraction bits fit.  Where kSideBySide lanes or more
+// have marked values, each decides one of its own instead (two rows at a time: all eight held
+// spilled); below, two turns at most do (tie block: turns alone 117 us).
+constexpr int kTieFrac = 46;
+constexpr int kSideBySide = 8;
+template <typename Block>
+__device__ __forceinline__ void decide_ties(Block block, uint64_t pitch, uint32_t c, int k, uint32_t mlo, uint32_t mhi,
+                                            int16_t* pub0, int16_t* priv0, const uint32_t* table, int lane, int& nties,
+                                            int& esc, bool& fail) {
+  uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
+  if (__builtin_expect(who == 0, 1)) return;
+  // read here, so that what depends on it is not kept through the subtiles without near ties
+  asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+  nties += (int)__reduce_add_sync(0xffffffffu, (uint32_t)(__popc(mlo) + __popc(mhi)));
+  const unsigned long long blk = reinterpret_cast<unsigned long long>(block());
+  const long long cos_l = group_cos<kTieFrac>(lane);
+  const int l = lane & 7;
+  auto put = [&](int src, int pos, int q) {
+    const int z = c_zigzag.z[pos];
+    *(z <= k ? priv0 + src * (k + 1) + z : pub0 + src * (63 - k) + (z - k - 1)) = (int16_t)q;
+  };
+  uint32_t hlo = 0, hhi = 0;               // side by side, too near a boundary: by a group after all
+  while (__popc(who) >= kSideBySide) {
+    if (mlo | mhi) {
+      const int pos = mlo ? __ffs(mlo) - 1 : __ffs(mhi) + 31;
+      const uint8_t* row = reinterpret_cast<const uint8_t*>(blk);
+      int n[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll 1
+      for (int g = 0; g < 4; ++g) {
+        const uint4* t4 = reinterpret_cast<const uint4*>(table + pos * 128) + g;
+        uint32_t P[4];
+        pixel_row_global(row, c, P[0], P[1]);
+        pixel_row_global(row + pitch, c, P[2], P[3]);
+        row += 2 * pitch;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint4 w = __ldg(t4 + 4 * j);
+          n[j] = dp4a_us(P[1], w.y, dp4a_us(P[0], w.x, n[j]));
+          n[j] = dp4a_us(P[3], w.w, dp4a_us(P[2], w.z, n[j]));
+        }
+      }
+      bool sure;
+      put(lane, pos, round_lane<kTieFrac>(n, sure));
+      const uint32_t lo = mlo & -mlo, hi = mlo ? 0u : mhi & -mhi;
+      mlo ^= lo;
+      mhi ^= hi;
+      if (!sure) hlo |= lo, hhi |= hi;
     }
+    who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
+  }
+  mlo |= hlo;
+  mhi |= hhi;
+  who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
+  while (who) {
+    const TieTurn t = take_ties(who, mlo, mhi, lane);
+    const uint8_t* row = reinterpret_cast<const uint8_t*>(__shfl_sync(0xffffffffu, blk, t.src)) + l * pitch;
+    const uint32_t sc = __shfl_sync(0xffffffffu, c, t.src);
+    int n[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (t.on) {
+      const uint2* w2 = reinterpret_cast<const uint2*>(table + t.pos * 128) + l;
+      uint32_t lo, hi;
+      pixel_row_global(row, sc, lo, hi);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const uint2 w = __ldg(w2 + 8 * j);
+        n[j] = dp4a_us(hi, w.y, dp4a_us(lo, w.x, 0));
+      }
+    }
+    const int q = round_group<kTieFrac, 1 << 15>(group_sum(n, lane), cos_l, t.on, lane, esc, fail);
+    if (t.on && l == 0) put(t.src, t.pos, q);
+    who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
   }
 }
 
@@ -546,7 +554,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
   uint32_t* list = reinterpret_cast<uint32_t*>(area + kWList);
   uint32_t* wins = reinterpret_cast<uint32_t*>(smem_cta + (kWWin - win0));
   uint32_t* next = wins + 5 * kWins;
-  uint4* ctab = reinterpret_cast<uint4*>(next + 4);
   const int k = K >= 0 ? K : a.k;
   const int npub = 63 - k;
   const uint32_t nb = 4u * (uint32_t)(k + 1);       // keystream blocks per subtile
@@ -581,11 +588,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
   };
   if (t < tend) load(t);
   if (threadIdx.x == 0) *next = s0 + act;
-  if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
-    const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
-    const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
-    ctab[lane] = make_uint4(f >> 1 == 0 ? one : 0u, f >> 1 == 1 ? one : 0u, f >> 1 == 2 ? one : 0u, f >> 1 == 3 ? one : 0u);
-  }
   fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
   __syncthreads();
   if (PACK == 0 && !a.plain_private) {
@@ -636,7 +638,12 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
     int16_t* priv_cb = reinterpret_cast<int16_t*>(privst) + ((PACK ? 0 : acc * kWCb) + lane) * (k + 1);
     uint32_t mlo, mhi;
     stage_columns(P, V, k, (uint32_t)lane < n, pub_cb, priv_cb, mlo, mhi);
-    decide_ties(a.pixels_in, pitch, (uint32_t)a.bx_count, 32u * t, c, k, mlo, mhi, pub_cb, priv_cb, ctab, lane, nties, esc, fail);
+    decide_ties(
+        [&] {
+          const CbPos p = cb_pos(a, 32u * t + lane);
+          return a.pixels_in + (uint64_t)p.by * (8 * pitch) + 24ull * p.bx;
+        },
+        pitch, c, k, mlo, mhi, pubst, priv_cb - lane * (k + 1), a.cfwd, lane, nties, esc, fail);
     if constexpr (PACK != 0) {
       constexpr int kPW = PACK ? PACK : 8;
       __syncwarp();                        // every staged coefficient is final
@@ -713,8 +720,8 @@ constexpr int kPArea = (kPWins + 40 + 31) & ~31;
 constexpr int kPBelow = ((int)kTpairWin - 1024) / kPArea;
 constexpr int kPLow = (int)kTpairWin - kPBelow * kPArea;
 constexpr int kPAbove = kWarps > kPBelow ? kWarps - kPBelow : 0;
-constexpr int kPTail = (int)kTpairWin + kTpairBytes + kPAbove * kPArea;   // counter, folded c(m)
-constexpr int kPEnd = kPTail + 16 + 512;
+constexpr int kPTail = (int)kTpairWin + kTpairBytes + kPAbove * kPArea;   // counter
+constexpr int kPEnd = kPTail + 16;
 static_assert(kPEnd <= 227 * 1024 && kPSlot % 8 == 0, "protect (batches) shared memory");
 
 // acc_tiles(k), at most a tile
@@ -750,7 +757,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
   PlanSlot* const slots = reinterpret_cast<PlanSlot*>(area + kPSlot);
   uint32_t* const wins = reinterpret_cast<uint32_t*>(area + kPWins);
   uint32_t* const next = reinterpret_cast<uint32_t*>(smem_cta + (kPTail - win0));
-  uint4* const ctab = reinterpret_cast<uint4*>(next + 4);
   const int act = a.groups;
   PlanClaim claim(a, act);
   Loads ld;
@@ -784,11 +790,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
   if (warp < act) {                        // the first run starts loading before the tables are filled
     claim(a, act, next, s, s, c_acc.n, warp, lane, t, end);
     if (t < end) at = load(s, t, bulk);
-  }
-  if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
-    const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
-    const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
-    ctab[lane] = make_uint4(f >> 1 == 0 ? one : 0u, f >> 1 == 1 ? one : 0u, f >> 1 == 2 ? one : 0u, f >> 1 == 3 ? one : 0u);
   }
   fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
   __syncthreads();
@@ -828,7 +829,12 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
       int16_t* const priv_cb = reinterpret_cast<int16_t*>(privst) + (acc * kWCb + lane) * (k + 1);
       uint32_t mlo, mhi;
       stage_columns(P, V, k, (uint32_t)lane < n, pub_cb, priv_cb, mlo, mhi);
-      decide_ties(s->px, pitch, s->bx_count, 32u * t, c, k, mlo, mhi, pub_cb, priv_cb, ctab, lane, nties, esc, fail);
+      decide_ties(
+          [&] {
+            const uint32_t b = (32u * t + lane) / 3, by = b / s->bx_count;
+            return s->px + (uint64_t)by * (8 * pitch) + 24ull * (b - by * s->bx_count);
+          },
+          pitch, c, k, mlo, mhi, reinterpret_cast<int16_t*>(stage), priv_cb - lane * (k + 1), a.cfwd, lane, nties, esc, fail);
       fence_proxy_async();                 // staged coefficients, before the bulk store
       __syncwarp();
       if (lane == 0) store_run(s->pub + (uint64_t)t * (64u * npub), stage, (int)n * 2 * npub);

@@ -14,8 +14,8 @@
 //      free, so the next subtile's public part starts loading
 //   2. row butterflies, round and clamp, bytes into the warp's pixel buffer; a row in which some
 //      lane has a value within the error guard of a half-integer marks those values
-//   3. marked values are decided exactly by the whole warp at once (round_warp_inv): public
-//      coefficients from global memory, private ones from the decrypted buffer
+//   3. marked values are decided exactly, four at a time (decide_pixels): public coefficients from
+//      global memory, private ones from the decrypted buffer
 //   4. the ten whole blocks go out as 8-byte pieces, each lane its block's piece c; the two
 //      channel-blocks of a block shared with a neighbouring subtile as bytes
 // Private parts come in runs of subtiles whose keystream blocks fill whole warps (k = 5: four
@@ -35,7 +35,7 @@ constexpr int kRFragBytes = 6784;                 // subtiles, twice where that 
 constexpr int kRBar = kRFrag + kRFragBytes;       // mbarriers: public, private (two)
 constexpr int kRSlot = kRBar + 3 * 8;             // what a warp looks at once per run (WarpSlot)
 constexpr int kRArea = (kRSlot + 32 + 31) & ~31;
-constexpr int kRWinBytes = 20 * kWins + 16 + 512 + 128;   // windows, subtile counter, folded c(m), (u, v) by zigzag
+constexpr int kRWinBytes = 20 * kWins + 16;       // windows, subtile counter
 constexpr int kRBelow = ((int)kTpairWin - 1024) / kRArea;
 constexpr int kRLow = (int)kTpairWin - kRBelow * kRArea;
 constexpr int kRAbove = kWarps > kRBelow ? kWarps - kRBelow : 0;
@@ -80,60 +80,6 @@ struct WarpSlot {
   uint64_t wbase;
 };
 static_assert(sizeof(WarpSlot) == 32, "WarpSlot");
-
-// Exact rounding of pixel pos of one channel-block by the whole warp: pub / priv its public and
-// (decrypted) private coefficients.  As in protect (round_warp there), with 32-bit coordinates:
-// int16 coefficients of any value make |n_j| <= 2^22, so the constants carry 40 fraction bits and
-// the error bound is the sum of the |n_j|.
-__device__ __noinline__ int round_far_inv(const int (&n)[9], int* esc, bool* fail) { return exact_round(n, esc, fail); }
-template <bool PUBIMG, bool STAGED = false>
-__device__ __forceinline__ int round_warp_inv(const int16_t* pub, const int16_t* priv, int k, int pos, const uint4* ctab,
-                                              const uint8_t* uv, int lane, WarpSlot* slot) {
-  const int y = pos >> 3, x = pos & 7;
-  uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int z = 2 * lane + i, t = uv[z], u = t >> 3, v = t & 7;
-    const int q = z <= k ? (PUBIMG ? (z == 0 ? 1024 : 0) : priv[z]) : (STAGED ? pub[z - k - 1] : __ldg(pub + z - k - 1));
-    const int a = u ? (2 * y + 1) * u : 4, b = v ? (2 * x + 1) * v : 4;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const uint4 f = ctab[(h ? a + b : a - b) & 31];            // +-1 in one 16-bit field
-      const uint32_t fw[4] = {f.x, f.y, f.z, f.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int lo = (int16_t)(fw[j] & 0xffffu), hi = (int)(fw[j] - (uint32_t)lo) >> 16;
-        w[2 * j] += (uint32_t)(q * lo);
-        w[2 * j + 1] += (uint32_t)(q * hi);
-      }
-    }
-  }
-  int n[9];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) n[j] = (int)__reduce_add_sync(0xffffffffu, w[j]);
-  n[8] = 0;
-  constexpr int kFrac = 40;
-  long long d = ((long long)n[0] + 4) << kFrac;
-  long long err = 0;
-#pragma unroll
-  for (int j = 1; j < 8; ++j) {
-    d += (long long)n[j] * (c_cos_q62[j - 1] >> (62 - kFrac));
-    err += n[j] < 0 ? -n[j] : n[j];
-  }
-  // d / 2^43 = p + 1/2
-  const int q = (int)(d >> (kFrac + 3));
-  const long long rem = d & ((8ll << kFrac) - 1);
-  if (err == 0) return rem == 0 && q <= 0 ? q - 1 : q;      // rational: a tie goes away from zero
-  if (rem > err && rem < (8ll << kFrac) - err) return q;
-  int e = 0;
-  bool fail = false;
-  const int r = round_far_inv(n, &e, &fail);
-  if (lane == 0) {
-    slot->esc += e;
-    slot->fail |= fail;
-  }
-  return r;
-}
 
 // The coefficients of a lane's channel-block (z = 0 .. k at priv_cb, the rest at pub_cb) to
 // floats, two columns at a time through the column butterflies; returns sum |F|
@@ -202,24 +148,96 @@ __device__ __forceinline__ void emit_rows(const float2 (&G2)[8][4], float l1, bo
   }
 }
 
-// The marked values of a subtile, one after another, each decided by the whole warp and written
-// by its lane (priv_cb, out: the lane's own; pub_g: the subtile's public coefficients in global
-// memory, or STAGED in shared memory)
+// The marked pixels of a subtile, decided exactly (take_ties) and written to the pixel buffer pix, where
+// out is the lane's own block and channel.  pub_g: the subtile's public coefficients in global memory,
+// or STAGED in shared memory; priv0: the first lane's (decrypted) private ones; table: a.cinv, whose
+// row of a position holds a word for four coefficients in zigzag order: a lane takes eight of them.
+// int16 coefficients of any value make the sum of the |n_j| at most 2^22, so 40 fraction bits fit.
+// Of a channel-block with kBlockTies marked pixels or more (flat ones, a half level off, have 64), the
+// whole warp decides 32 at a time, a pixel a lane, and passes over coefficients that are zero (turns
+// alone: 1316 us for DC-only blocks).  From 6 or 8 on it was slower where blocks are not sparse: public
+// image of random rectangles 24.6 -> 26.5 and 27.1 us.
+constexpr int kPixFrac = 40;
+constexpr int kBlockTies = 16;
 template <bool PUBIMG, bool STAGED = false>
-__device__ __forceinline__ void decide_pixels(uint32_t mlo, uint32_t mhi, const int16_t* pub_g, const int16_t* priv_cb, int k,
-                                              const uint4* ctab, const uint8_t* uv, int lane, WarpSlot* slot, uint8_t* out) {
-  // near ties, one after another, decided by the whole warp
-  for (uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0); who; who &= who - 1) {
-    const int src = __ffs(who) - 1;
-    uint64_t mask = (uint64_t)__shfl_sync(0xffffffffu, mhi, src) << 32 | __shfl_sync(0xffffffffu, mlo, src);
-    const int16_t* pub_s = pub_g + (uint64_t)src * (63 - k);
-    const int16_t* priv_s = priv_cb + (src - lane) * (k + 1);
-    if (lane == 0) slot->ties += __popcll(mask);
-    for (; mask; mask &= mask - 1) {
-      const int pos = __ffsll((long long)mask) - 1;
-      const int p = round_warp_inv<PUBIMG, STAGED>(pub_s, priv_s, k, pos, ctab, uv, lane, slot);
-      if (lane == src) out[(pos >> 3) * kRPitch + 3 * (pos & 7)] = (uint8_t)(p < 0 ? 0 : (p > 255 ? 255 : p));
+__device__ __forceinline__ void decide_pixels(uint32_t mlo, uint32_t mhi, const int16_t* pub_g, const int16_t* priv0, int k,
+                                              const uint32_t* table, int lane, WarpSlot* slot, uint8_t* pix,
+                                              const uint8_t* out) {
+  uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
+  if (__builtin_expect(who == 0, 1)) return;
+  // read here, so that what depends on it is not kept through the subtiles without near ties
+  asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+  int esc = 0;
+  bool fail = false;
+  const int nties = (int)__reduce_add_sync(0xffffffffu, (uint32_t)(__popc(mlo) + __popc(mhi)));
+  const uint32_t at = (uint32_t)(out - pix);
+  const long long cos_l = group_cos<kPixFrac>(lane);
+  const int l = lane & 7;
+  auto coef = [&](const int16_t* pub, const int16_t* priv, int z) -> int {
+    return z <= k ? (PUBIMG ? (z == 0 ? 1024 : 0) : priv[z]) : (STAGED ? pub[z - k - 1] : __ldg(pub + z - k - 1));
+  };
+  auto put = [&](uint32_t to, int pos, int p) {
+    pix[to + (pos >> 3) * kRPitch + 3 * (pos & 7)] = (uint8_t)(p < 0 ? 0 : (p > 255 ? 255 : p));
+  };
+  for (uint32_t many = __ballot_sync(0xffffffffu, __popc(mlo) + __popc(mhi) >= kBlockTies); many; many &= many - 1) {
+    const int src = __ffs(many) - 1;
+    const uint32_t to = __shfl_sync(0xffffffffu, at, src);
+    const int16_t* pub = pub_g + src * (63 - k);
+    const int16_t* priv = priv0 + src * (k + 1);
+    const uint32_t Q = __byte_perm((uint32_t)coef(pub, priv, 2 * lane), (uint32_t)coef(pub, priv, 2 * lane + 1), 0x5410u);
+    const uint32_t used = __ballot_sync(0xffffffffu, Q != 0);
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      const bool on = (__shfl_sync(0xffffffffu, h ? mhi : mlo, src) >> lane) & 1u;
+      int n[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+      for (uint32_t m = used; m;) {        // four coefficients at a time
+        const int t = (__ffs(m) - 1) >> 1;
+        m &= ~(3u << (2 * t));
+        const uint32_t q0 = __shfl_sync(0xffffffffu, Q, 2 * t), q1 = __shfl_sync(0xffffffffu, Q, 2 * t + 1);
+        const uint32_t* w = table + 64 * 128 + 512 * t + 32 * h + lane;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t x = __ldg(w + 64 * j);
+          n[j] = dp2a_hi(q1, x, dp2a_lo(q0, x, n[j]));
+        }
+      }
+      bool sure;
+      const int p = round_lane<kPixFrac>(n, sure);
+      if (on) put(to, 32 * h + lane, p);
+      const uint32_t left = __ballot_sync(0xffffffffu, on && !sure);
+      if (lane == src) (h ? mhi : mlo) = left;
     }
+  }
+  who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
+  while (who) {
+    const TieTurn t = take_ties(who, mlo, mhi, lane);
+    const uint32_t to = __shfl_sync(0xffffffffu, at, t.src);
+    int n[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (t.on) {
+      const uint2* w2 = reinterpret_cast<const uint2*>(table + t.pos * 128) + l;
+      const int16_t* pub = pub_g + t.src * (63 - k);
+      const int16_t* priv = priv0 + t.src * (k + 1);
+      uint32_t Q[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        int q[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) q[h] = coef(pub, priv, 8 * l + 2 * i + h);
+        Q[i] = __byte_perm((uint32_t)q[0], (uint32_t)q[1], 0x5410u);
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const uint2 w = __ldg(w2 + 8 * j);
+        n[j] = dp2a_hi(Q[3], w.y, dp2a_lo(Q[2], w.y, dp2a_hi(Q[1], w.x, dp2a_lo(Q[0], w.x, 0))));
+      }
+    }
+    const int p = round_group<kPixFrac, 1 << 22>(group_sum(n, lane), cos_l, t.on, lane, esc, fail);
+    if (t.on && l == 0) put(to, t.pos, p);
+    who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
+  }
+  if (lane == 0) {
+    slot->ties += nties;
+    if (esc | fail) slot->esc += esc, slot->fail |= fail;
   }
 }
 
@@ -267,8 +285,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
   uint64_t* const bars = reinterpret_cast<uint64_t*>(area + kRBar);
   uint32_t* wins = reinterpret_cast<uint32_t*>(smem_cta + (kRWin - win0));
   uint32_t* const next = wins + 5 * kWins;
-  uint4* const ctab = reinterpret_cast<uint4*>(next + 4);
-  uint8_t* const uv = reinterpret_cast<uint8_t*>(ctab + 32);
   const int k = K >= 0 ? K : a.k;
   const int npub = 63 - k;
   const uint32_t nb = 4u * (uint32_t)(k + 1);       // keystream blocks per subtile
@@ -344,12 +360,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
     }
   }
   if (threadIdx.x == 0) *next = own ? sfree : s0 + act;
-  if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
-    const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
-    const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
-    ctab[lane] = make_uint4(f >> 1 == 0 ? one : 0u, f >> 1 == 1 ? one : 0u, f >> 1 == 2 ? one : 0u, f >> 1 == 3 ? one : 0u);
-  }
-  if (threadIdx.x < 64) uv[zigzag_of((int)threadIdx.x >> 3, (int)threadIdx.x & 7)] = (uint8_t)threadIdx.x;
   if (cipher) fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
   __syncthreads();
   if (cipher) {
@@ -431,7 +441,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
       uint8_t* const out = pix + 8 * (c0 + lane - at.c) + at.c;
       uint32_t mlo, mhi;
       emit_rows(G2, l1, lane < n, out, mlo, mhi);
-      decide_pixels<PUBIMG>(mlo, mhi, a.pub_in + (uint64_t)(32u * t) * npub, priv_cb, k, ctab, uv, lane, slot, out);
+      decide_pixels<PUBIMG>(mlo, mhi, a.pub_in + (uint64_t)(32u * t) * npub, priv_cb - lane * (k + 1), k, a.cinv, lane, slot, pix,
+                            out);
       if (!PUBIMG && !twice) fence_proxy_async();
       __syncwarp();                        // the pixel rows are complete
       if (!PUBIMG && !twice && ti + 1 == cnt && run_n < s1) load_priv(run_n, cnt_n, 0);
@@ -468,8 +479,8 @@ constexpr int kUArea = (kUSlot + 32 + 31) & ~31;
 constexpr int kUBelow = ((int)kTpairWin - 1024) / kUArea;
 constexpr int kULow = (int)kTpairWin - kUBelow * kUArea;
 constexpr int kUAbove = kWarps > kUBelow ? kWarps - kUBelow : 0;
-constexpr int kUTail = (int)kTpairWin + kTpairBytes + kUAbove * kUArea;   // folded c(m), (u, v) by zigzag
-constexpr int kUEnd = kUTail + 512 + 64;
+constexpr int kUTail = (int)kTpairWin + kTpairBytes + kUAbove * kUArea;
+constexpr int kUEnd = kUTail;
 static_assert(kUEnd <= 227 * 1024 && kUSlot % 8 == 0, "packed restore shared memory");
 
 template <int W>
@@ -576,8 +587,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_packed_kernel(const __
   uint8_t* const pix = area + kUPix;
   uint64_t* const bars = reinterpret_cast<uint64_t*>(area + kUBar);
   WarpSlot* const slot = reinterpret_cast<WarpSlot*>(area + kUSlot);
-  uint4* const ctab = reinterpret_cast<uint4*>(smem_cta + (kUTail - win0));
-  uint8_t* const uv = reinterpret_cast<uint8_t*>(ctab + 32);
   const int k = K >= 0 ? K : a.k;
   const int npub = 63 - k, period = kDcBits + k * W;
   const uint32_t pub_per = 4u * (uint32_t)(npub * W), priv_per = 4u * (uint32_t)period;
@@ -620,12 +629,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_packed_kernel(const __
     skew_pub = load_pub(t0);
     skew_priv = load_priv(t0);
   }
-  if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
-    const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
-    const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
-    ctab[lane] = make_uint4(f >> 1 == 0 ? one : 0u, f >> 1 == 1 ? one : 0u, f >> 1 == 2 ? one : 0u, f >> 1 == 3 ? one : 0u);
-  }
-  if (threadIdx.x < 64) uv[zigzag_of((int)threadIdx.x >> 3, (int)threadIdx.x & 7)] = (uint8_t)threadIdx.x;
   fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
   __syncthreads();
 
@@ -689,7 +692,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_packed_kernel(const __
     uint8_t* const out = pix + 8 * (c0 + lane - at.c) + at.c;
     uint32_t mlo, mhi;
     emit_rows(G2, l1, lane < n, out, mlo, mhi);
-    decide_pixels<false, true>(mlo, mhi, pubst, priv_cb, k, ctab, uv, lane, slot, out);
+    decide_pixels<false, true>(mlo, mhi, pubst, privst, k, a.cinv, lane, slot, pix, out);
     __syncwarp();                          // the pixel rows are complete
     store_pixels(a.pixels_out, 3ull * (uint64_t)a.width, at, c0, n, lane, pix);
     __syncwarp();                          // the staging area and the pixel buffer may be written again
@@ -735,8 +738,8 @@ constexpr int kQArea = (kQWins + 40 + 31) & ~31;
 constexpr int kQBelow = ((int)kTpairWin - 1024) / kQArea;
 constexpr int kQLow = (int)kTpairWin - kQBelow * kQArea;
 constexpr int kQAbove = kWarps > kQBelow ? kWarps - kQBelow : 0;
-constexpr int kQTail = (int)kTpairWin + kTpairBytes + kQAbove * kQArea;   // counter, folded c(m), (u, v) by zigzag
-constexpr int kQEnd = kQTail + 16 + 512 + 64;
+constexpr int kQTail = (int)kTpairWin + kTpairBytes + kQAbove * kQArea;   // counter
+constexpr int kQEnd = kQTail + 16;
 static_assert(kQEnd <= 227 * 1024, "restore (batches) shared memory");
 
 // by k: run_tiles (at most a tile), and 16 where two runs fit
@@ -774,8 +777,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
   PlanSlot* const slots = reinterpret_cast<PlanSlot*>(area + kQSlot);
   uint32_t* const wins = reinterpret_cast<uint32_t*>(area + kQWins);
   uint32_t* const next = reinterpret_cast<uint32_t*>(smem_cta + (kQTail - win0));
-  uint4* const ctab = reinterpret_cast<uint4*>(next + 4);
-  uint8_t* const uv = reinterpret_cast<uint8_t*>(ctab + 32);
   const int act = a.groups;
   PlanClaim claim(a, act);
   auto nof = [&](const PlanSlot* s, uint32_t t) { return (int)min(32u, s->ncb - 32u * t); };
@@ -813,12 +814,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
       load_pub(s, r);
     }
   }
-  if (threadIdx.x < 32) {                  // c(m) = +-c(j), as +-1 in field j
-    const int m = lane <= 16 ? lane : 32 - lane, f = m > 8 ? 16 - m : m;
-    const uint32_t one = (f & 1 ? 0x10000u : 1u) * (m > 8 ? 0xffffffffu : 1u);
-    ctab[lane] = make_uint4(f >> 1 == 0 ? one : 0u, f >> 1 == 1 ? one : 0u, f >> 1 == 2 ? one : 0u, f >> 1 == 3 ? one : 0u);
-  }
-  if (threadIdx.x < 64) uv[zigzag_of((int)threadIdx.x >> 3, (int)threadIdx.x & 7)] = (uint8_t)threadIdx.x;
   fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
   __syncthreads();
   if (warp >= act) return;
@@ -880,8 +875,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
       uint8_t* const out = pix + 8 * (c0 + lane - at.c) + at.c;
       uint32_t mlo, mhi;
       emit_rows(G2, l1, lane < m, out, mlo, mhi);
-      decide_pixels<false>(mlo, mhi, reinterpret_cast<const int16_t*>(s->pub) + (uint64_t)(32u * t) * npub, priv_cb, k, ctab, uv,
-                           lane, slot, out);
+      decide_pixels<false>(mlo, mhi, reinterpret_cast<const int16_t*>(s->pub) + (uint64_t)(32u * t) * npub, priv_cb - lane * (k + 1),
+                           k, a.cinv, lane, slot, pix, out);
       if (ti + 1 == cnt && have && !(twice && pipe)) fence_proxy_async();
       __syncwarp();                        // the pixel rows are complete
       if (ti + 1 == cnt && have && !(twice && pipe)) {

@@ -352,21 +352,23 @@ __device__ __forceinline__ void coords_fwd(const uint8_t* tile, int b, int c, in
   coords_from_pixels(P, pos, table, n);
 }
 
-// the same from the image in global memory: blk = the block's top-left pixel (8-byte
-// aligned), row = bytes per image row
+// the eight pixels of channel c of a block's row in global memory (8-byte aligned), as row_pixels
+__device__ __forceinline__ void pixel_row_global(const uint8_t* row, int c, uint32_t& lo, uint32_t& hi) {
+  const uint2* rp = reinterpret_cast<const uint2*>(row);
+  const uint2 w01 = __ldg(rp), w23 = __ldg(rp + 1), w45 = __ldg(rp + 2);
+  const uint32_t r[7] = {w01.x, w01.y, w23.x, w23.y, w45.x, w45.y, 0u};
+  uint32_t w[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) w[i] = __funnelshift_r(r[i], r[i + 1], 8 * c);
+  row_pixels(w, lo, hi);
+}
+// coords_fwd from the image in global memory: blk = the block's top-left pixel, row = bytes per image
+// row
 __device__ __forceinline__ void coords_fwd_global(const uint8_t* blk, uint64_t row, int c, int pos,
                                                   const uint32_t* table, int (&n)[9]) {
   uint32_t P[16];
 #pragma unroll
-  for (int y = 0; y < 8; ++y) {
-    const uint2* rp = reinterpret_cast<const uint2*>(blk + y * row);
-    const uint2 w01 = __ldg(rp), w23 = __ldg(rp + 1), w45 = __ldg(rp + 2);
-    const uint32_t r[7] = {w01.x, w01.y, w23.x, w23.y, w45.x, w45.y, 0u};
-    uint32_t w[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) w[i] = __funnelshift_r(r[i], r[i + 1], 8 * c);
-    row_pixels(w, P[2 * y], P[2 * y + 1]);
-  }
+  for (int y = 0; y < 8; ++y) pixel_row_global(blk + y * row, c, P[2 * y], P[2 * y + 1]);
   coords_from_pixels(P, pos, table, n);
 }
 

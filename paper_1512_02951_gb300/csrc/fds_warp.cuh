@@ -116,6 +116,145 @@ __device__ __forceinline__ void put_window(const TileArgs& a, uint64_t q, int sl
   }
 }
 
+// ---- near ties: the marked values of a subtile (bit pos of a lane's mhi:mlo), decided exactly four at
+// a time, each by a group of eight lanes.  Eight times the value is n_0 + sum n_j c(j) (fds_device.cuh);
+// a lane takes an eighth of the block and of the coordinate table's row (dot products of packed
+// bytes), a transposing sum leaves lane j of the group with n_j, and the eight products with c(j) in
+// 64-bit fixed point are summed again.  Where many lanes (protect) or many values of one lane (restore)
+// are marked, a lane takes a whole value: a pass of the warp then decides up to 32, for the price of
+// two to four turns.  What bounds it is issue where ties are many and the chain of a turn (loads from
+// L2, three exchanges, twice) where one block has many.  A whole warp for each value, as before, made
+// content with many near ties slow; 2048 x 2048, k = 5, us: protect of black and white noise 57.9 ->
+// 33.1, of a slow ramp 81.6 -> 44.1, of a block of four ties repeated 303 -> 37.5; the public image of
+// text 48.6 -> 21.0; restore of DC-only blocks half a level off (every pixel a tie, k = 0) 3457 -> 124;
+// smooth scenes with ten ties a thousand channel-blocks 21.1 -> 20.8 and 24.3 -> 22.9.
+
+// zigzag index by position 8 u + v
+struct ZigzagTable {
+  uint8_t z[64];
+};
+constexpr ZigzagTable make_zigzag_table() {
+  ZigzagTable t{};
+  for (int i = 0; i < 64; ++i) t.z[i] = (uint8_t)zigzag_of(i >> 3, i & 7);
+  return t;
+}
+static __constant__ ZigzagTable c_zigzag = make_zigzag_table();
+
+// The value that the lane's group takes this turn: of lane src, at pos (on: there is one).  who: the
+// lanes that have marked values, which drop those taken: one of each of the first four lanes, or two
+// of each of two, or four of one.
+struct TieTurn {
+  int src, pos;
+  bool on;
+};
+__device__ __forceinline__ void drop_lowest(uint32_t& lo, uint32_t& hi) {
+  if (lo)
+    lo &= lo - 1;
+  else
+    hi &= hi - 1;
+}
+__device__ __forceinline__ TieTurn take_ties(uint32_t who, uint32_t& mlo, uint32_t& mhi, int lane) {
+  const int m = __popc(who), g = lane >> 3;
+  TieTurn t;
+  int skip = 0, taken = 0;                 // of src's values, for the groups before; of the lane's own
+  bool on = true;
+  if (m > 2) {
+    uint32_t w = who;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      if (i < g) w &= w - 1;
+    on = w != 0;
+    t.src = (__ffs(w) - 1) & 31;
+    taken = __popc(who & ((1u << lane) - 1u)) < 4 ? 1 : 0;
+  } else {
+    t.src = m == 2 && g & 1 ? 31 - __clz(who) : __ffs(who) - 1;
+    skip = m == 2 ? g >> 1 : g;
+    taken = m == 2 ? 2 : 4;
+  }
+  uint32_t lo = __shfl_sync(0xffffffffu, mlo, t.src), hi = __shfl_sync(0xffffffffu, mhi, t.src);
+  for (int i = 0; i < skip && (lo | hi); ++i) drop_lowest(lo, hi);
+  t.on = on && (lo | hi) != 0;
+  t.pos = t.on ? (lo ? __ffs(lo) - 1 : __ffs(hi) + 31) : 0;
+  for (int i = 0; i < taken && (mlo | mhi); ++i) drop_lowest(mlo, mhi);
+  return t;
+}
+
+// the sum over the lane's group of n[l], l the lane's place in it
+__device__ __forceinline__ int group_sum(const int (&n)[8], int lane) {
+  int a[4], b[2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    a[i] = (lane & 4 ? n[i + 4] : n[i]) + __shfl_xor_sync(0xffffffffu, lane & 4 ? n[i] : n[i + 4], 4);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    b[i] = (lane & 2 ? a[i + 2] : a[i]) + __shfl_xor_sync(0xffffffffu, lane & 2 ? a[i] : a[i + 2], 2);
+  return (lane & 1 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, lane & 1 ? b[0] : b[1], 1);
+}
+
+// exact_round of the values of the groups that fixed point could not decide, in their first lanes; q:
+// the others' results
+static __device__ __noinline__ int round_far(int n_l, bool far, int q, int lane, int* esc, bool* fail) {
+  int n[9], e = 0;
+  bool f = false;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) n[j] = __shfl_sync(0xffffffffu, n_l, (lane & 24) + j);
+  n[8] = 0;
+  if (far && (lane & 7) == 0) q = exact_round(n, &e, &f);
+  *esc += __popc(__ballot_sync(0xffffffffu, e != 0));
+  *fail |= (bool)__any_sync(0xffffffffu, f);
+  return q;
+}
+
+// c(l) with FRAC fraction bits, l the lane's place in its group
+template <int FRAC>
+__device__ __forceinline__ long long group_cos(int lane) {
+  const int l = lane & 7;
+  return l ? c_cos_q62[l - 1] >> (62 - FRAC) : 1ll << FRAC;
+}
+
+// A value alone in its lane, all its coordinates at hand: the same in one lane.  sure: decided; else too
+// near a boundary for fixed point (left to a group)
+template <int FRAC>
+__device__ __forceinline__ int round_lane(const int (&n)[8], bool& sure) {
+  long long d = ((long long)n[0] + 4) << FRAC;
+  int err = 0;
+#pragma unroll
+  for (int j = 1; j < 8; ++j) {
+    d += n[j] * (c_cos_q62[j - 1] >> (62 - FRAC));
+    err += abs(n[j]);
+  }
+  const int q = (int)(d >> (FRAC + 3));
+  const long long rem = d & ((8ll << FRAC) - 1);
+  sure = err == 0 || (rem > err && rem < (8ll << FRAC) - err);
+  return err == 0 && rem == 0 && q <= 0 ? q - 1 : q;
+}
+
+// Rounds, half away from zero, the value of the lane's group whose eightfold has the coordinates n_l
+// (one a lane; on: there is one); the result is the group's first lane's.  Each c(j) 2^FRAC is within a
+// unit, so the sum is within sum |n_j| <= BOUND units.  Nearer than that to a boundary it is a tie if it
+// is rational (about half of all near ties of protect: positions whose u and v are 2 or 6), and else
+// left to exact_round.
+template <int FRAC, int BOUND>
+__device__ __forceinline__ int round_group(int n_l, long long cos_l, bool on, int lane, int& esc, bool& fail) {
+  const bool rational = ((__ballot_sync(0xffffffffu, (lane & 7) && n_l != 0) >> (lane & 24)) & 0xffu) == 0;
+  long long d = n_l * cos_l;
+#pragma unroll
+  for (int i = 1; i < 8; i <<= 1) d += __shfl_xor_sync(0xffffffffu, d, i);
+  d += 4ll << FRAC;                        // d / 2^(FRAC + 3) = the value + 1/2
+  int q = (int)(d >> (FRAC + 3));
+  const long long rem = d & ((8ll << FRAC) - 1);
+  if (rational && rem == 0 && q <= 0) --q;
+  const bool far = on && !rational && (rem <= BOUND || rem >= (8ll << FRAC) - BOUND);
+  if (__any_sync(0xffffffffu, far)) {
+    int e = 0;
+    bool f = false;
+    q = round_far(n_l, far, q, lane, &e, &f);
+    esc += e;
+    fail |= f;
+  }
+  return q;
+}
+
 // ---- batches: what a warp knows about the image of a tile it works on (shared memory; two per
 // warp, the tile's and the next one's)
 struct PlanSlot {
