@@ -369,14 +369,29 @@ __device__ __forceinline__ uint32_t tpair(uint32_t w, uint32_t lc) {
 }
 // Fill the pair table at `tab` (shared memory, window address kTpairWin) from T0 in global
 // memory (256 words): threads t = 0 .. nthreads - 1 of the CTA; a barrier must follow
-__device__ __forceinline__ void fill_pair_table(uint8_t* tab, const uint32_t* T0, int t, int nthreads) {
-  for (int i = t; i < 2048; i += nthreads) {
-    const int x = i >> 3, m = i & 7;
-    const uint32_t t0 = __ldg(T0 + x), t2 = __byte_perm(t0, t0, 0x1032u);
-    reinterpret_cast<uint4*>(tab + 256 * x)[m] = make_uint4(t0, t0, t0, t0);
-    reinterpret_cast<uint4*>(tab + 256 * x + 128)[m] = make_uint4(t2, t2, t2, t2);
-  }
+__device__ __forceinline__ void put_pair_entry(uint8_t* tab, int i, uint32_t t0) {
+  const int x = i >> 3, m = i & 7;
+  const uint32_t t2 = __byte_perm(t0, t0, 0x1032u);
+  reinterpret_cast<uint4*>(tab + 256 * x)[m] = make_uint4(t0, t0, t0, t0);
+  reinterpret_cast<uint4*>(tab + 256 * x + 128)[m] = make_uint4(t2, t2, t2, t2);
 }
+__device__ __forceinline__ void fill_pair_table(uint8_t* tab, const uint32_t* T0, int t, int nthreads) {
+  for (int i = t; i < 2048; i += nthreads) put_pair_entry(tab, i, __ldg(T0 + (i >> 3)));
+}
+// the same in two steps, for N threads: the loads, then the stores
+template <int N>
+struct PairFill {
+  static constexpr int kPer = 2048 / N;
+  uint32_t v[kPer];
+  __device__ __forceinline__ void load(const uint32_t* T0, int t) {
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) v[r] = __ldg(T0 + ((t + r * N) >> 3));
+  }
+  __device__ __forceinline__ void store(uint8_t* tab, int t) const {
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) put_pair_entry(tab, t + r * N, v[r]);
+  }
+};
 __device__ __forceinline__ void aes128_encrypt_pair(uint32_t (&s)[4], const uint32_t* rk, PairLanes lc) {
   auto r8 = [](uint32_t x) { return __byte_perm(x, x, 0x2103u); };
   uint32_t s0 = s[0] ^ rk[0], s1 = s[1] ^ rk[1], s2 = s[2] ^ rk[2], s3 = s[3] ^ rk[3];

@@ -758,7 +758,10 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
   uint32_t* const wins = reinterpret_cast<uint32_t*>(area + kPWins);
   uint32_t* const next = reinterpret_cast<uint32_t*>(smem_cta + (kPTail - win0));
   const int act = a.groups;
+  PairFill<kWarps * 32> fill;
+  fill.load(a.T, (int)threadIdx.x);
   PlanClaim claim(a, act);
+  PlanKeys keys;
   Loads ld;
   // subtile t of slot s starts loading; bulk: by bulk copies (they complete on the mbarrier)
   auto load = [&](const PlanSlot* s, uint32_t t, bool& bulk) {
@@ -788,15 +791,17 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __gr
   PlanSlot *s = slots, *sn = slots + 1;
   PixAt at{};
   if (warp < act) {                        // the first run starts loading before the tables are filled
-    claim(a, act, next, s, s, c_acc.n, warp, lane, t, end);
+    claim(a, act, next, s, s, c_acc.n, warp, lane, t, end, keys);
     if (t < end) at = load(s, t, bulk);
   }
-  fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
+  fill.store(smem_cta + (kTpairWin - win0), (int)threadIdx.x);
+  put_keys(s, keys, lane);
   __syncthreads();
   if (warp >= act) return;
 
   while (t < end && !lost) {
-    claim(a, act, next, sn, s, c_acc.n, warp, lane, tn, endn);
+    claim(a, act, next, sn, s, c_acc.n, warp, lane, tn, endn, keys);
+    put_keys(sn, keys, lane);
     const int k = K >= 0 ? K : s->k, npub = 63 - k;
     const int G = s->acc;
     uint8_t* const privst = stage + kWCb * 2 * npub;

@@ -778,7 +778,10 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
   uint32_t* const wins = reinterpret_cast<uint32_t*>(area + kQWins);
   uint32_t* const next = reinterpret_cast<uint32_t*>(smem_cta + (kQTail - win0));
   const int act = a.groups;
+  PairFill<kWarps * 32> fill;
+  fill.load(a.T, (int)threadIdx.x);
   PlanClaim claim(a, act);
+  PlanKeys keys;
   auto nof = [&](const PlanSlot* s, uint32_t t) { return (int)min(32u, s->ncb - 32u * t); };
   Loads ld;                                // barrier 0: public, 1 and 2: the private buffers
   auto load_pub = [&](const PlanSlot* s, uint32_t t) {
@@ -808,13 +811,14 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
   uint32_t r = 0, end = 0;                 // the run's first subtile, the end of what was claimed
   int half = 0;
   if (warp < act) {                        // the first run starts loading before the tables are filled
-    claim(a, act, next, s, s, c_run.n, warp, lane, r, end);
+    claim(a, act, next, s, s, c_run.n, warp, lane, r, end, keys);
     if (r < end) {
       load_priv(s, r, min(s->acc & 15, (int)(end - r)), 0);
       load_pub(s, r);
     }
   }
-  fill_pair_table(smem_cta + (kTpairWin - win0), a.T, (int)threadIdx.x, kWarps * 32);
+  fill.store(smem_cta + (kTpairWin - win0), (int)threadIdx.x);
+  put_keys(s, keys, lane);
   __syncthreads();
   if (warp >= act) return;
 
@@ -827,7 +831,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __gr
     uint32_t rn = r + cnt, endn = end;
     if (rn >= end) {
       n = sx;
-      claim(a, act, next, n, s, c_run.n, warp, lane, rn, endn);
+      claim(a, act, next, n, s, c_run.n, warp, lane, rn, endn, keys);
+      put_keys(n, keys, lane);
     }
     const bool have = rn < endn, pipe = have && (K >= 0 || n->k == k);
     const int cntn = have ? min(n->acc & 15, (int)(endn - rn)) : 0;

@@ -269,10 +269,24 @@ struct PlanSlot {
 static_assert(sizeof(PlanSlot) % 8 == 0, "PlanSlot");
 constexpr int kTileSubs = kTileCb / kWCb;         // subtiles of a 64-block tile
 
-// The image of tile g into slot s (the whole warp; acc_of: subtiles between two AES phases by k);
-// hint: a slot whose image it often is; returns the tile's index in the image
+// Round keys on their way from global memory into a slot (a lane's two words)
+struct PlanKeys {
+  uint32_t lo, hi;
+  bool due = false;
+};
+__device__ __forceinline__ void put_keys(PlanSlot* s, PlanKeys& keys, int lane) {
+  if (!keys.due) return;
+  s->rk[lane] = keys.lo;
+  if (lane < 12) s->rk[32 + lane] = keys.hi;
+  keys.due = false;
+  __syncwarp();
+}
+
+// The image of tile g into slot s (the whole warp; acc_of: subtiles between two AES phases by k), but
+// for its round keys, which put_keys stores; hint: a slot whose image it often is; returns the tile's
+// index in the image
 __device__ __forceinline__ int plan_slot(const TileArgs& a, int g, PlanSlot* s, const PlanSlot* hint, const uint8_t* acc_of,
-                                         int lane) {
+                                         int lane, PlanKeys& keys) {
   uint32_t im = hint->image;
   if (!(im < (uint32_t)a.n_images && __ldg(a.tile_start + im) <= g && g < __ldg(a.tile_start + im + 1))) {
     int lo = 0, hi = a.n_images;                 // tile_start[lo] <= g < tile_start[hi]
@@ -289,8 +303,10 @@ __device__ __forceinline__ int plan_slot(const TileArgs& a, int g, PlanSlot* s, 
   __syncwarp();
   if (other) {
     const BatchImage& b = a.images[im];
-    const int slot = b.key_slot;
-    for (int i = lane; i < 44; i += 32) s->rk[i] = __ldg(a.round_keys + 44 * slot + i);
+    const uint32_t* rk = a.round_keys + 44 * b.key_slot;
+    keys.lo = __ldg(rk + lane);
+    keys.hi = lane < 12 ? __ldg(rk + 32 + lane) : 0u;
+    keys.due = true;
     if (lane == 0) {
       s->px = const_cast<uint8_t*>(a.pixels_in ? a.pixels_in : a.pixels_out) + b.pixel_offset;
       s->pub = reinterpret_cast<uint8_t*>(a.pub_in ? const_cast<int16_t*>(a.pub_in) : a.pub_out) + b.public_offset;
@@ -318,11 +334,17 @@ __device__ __forceinline__ int plan_slot(const TileArgs& a, int g, PlanSlot* s, 
 // end together: with all but the last whole, 12 tiles a CTA left warps idle for a whole tile (30
 // images of mixed k, protect 56.0 -> 49.3 us, restore 61.8 -> 56.5).  A warp's first run is its own,
 // so that it starts loading before the CTA's tables are filled; the others come from `next`, which
-// starts at act and is set before any claim (a first run may be an empty one).  Or (a.dispenser)
-// every warp takes tiles from one counter.
+// starts at act and is set before any claim (a first run may be an empty one).  A CTA with no more
+// units than warps has nothing behind the first runs, and does not ask (batches of a few hundred
+// tiles, below).  Or (a.dispenser) every warp takes tiles from one counter.
+// A call of one round of units is a chain in one warp, about 17,000 cycles long (restore, k = 0, a few
+// hundred tiles).  The AES table's entries are on their way from the kernel's start and stored while the
+// first run's parts and keys are still coming, and nothing is claimed where nothing is left: restore of
+// eight images, k = 0, 14.3 -> 12.3 us and 28.7 -> 26.9 (12.3 and 28.6 before the warp form), protect
+// 26.4 -> 24.7 (25.6); of thirty images of mixed k 56.1 -> 55.0 and 48.0 -> 46.7.
 struct PlanClaim {
   int g0, g1, whole, halves;
-  bool first;
+  bool first, more;
 
   __device__ __forceinline__ PlanClaim(const TileArgs& a, int act) {
     g0 = (int)((int64_t)a.total_tiles * blockIdx.x / gridDim.x);
@@ -331,10 +353,12 @@ struct PlanClaim {
     whole = rest / act * act;
     halves = rest - whole;
     first = true;
+    more = a.dispenser != nullptr || whole + 2 * halves + kTileSubs * (g1 - g0 - whole - halves) > act;
   }
   __device__ __forceinline__ void operator()(const TileArgs& a, int act, uint32_t* next, PlanSlot* s, const PlanSlot* hint,
-                                             const uint8_t* acc_of, int warp, int lane, uint32_t& t, uint32_t& end) {
-    for (;;) {
+                                             const uint8_t* acc_of, int warp, int lane, uint32_t& t, uint32_t& end,
+                                             PlanKeys& keys) {
+    while (first || more) {
       uint32_t u = 0;
       if (a.dispenser == nullptr) {
         if (first)
@@ -366,7 +390,7 @@ struct PlanClaim {
         g += g0;
         if (g >= g1) break;
       }
-      const int local = plan_slot(a, g, s, hint, acc_of, lane);
+      const int local = plan_slot(a, g, s, hint, acc_of, lane, keys);
       t = (uint32_t)(local * kTileSubs + sub);
       end = min(t + len, (s->ncb + 31u) >> 5);
       if (t < end) return;
