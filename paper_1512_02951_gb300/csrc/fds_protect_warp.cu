@@ -140,13 +140,13 @@ __device__ __forceinline__ PixAt load_subtile(const uint8_t* img, uint64_t pitch
   return at;
 }
 
-// AES-128-CTR over the private parts of n staged subtiles (list[0 .. n - 1]; nb = 4 (k + 1)
-// keystream blocks each); wc: the constants of the windows from wbase on
-__device__ __forceinline__ void ctr_warp(const TileArgs& a, uint8_t* buf, const uint32_t* list, int n, uint32_t nb,
+// AES-128-CTR over the first `total` keystream blocks of staged private parts (subtiles list[0 ..],
+// nb = 4 (k + 1) blocks each); wc: the constants of the windows from wbase on
+__device__ __forceinline__ void ctr_warp(const TileArgs& a, uint8_t* buf, const uint32_t* list, uint32_t total, uint32_t nb,
                                          const uint32_t* wc, uint64_t wbase, int lane) {
   const PairLanes lc = pair_lanes();
 #pragma unroll 1
-  for (uint32_t i = lane; i < n * nb; i += 32) {
+  for (uint32_t i = lane; i < total; i += 32) {
     const uint32_t j = i / nb;
     const uint64_t b = (a.iv_lo & 255u) + (uint64_t)list[j] * nb + (i - j * nb);   // from the IV's window
     const uint32_t* src = wc + 5 * (uint32_t)((b >> 8) - wbase);
@@ -688,7 +688,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
             __syncwarp();
           }
         }
-        ctr_warp(a, privst, list, acc, nb, wins, wbase, lane);
+        // the image's last, short subtile, if it is among them, was claimed last
+        ctr_warp(a, privst, list, (acc - 1) * nb + ((n * 2 * (k + 1) + 15) >> 4), nb, wins, wbase, lane);
         fence_proxy_async();
         __syncwarp();
       }

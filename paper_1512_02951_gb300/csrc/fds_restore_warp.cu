@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
       __syncwarp();
       if (cipher) {
         uint8_t* const buf = privst + half * priv_half;
-        const uint32_t total = (uint32_t)cnt * nb;
+        const uint32_t total = (uint32_t)(((cnt - 1) * 32 + nof(run + cnt - 1)) * 2 * (k + 1) + 15) >> 4;
         const uint64_t b0 = iv8 + (uint64_t)run * nb;     // from the IV's window
         uint64_t wbase = slot->wbase;
         if (!table && ((b0 >> 8) < wbase || ((b0 + total - 1) >> 8) > wbase + 1)) {
