@@ -888,7 +888,7 @@ static cudaError_t launch_w(const TileArgs& a, cudaStream_t s, int sms) {
   const long long nsub = (3ll * a.nblocks + 31) / 32;
   const int grid = (int)(nsub < sms ? nsub : sms);
   const long long per = (nsub + grid - 1) / (grid ? grid : 1);
-  b.groups = (int)(per < kWarps ? per : kWarps);
+  b.groups = PACK ? working_warps(per) : (int)(per < kWarps ? per : kWarps);
   bx_division(b);
   b.aes_pair = PACK == 11 ? pack_acc_tiles<11>(a.k) : (PACK == 8 ? pack_acc_tiles<8>(a.k) : acc_tiles(a.k));
   if (grid > 0) protect_warp_kernel<K, BULK, PACK><<<grid, kWarps * 32, kWEnd, s>>>(b);

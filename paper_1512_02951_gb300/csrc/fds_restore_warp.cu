@@ -722,8 +722,7 @@ static cudaError_t launch_packed(const TileArgs& a, cudaStream_t s, int sms) {
   TileArgs b = a;
   const long long nsub = (3ll * a.nblocks + 31) / 32;
   const int grid = (int)(nsub < sms ? nsub : sms);
-  const long long per = (nsub + grid - 1) / (grid ? grid : 1);
-  b.groups = (int)(per < kWarps ? per : kWarps);
+  b.groups = working_warps((nsub + grid - 1) / (grid ? grid : 1));
   bx_division(b);
   b.aes_pair = run_tiles_packed<W>(a.k);
   if (grid > 0) restore_packed_kernel<K, W><<<grid, kWarps * 32, kUEnd, s>>>(b);

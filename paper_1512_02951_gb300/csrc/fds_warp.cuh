@@ -39,11 +39,13 @@ __device__ __forceinline__ CbPos cb_pos(const TileArgs& a, uint32_t cb) {
 }
 
 // Working warps of a CTA for `per` subtiles an SM.  Up to three warps on a scheduler a round takes
-// the latency of one subtile, the fourth makes it longer; so two rounds of twelve take less than
-// one of sixteen and a short one (restore of 4096 x 512, k = 5, 20 subtiles an SM: 18.4 -> 17.6 us)
+// the latency of one subtile, the fourth makes it longer; so twelve warps take less than sixteen where
+// they need no more rounds (17 .. 24 and 33 .. 36): restore of 4096 x 512, k = 5, 20 subtiles an SM, 18.4
+// -> 17.6 us; packed protect of 20000 x 88, k = 17 (18 an SM), 27.0 -> 25.3, of 2600 x 1400 (36), 8 bits,
+// 39.2 -> 33.7.  Evening the rounds out further (two of fourteen for 28) was slower: 31.3 -> 33.1.
 inline int working_warps(long long per) {
-  if (per > kWarps && per <= 24) return 12;
-  return (int)(per < kWarps ? per : kWarps);
+  if (per <= kWarps) return (int)per;
+  return (per + 11) / 12 == (per + kWarps - 1) / kWarps ? 12 : kWarps;
 }
 
 // block / bx_count as a multiply and a shift, exact for block numbers below 2^31: with l the
