@@ -169,16 +169,16 @@ int fds_plan_set_direction_schedule(fds_plan* plan, int32_t direction, int32_t c
 int fds_plan_get_direction_schedule(const fds_plan* plan, int32_t direction,
                                     int32_t* ctas_per_sm, int32_t* dynamic, int32_t* aes_pair);
 
-/* Time every protect schedule on this batch (tile order x ctas_per_sm 1 .. 4 x dynamic x
- * aes_pair, `reps` launches each after one warm-up, on `stream`) and keep the fastest.  The
+/* Time every protect schedule on this batch (tile order x ctas_per_sm 1 .. 4 x dynamic, `reps`
+ * launches each after one warm-up, on `stream`) and keep the fastest, with aes_pair 0.  The
  * buffers are written to; their previous contents are lost.  Synchronises the device. */
 int fds_plan_autotune(fds_plan* plan, const uint8_t* pixels, int16_t* public_out,
                       uint8_t* private_out, int32_t reps, void* stream);
 
 /* The same for both directions, tuned separately: protect writes public_buf / private_buf,
  * restore reads them and writes pixels_out (all three overwritten).  Each direction keeps
- * its fastest ctas_per_sm / dynamic / aes_pair; the tile order, which the directions share,
- * is the one with the smaller sum of their best times. */
+ * its fastest ctas_per_sm / dynamic, with aes_pair 0; the tile order, which the directions
+ * share, is the one with the smaller sum of their best times. */
 int fds_plan_autotune_directions(fds_plan* plan, const uint8_t* pixels, int16_t* public_buf,
                                  uint8_t* private_buf, uint8_t* pixels_out, int32_t reps,
                                  void* stream);
@@ -187,7 +187,8 @@ int fds_plan_autotune_directions(fds_plan* plan, const uint8_t* pixels, int16_t*
  * caller may store it: "t<a>-T<b>-k<k>", 2^a the median image's tiles of 64 blocks and 2^b
  * the batch's tiles, each rounded up to a power of two, k the uniform k or "mixed"),
  * "largest_first", "protect" and "restore" ({"ctas_per_sm", "dynamic", "aes_pair"}), and
- * "candidates": every schedule the last autotune timed with its mean ms per launch.
+ * "candidates": every schedule the last autotune timed with its mean ms per launch (both
+ * values of aes_pair, which launch the same kernel, with one time).
  * *length (may be NULL) receives the size including the NUL; buf may be NULL to ask for it.
  * FDS_E_INVALID when capacity is smaller than that size. */
 int fds_plan_schedule_json(const fds_plan* plan, char* buf, int64_t capacity, int64_t* length);
