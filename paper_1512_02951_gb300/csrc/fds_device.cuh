@@ -76,23 +76,6 @@ __device__ __forceinline__ void dct8_sd(const float (&s)[4], const float (&d)[4]
   x[7] = fmaf(d[3], -h1, fmaf(d[2], h3, fmaf(d[1], -h5, d[0] * h7)));
 }
 
-template <bool RAT_UNSCALED, bool IRR_LAMBDA>
-__device__ __forceinline__ void dct8(float (&x)[8]) {
-  const float s[4] = {x[0] + x[7], x[1] + x[6], x[2] + x[5], x[3] + x[4]};
-  const float d[4] = {x[0] - x[7], x[1] - x[6], x[2] - x[5], x[3] - x[4]};
-  dct8_sd<RAT_UNSCALED, IRR_LAMBDA>(s, d, x);
-}
-
-// Row pass straight from pixel bytes.  X_i = 2^23 + p_i (a float built from the byte), so
-// d_i = X_i - X_(7-i) = p_i - p_(7-i) and s_i = (X_i - (2^24 + 256)) + X_(7-i) =
-// (p_i - 128) + (p_(7-i) - 128) are exact: the level shift by 128 costs nothing.
-__device__ __forceinline__ void dct8_row_bytes(const float (&X)[8], float (&x)[8]) {
-  constexpr float c2 = 16777472.0f;  // 2^24 + 256
-  const float s[4] = {(X[0] - c2) + X[7], (X[1] - c2) + X[6], (X[2] - c2) + X[5], (X[3] - c2) + X[4]};
-  const float d[4] = {X[0] - X[7], X[1] - X[6], X[2] - X[5], X[3] - X[4]};
-  dct8_sd<true, false>(s, d, x);
-}
-
 // Error weight of one 8-point pass over exact inputs: |d_0| + .. + |d_3| + |f_0| + |f_1| with
 // f_0 = s_0 - s_3, f_1 = s_1 - s_2 (small integers, so the sum is exact).  The rounding error
 // of every irrational output of the pass is at most 2.46 u times this weight (u = 2^-24).
@@ -100,7 +83,10 @@ __device__ __forceinline__ float pass_weight(const float (&s)[4], const float (&
   return ((fabsf(d[0]) + fabsf(d[1])) + (fabsf(d[2]) + fabsf(d[3]))) + (fabsf(s[0] - s[3]) + fabsf(s[1] - s[2]));
 }
 
-// dct8_row_bytes that also returns the row's error weight
+// Row pass straight from pixel bytes.  X_i = 2^23 + p_i (a float built from the byte), so
+// d_i = X_i - X_(7-i) = p_i - p_(7-i) and s_i = (X_i - (2^24 + 256)) + X_(7-i) =
+// (p_i - 128) + (p_(7-i) - 128) are exact: the level shift by 128 costs nothing.
+// Returns the row's error weight.
 __device__ __forceinline__ float dct8_row_bytes_w(const float (&X)[8], float (&x)[8]) {
   constexpr float c2 = 16777472.0f;  // 2^24 + 256
   const float s[4] = {(X[0] - c2) + X[7], (X[1] - c2) + X[6], (X[2] - c2) + X[5], (X[3] - c2) + X[4]};
@@ -146,7 +132,8 @@ __device__ __forceinline__ void dct8_2(float2 (&x)[8]) {
   dct8_sd2<RAT_UNSCALED, IRR_LAMBDA>(s, d, x);
 }
 
-// dct8<true, true> on two exact-integer columns at once; returns the sum of their error weights
+// the column pass of two exact-integer columns at once, IRR_LAMBDA and unscaled; returns the sum of
+// their error weights
 __device__ __forceinline__ float dct8_rat_w2(float2 (&x)[8]) {
   const float2 s[4] = {add2(x[0], x[7]), add2(x[1], x[6]), add2(x[2], x[5]), add2(x[3], x[4])};
   const float2 d[4] = {sub2(x[0], x[7]), sub2(x[1], x[6]), sub2(x[2], x[5]), sub2(x[3], x[4])};
@@ -440,16 +427,6 @@ __device__ __forceinline__ void ctr_block(uint64_t iv_hi, uint64_t iv_lo, uint64
 
 // cos(j pi/16), j = 1..7, to 256 fractional bits (each translation unit holds its own copy)
 static __constant__ uint32_t c_cos_limbs[7][8] = FDS_COS_LIMBS_INIT;
-
-// fold c(m) to +-c(j): accumulate `val` into coordinate j of acc (c(8) = 0 is dropped)
-__device__ __forceinline__ void add_cos_term(int (&acc)[9], int m, int val) {
-  m &= 31;
-  if (m > 16) m = 32 - m;
-  if (m > 8)
-    acc[16 - m] -= val;
-  else
-    acc[m] += val;
-}
 
 // Sign of a0 + sum_{j=1..7} n[j] c(j), evaluated with c(j) to 256 fractional bits.
 // A nonzero value of this form has modulus >= 1 / (2 (2|a0| + 2 sum|n|)^7) (2 c(j) are

@@ -175,31 +175,13 @@ __device__ __forceinline__ void store_run(uint8_t* dst, const uint8_t* src, int 
     *reinterpret_cast<uint16_t*>(dst + j) = *reinterpret_cast<const uint16_t*>(src + j);
 }
 
-// Row butterflies of a lane's channel-block from its pixel buffer: outputs as pairs of columns
-// (0, 4), (1, 2), (3, 5), (6, 7), so that the column pass runs on two columns per packed f32x2
-// instruction; returns the row passes' error weight
+// Row butterflies of a lane's channel-block from its pixel buffer; returns their error weight
 __device__ __forceinline__ float transform_rows(const uint8_t* px_even, const uint8_t* px_odd, uint32_t c, float2 (&P)[8][4]) {
   float V = 0.0f;
 #pragma unroll
   for (int y = 0; y < 8; ++y) {
     const uint2* rp = reinterpret_cast<const uint2*>((y & 1 ? px_odd : px_even) + y * kWPixPitch);
-    const uint2 w01 = rp[0], w23 = rp[1], w45 = rp[2];
-    const uint32_t r[7] = {w01.x, w01.y, w23.x, w23.y, w45.x, w45.y, 0u};
-    uint32_t w[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) w[i] = __funnelshift_r(r[i], r[i + 1], 8 * c);
-    float X[8];
-#pragma unroll
-    for (int x = 0; x < 8; ++x) {
-      const int byte = 3 * x;
-      X[x] = __int_as_float(__byte_perm(w[byte >> 2], 0x4B000000u, 0x7440u | (byte & 3)));
-    }
-    float fr[8];
-    V += dct8_row_bytes_w(X, fr);
-    P[y][0] = make_float2(fr[0], fr[4]);
-    P[y][1] = make_float2(fr[1], fr[2]);
-    P[y][2] = make_float2(fr[3], fr[5]);
-    P[y][3] = make_float2(fr[6], fr[7]);
+    V += row_pass(rp[0], rp[1], rp[2], c, P[y]);
   }
   return V;
 }
@@ -221,14 +203,8 @@ __device__ __forceinline__ void stage_columns(const float2 (&P)[8][4], float V, 
 #pragma unroll
   for (int j = 0; j < 4; ++j) {          // a pair of columns: transformed, rounded and staged
     float2 col[8];
-#pragma unroll
-    for (int y = 0; y < 8; ++y) col[y] = P[y][j];
-    if (j == 0) {
-      const float W = dct8_rat_w2(col);
-      if (live) thr = 0.5f - fminf(fmaf(V, kGuardV, fmaf(W, kGuardW, kGuardU)), kGuardFwd);
-    } else {
-      dct8_2<false, false>(col);
-    }
+    const float W = column_pass(P, j, col);
+    if (j == 0 && live) thr = 0.5f - fminf(fmaf(V, kGuardV, fmaf(W, kGuardW, kGuardU)), kGuardFwd);
     float big = 0.0f;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {

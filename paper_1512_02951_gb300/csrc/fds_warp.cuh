@@ -118,6 +118,41 @@ __device__ __forceinline__ void put_window(const TileArgs& a, uint64_t q, int sl
   }
 }
 
+// ---- the forward transform of a channel-block, as protect computes it and as the coefficients are
+// exported before rounding
+
+// Row butterflies of channel c of one row of a block (24 bytes): outputs as pairs of columns (0, 4),
+// (1, 2), (3, 5), (6, 7), so that the column pass runs on two columns per packed f32x2 instruction;
+// returns the row's error weight
+__device__ __forceinline__ float row_pass(uint2 w01, uint2 w23, uint2 w45, uint32_t c, float2 (&P)[4]) {
+  const uint32_t r[7] = {w01.x, w01.y, w23.x, w23.y, w45.x, w45.y, 0u};
+  uint32_t w[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) w[i] = __funnelshift_r(r[i], r[i + 1], 8 * c);
+  float X[8];
+#pragma unroll
+  for (int x = 0; x < 8; ++x) {
+    const int byte = 3 * x;
+    X[x] = __int_as_float(__byte_perm(w[byte >> 2], 0x4B000000u, 0x7440u | (byte & 3)));
+  }
+  float fr[8];
+  const float weight = dct8_row_bytes_w(X, fr);
+  P[0] = make_float2(fr[0], fr[4]);
+  P[1] = make_float2(fr[1], fr[2]);
+  P[2] = make_float2(fr[3], fr[5]);
+  P[3] = make_float2(fr[6], fr[7]);
+  return weight;
+}
+// Column butterflies of pair j (columns 0 and 4, pair 0, start from exact integers and stay unscaled
+// at the four rational positions); returns pair 0's error weight
+__device__ __forceinline__ float column_pass(const float2 (&P)[8][4], int j, float2 (&col)[8]) {
+#pragma unroll
+  for (int y = 0; y < 8; ++y) col[y] = P[y][j];
+  if (j == 0) return dct8_rat_w2(col);
+  dct8_2<false, false>(col);
+  return 0.0f;
+}
+
 // ---- near ties: the marked values of a subtile (bit pos of a lane's mhi:mlo), decided exactly four at
 // a time, each by a group of eight lanes.  Eight times the value is n_0 + sum n_j c(j) (fds_device.cuh);
 // a lane takes an eighth of the block and of the coordinate table's row (dot products of packed
