@@ -183,8 +183,8 @@ def _peaks():
 
 # the sources each kernel is compiled from (its translation unit and the shared headers)
 KERNEL_SOURCES = {
-    "protect_kernel": ["fds_protect_warp.cu", "fds_warp.cuh"],
-    "restore_kernel": ["fds_restore_warp.cu", "fds_warp.cuh"],
+    "protect_kernel": ["fds_protect_warp.cu", "fds_warp.cuh", "fds_loads.h"],
+    "restore_kernel": ["fds_restore_warp.cu", "fds_warp.cuh", "fds_loads.h"],
     "protect_tc_kernel": ["fds_protect_tc.cu"],
     "aes_ctr_full_kernel": ["fds_aes_full.cu"],
 }

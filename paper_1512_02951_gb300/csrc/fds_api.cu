@@ -1490,7 +1490,6 @@ TileArgs plan_args(const fds_plan* p, int dir) {
   a.total_tiles = p->total_tiles;
   a.k = p->k_uniform;
   a.dispenser = p->dynamic[dir] ? p->d_dispenser : nullptr;
-  a.aes_pair = p->aes_pair[dir];
   return a;
 }
 

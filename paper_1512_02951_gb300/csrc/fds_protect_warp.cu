@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
   }
 
   constexpr int kG = K >= 0 ? acc_tiles(K >= 0 ? K : 0) : 0;
-  const int G = K >= 0 ? kG : a.aes_pair;           // subtiles between two AES phases
+  const int G = K >= 0 ? kG : a.run_tiles;           // subtiles between two AES phases
   int esc = 0, nties = 0;
   bool fail = false, lost = false;         // exact_round failed; a load did not arrive in time
   int acc = 0;
@@ -627,7 +627,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) protect_warp_kernel(const __gr
       store_packed(reinterpret_cast<uint8_t*>(a.pub_out) + (uint64_t)t * pack_pub_bytes<kPW>(k), stage,
                    ((int)n * npub * kPW + 7) >> 3, lane);
       const uint32_t per = pack_priv_bytes<kPW>(k);
-      const int GP = K >= 0 ? pack_acc_tiles<kPW>(K >= 0 ? K : 0) : a.aes_pair;
+      const int GP = K >= 0 ? pack_acc_tiles<kPW>(K >= 0 ? K : 0) : a.run_tiles;
       uint8_t* const pst = GP ? stage + kWCb * 128 : privst;
       if constexpr (K >= 0 && pack_acc_tiles<kPW>(K >= 0 ? K : 0) > 0)
         pack_private_k<K, kPW>(reinterpret_cast<const int16_t*>(privst), reinterpret_cast<uint32_t*>(pst + acc * per), (int)n,
@@ -866,7 +866,7 @@ static cudaError_t launch_w(const TileArgs& a, cudaStream_t s, int sms) {
   const long long per = (nsub + grid - 1) / (grid ? grid : 1);
   b.groups = PACK ? working_warps(per) : (int)(per < kWarps ? per : kWarps);
   bx_division(b);
-  b.aes_pair = PACK == 11 ? pack_acc_tiles<11>(a.k) : (PACK == 8 ? pack_acc_tiles<8>(a.k) : acc_tiles(a.k));
+  b.run_tiles = PACK == 11 ? pack_acc_tiles<11>(a.k) : (PACK == 8 ? pack_acc_tiles<8>(a.k) : acc_tiles(a.k));
   if (grid > 0) protect_warp_kernel<K, BULK, PACK><<<grid, kWarps * 32, kWEnd, s>>>(b);
   return cudaGetLastError();
 }

@@ -27,9 +27,7 @@ constexpr int kSlotBytes = (sizeof(TileSlot) + 15) & ~15;
 constexpr int kSmemBar = kSmemSlot + 3 * kSlotBytes;         // 2 mbarriers (staging areas)
 constexpr int kSmemMisc = kSmemBar + 16;
 constexpr int kSmemBytes = kSmemMisc + 32;
-// one image in int16 storage: the lane-replicated AES table (32 KB; conflict-free lookups)
-// after the rest (measured: 88.7 -> 86.7 us on 4096 x 4096 at k = 5; the batched form, whose
-// tiles mostly carry little keystream, was slower with it, 2.96 -> 3.11 ms on 2000 images)
+// the AES table T0 replicated per lane (32 KB; conflict-free lookups) after the rest
 constexpr int kSmemTrep = kSmemBytes;
 constexpr int kSmemBytesRep = kSmemTrep + 4 * kTrepWords;
 // tensor-core inverse (TC): after the rest, on a 1024-byte boundary, the A operand (256 rows
@@ -59,7 +57,6 @@ __device__ __forceinline__ void gather_coefs(const int16_t* pubst, const int16_t
   }
 }
 
-// cp.async the public and private ranges of slot sl's tile into staging area st
 // True if both fragment ranges of the tile are whole 16-byte units (then each arrives as one
 // bulk copy completing on an mbarrier; else as 16-byte cp.async pieces)
 __device__ __forceinline__ bool frag_bulk(const TileSlot* sl) {

@@ -288,8 +288,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
   const int k = K >= 0 ? K : a.k;
   const int npub = 63 - k;
   const uint32_t nb = 4u * (uint32_t)(k + 1);       // keystream blocks per subtile
-  const int G = K >= 0 ? run_tiles(K >= 0 ? K : 0) : a.aes_pair & 15;
-  const bool twice = K >= 0 ? run_twice(K >= 0 ? K : 0) : (a.aes_pair & 16) != 0;
+  const int G = K >= 0 ? run_tiles(K >= 0 ? K : 0) : a.run_tiles & 15;
+  const bool twice = K >= 0 ? run_twice(K >= 0 ? K : 0) : (a.run_tiles & 16) != 0;
   const bool cipher = !PUBIMG && !a.plain_private;
   uint8_t* const pubst = area + kRFrag;
   uint8_t* const privst = pubst + kWCb * 2 * npub;
@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_packed_kernel(const __
   const int k = K >= 0 ? K : a.k;
   const int npub = 63 - k, period = kDcBits + k * W;
   const uint32_t pub_per = 4u * (uint32_t)(npub * W), priv_per = 4u * (uint32_t)period;
-  const int G = K >= 0 ? run_tiles_packed<W>(K >= 0 ? K : 0) : a.aes_pair;
+  const int G = K >= 0 ? run_tiles_packed<W>(K >= 0 ? K : 0) : a.run_tiles;
   uint8_t* const land_pub = area + kULand;
   uint8_t* const land_priv = land_pub + land_pub_bytes<W>(k);
   int16_t* const pubst = reinterpret_cast<int16_t*>(area + kUStage);
@@ -724,7 +724,7 @@ static cudaError_t launch_packed(const TileArgs& a, cudaStream_t s, int sms) {
   const int grid = (int)(nsub < sms ? nsub : sms);
   b.groups = working_warps((nsub + grid - 1) / (grid ? grid : 1));
   bx_division(b);
-  b.aes_pair = run_tiles_packed<W>(a.k);
+  b.run_tiles = run_tiles_packed<W>(a.k);
   if (grid > 0) restore_packed_kernel<K, W><<<grid, kWarps * 32, kUEnd, s>>>(b);
   return cudaGetLastError();
 }
@@ -927,7 +927,7 @@ static cudaError_t launch_w(const TileArgs& a, cudaStream_t s, int sms) {
   const long long per = (nsub + grid - 1) / (grid ? grid : 1);
   b.groups = working_warps(per);
   bx_division(b);
-  b.aes_pair = run_tiles(a.k) | (run_twice(a.k) ? 16 : 0);
+  b.run_tiles = run_tiles(a.k) | (run_twice(a.k) ? 16 : 0);
   if (grid > 0) restore_warp_kernel<K, PUBIMG><<<grid, kWarps * 32, kREnd, s>>>(b);
   return cudaGetLastError();
 }

@@ -1,6 +1,6 @@
-// What the fused kernels share: their arguments, copies and barriers, and the tiles of the kernels
-// that work on 64 blocks at a time (packed restore, the tensor-core forms; the plans' schedules
-// count in them too).
+// What the fused kernels share: their arguments, copies and barriers, and the tiles of the
+// tensor-core forms, which work on 64 blocks at a time (the plans' schedules count in them too; the
+// warp forms split a tile into six subtiles, fds_warp.cuh).
 //
 // A tile is 64 consecutive 8x8 pixel blocks (row-major over an image's block grid), 192
 // channel-blocks (cb = 3 * block + channel).  Its public and private parts are contiguous,
@@ -100,9 +100,9 @@ struct TileArgs {
   int32_t pack;
   // restore in the public-image form (one image): private positions zero, DC 1024
   int32_t public_image;
-  // warp forms of one image: subtiles whose private parts go through AES together (filled in by
-  // the launcher).  A plan's AES lane schedule arrives here too; its kernels have only one.
-  int32_t aes_pair;
+  // warp forms of one image, filled in by the launcher: subtiles whose private parts go through AES
+  // together (restore of int16 storage: and 16 where two such runs fit)
+  int32_t run_tiles;
   // warp forms: working warps of each CTA (filled in by the launcher)
   int32_t groups;
   // strong level (protect of one image): Part 1 is also left here in plaintext
