@@ -241,35 +241,20 @@ __device__ __forceinline__ void stage_columns(const float2 (&P)[8][4], float V, 
   }
 }
 
-// The marked values of a subtile, decided exactly (take_ties) and staged.  block(): the lane's own
-// block in the image; pub0, priv0: the first lane's place in the staging area; table: a.cfwd, whose
-// row of a position holds eight words a coordinate pair: a lane takes a pixel row and its two words.
-// |n_j| <= 2 . 64 . 255 and so is their sum, so 46 fraction bits fit.  Where kSideBySide lanes or more
-// have marked values, each decides one of its own instead (two rows at a time: all eight held
-// spilled); below, two turns at most do (tie block: turns alone 117 us).
 constexpr int kTieFrac = 46;
+// Where kSideBySide lanes or more have marked values, each decides one of its own in turn, until fewer
+// have any left; returns the lane's, and those too near a boundary for fixed point.  blk, pub_cb, priv_cb:
+// the lane's own.  Two pixel rows at a time (all eight held spilled); a function of its own, because
+// inside the kernel its code slowed down what runs without it (batch of 1000 images, k = 0: 863 us
+// against 782).  Below eight lanes two turns at most do (tie block: turns alone 117 us, with it 39.5).
 constexpr int kSideBySide = 8;
-template <typename Block>
-__device__ __forceinline__ void decide_ties(Block block, uint64_t pitch, uint32_t c, int k, uint32_t mlo, uint32_t mhi,
-                                            int16_t* pub0, int16_t* priv0, const uint32_t* table, int lane, int& nties,
-                                            int& esc, bool& fail) {
-  uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
-  if (__builtin_expect(who == 0, 1)) return;
-  // read here, so that what depends on it is not kept through the subtiles without near ties
-  asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
-  nties += (int)__reduce_add_sync(0xffffffffu, (uint32_t)(__popc(mlo) + __popc(mhi)));
-  const unsigned long long blk = reinterpret_cast<unsigned long long>(block());
-  const long long cos_l = group_cos<kTieFrac>(lane);
-  const int l = lane & 7;
-  auto put = [&](int src, int pos, int q) {
-    const int z = c_zigzag.z[pos];
-    *(z <= k ? priv0 + src * (k + 1) + z : pub0 + src * (63 - k) + (z - k - 1)) = (int16_t)q;
-  };
-  uint32_t hlo = 0, hhi = 0;               // side by side, too near a boundary: by a group after all
-  while (__popc(who) >= kSideBySide) {
+__device__ __noinline__ uint64_t decide_side_by_side(const uint8_t* blk, uint64_t pitch, uint32_t c, int k, uint32_t mlo,
+                                                     uint32_t mhi, int16_t* pub_cb, int16_t* priv_cb, const uint32_t* table) {
+  uint32_t hlo = 0, hhi = 0;               // too near a boundary: by a group after all
+  do {
     if (mlo | mhi) {
       const int pos = mlo ? __ffs(mlo) - 1 : __ffs(mhi) + 31;
-      const uint8_t* row = reinterpret_cast<const uint8_t*>(blk);
+      const uint8_t* row = blk;
       int n[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll 1
       for (int g = 0; g < 4; ++g) {
@@ -286,17 +271,40 @@ __device__ __forceinline__ void decide_ties(Block block, uint64_t pitch, uint32_
         }
       }
       bool sure;
-      put(lane, pos, round_lane<kTieFrac>(n, sure));
+      const int q = round_lane<kTieFrac>(n, sure), z = c_zigzag.z[pos];
+      *(z <= k ? priv_cb + z : pub_cb + (z - k - 1)) = (int16_t)q;
       const uint32_t lo = mlo & -mlo, hi = mlo ? 0u : mhi & -mhi;
       mlo ^= lo;
       mhi ^= hi;
       if (!sure) hlo |= lo, hhi |= hi;
     }
-    who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
+  } while (__popc(__ballot_sync(0xffffffffu, (mlo | mhi) != 0)) >= kSideBySide);
+  return (uint64_t)(mhi | hhi) << 32 | (mlo | hlo);
+}
+
+// The marked values of a subtile, decided exactly (take_ties) and staged.  block(): the lane's own
+// block in the image; pub0, priv0: the first lane's place in the staging area; table: a.cfwd, whose
+// row of a position holds eight words a coordinate pair: a lane takes a pixel row and its two words.
+// |n_j| <= 2 . 64 . 255 and so is their sum, so 46 fraction bits fit.
+template <typename Block>
+__device__ __forceinline__ void decide_ties(Block block, uint64_t pitch, uint32_t c, int k, uint32_t mlo, uint32_t mhi,
+                                            int16_t* pub0, int16_t* priv0, const uint32_t* table, int lane, int& nties,
+                                            int& esc, bool& fail) {
+  uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
+  if (__builtin_expect(who == 0, 1)) return;
+  // read here, so that what depends on it is not kept through the subtiles without near ties
+  asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+  nties += (int)__reduce_add_sync(0xffffffffu, (uint32_t)(__popc(mlo) + __popc(mhi)));
+  const unsigned long long blk = reinterpret_cast<unsigned long long>(block());
+  const long long cos_l = group_cos<kTieFrac>(lane);
+  const int l = lane & 7;
+  if (__popc(who) >= kSideBySide) {
+    const uint64_t left = decide_side_by_side(reinterpret_cast<const uint8_t*>(blk), pitch, c, k, mlo, mhi,
+                                              pub0 + lane * (63 - k), priv0 + lane * (k + 1), table);
+    mlo = (uint32_t)left;
+    mhi = (uint32_t)(left >> 32);
+    who = __ballot_sync(0xffffffffu, left != 0);
   }
-  mlo |= hlo;
-  mhi |= hhi;
-  who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
   while (who) {
     const TieTurn t = take_ties(who, mlo, mhi, lane);
     const uint8_t* row = reinterpret_cast<const uint8_t*>(__shfl_sync(0xffffffffu, blk, t.src)) + l * pitch;
@@ -313,7 +321,10 @@ __device__ __forceinline__ void decide_ties(Block block, uint64_t pitch, uint32_
       }
     }
     const int q = round_group<kTieFrac, 1 << 15>(group_sum(n, lane), cos_l, t.on, lane, esc, fail);
-    if (t.on && l == 0) put(t.src, t.pos, q);
+    if (t.on && l == 0) {
+      const int z = c_zigzag.z[t.pos];
+      *(z <= k ? priv0 + t.src * (k + 1) + z : pub0 + t.src * (63 - k) + (z - k - 1)) = (int16_t)q;
+    }
     who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
   }
 }

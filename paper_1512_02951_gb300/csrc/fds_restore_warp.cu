@@ -148,43 +148,35 @@ __device__ __forceinline__ void emit_rows(const float2 (&G2)[8][4], float l1, bo
   }
 }
 
-// The marked pixels of a subtile, decided exactly (take_ties) and written to the pixel buffer pix, where
-// out is the lane's own block and channel.  pub_g: the subtile's public coefficients in global memory,
-// or STAGED in shared memory; priv0: the first lane's (decrypted) private ones; table: a.cinv, whose
-// row of a position holds a word for four coefficients in zigzag order: a lane takes eight of them.
-// int16 coefficients of any value make the sum of the |n_j| at most 2^22, so 40 fraction bits fit.
-// Of a channel-block with kBlockTies marked pixels or more (flat ones, a half level off, have 64), the
-// whole warp decides 32 at a time, a pixel a lane, and passes over coefficients that are zero (turns
-// alone: 1316 us for DC-only blocks).  From 6 or 8 on it was slower where blocks are not sparse: public
-// image of random rectangles 24.6 -> 26.5 and 27.1 us.
+// A coefficient of a channel-block by zigzag index
+template <bool PUBIMG, bool STAGED>
+__device__ __forceinline__ int coefficient(const int16_t* pub, const int16_t* priv, int k, int z) {
+  return z <= k ? (PUBIMG ? (z == 0 ? 1024 : 0) : priv[z]) : (STAGED ? pub[z - k - 1] : __ldg(pub + z - k - 1));
+}
+__device__ __forceinline__ void put_pixel(uint8_t* block, int pos, int p) {
+  block[(pos >> 3) * kRPitch + 3 * (pos & 7)] = (uint8_t)(p < 0 ? 0 : (p > 255 ? 255 : p));
+}
+
+// Of the channel-blocks with kBlockTies marked pixels or more (flat ones, a half level off, have 64),
+// the whole warp decides 32 at a time, a pixel a lane, and passes over coefficients that are zero;
+// returns what the lane has left, and the pixels too near a boundary for fixed point.  Arguments as of
+// decide_pixels; at: the lane's block in the pixel buffer.  Turns alone took 1316 us for DC-only blocks
+// (119 with this).  From 6 or 8 marked pixels on it was slower where blocks are not sparse: public image
+// of random rectangles 24.6 -> 26.5 and 27.1 us.  A function of its own: inside the kernel it slowed down
+// what runs without it (batch of 300 images of mixed k, 599 us against 585).
 constexpr int kPixFrac = 40;
 constexpr int kBlockTies = 16;
-template <bool PUBIMG, bool STAGED = false>
-__device__ __forceinline__ void decide_pixels(uint32_t mlo, uint32_t mhi, const int16_t* pub_g, const int16_t* priv0, int k,
-                                              const uint32_t* table, int lane, WarpSlot* slot, uint8_t* pix,
-                                              const uint8_t* out) {
-  uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
-  if (__builtin_expect(who == 0, 1)) return;
-  // read here, so that what depends on it is not kept through the subtiles without near ties
-  asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
-  int esc = 0;
-  bool fail = false;
-  const int nties = (int)__reduce_add_sync(0xffffffffu, (uint32_t)(__popc(mlo) + __popc(mhi)));
-  const uint32_t at = (uint32_t)(out - pix);
-  const long long cos_l = group_cos<kPixFrac>(lane);
-  const int l = lane & 7;
-  auto coef = [&](const int16_t* pub, const int16_t* priv, int z) -> int {
-    return z <= k ? (PUBIMG ? (z == 0 ? 1024 : 0) : priv[z]) : (STAGED ? pub[z - k - 1] : __ldg(pub + z - k - 1));
-  };
-  auto put = [&](uint32_t to, int pos, int p) {
-    pix[to + (pos >> 3) * kRPitch + 3 * (pos & 7)] = (uint8_t)(p < 0 ? 0 : (p > 255 ? 255 : p));
-  };
+template <bool PUBIMG, bool STAGED>
+__device__ __noinline__ uint64_t decide_blocks(uint32_t mlo, uint32_t mhi, const int16_t* pub_g, const int16_t* priv0, int k,
+                                               const uint32_t* table, uint8_t* pix, uint32_t at) {
+  const int lane = (int)(threadIdx.x & 31);
   for (uint32_t many = __ballot_sync(0xffffffffu, __popc(mlo) + __popc(mhi) >= kBlockTies); many; many &= many - 1) {
     const int src = __ffs(many) - 1;
     const uint32_t to = __shfl_sync(0xffffffffu, at, src);
     const int16_t* pub = pub_g + src * (63 - k);
     const int16_t* priv = priv0 + src * (k + 1);
-    const uint32_t Q = __byte_perm((uint32_t)coef(pub, priv, 2 * lane), (uint32_t)coef(pub, priv, 2 * lane + 1), 0x5410u);
+    const uint32_t Q = __byte_perm((uint32_t)coefficient<PUBIMG, STAGED>(pub, priv, k, 2 * lane),
+                                   (uint32_t)coefficient<PUBIMG, STAGED>(pub, priv, k, 2 * lane + 1), 0x5410u);
     const uint32_t used = __ballot_sync(0xffffffffu, Q != 0);
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
@@ -203,12 +195,39 @@ __device__ __forceinline__ void decide_pixels(uint32_t mlo, uint32_t mhi, const 
       }
       bool sure;
       const int p = round_lane<kPixFrac>(n, sure);
-      if (on) put(to, 32 * h + lane, p);
+      if (on) put_pixel(pix + to, 32 * h + lane, p);
       const uint32_t left = __ballot_sync(0xffffffffu, on && !sure);
       if (lane == src) (h ? mhi : mlo) = left;
     }
   }
-  who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
+  return (uint64_t)mhi << 32 | mlo;
+}
+
+// The marked pixels of a subtile, decided exactly (take_ties) and written to the pixel buffer pix, where
+// out is the lane's own block and channel.  pub_g: the subtile's public coefficients in global memory,
+// or STAGED in shared memory; priv0: the first lane's (decrypted) private ones; table: a.cinv, whose
+// row of a position holds a word for four coefficients in zigzag order: a lane takes eight of them.
+// int16 coefficients of any value make the sum of the |n_j| at most 2^22, so 40 fraction bits fit.
+template <bool PUBIMG, bool STAGED = false>
+__device__ __forceinline__ void decide_pixels(uint32_t mlo, uint32_t mhi, const int16_t* pub_g, const int16_t* priv0, int k,
+                                              const uint32_t* table, int lane, WarpSlot* slot, uint8_t* pix,
+                                              const uint8_t* out) {
+  uint32_t who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
+  if (__builtin_expect(who == 0, 1)) return;
+  // read here, so that what depends on it is not kept through the subtiles without near ties
+  asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+  int esc = 0;
+  bool fail = false;
+  const int nties = (int)__reduce_add_sync(0xffffffffu, (uint32_t)(__popc(mlo) + __popc(mhi)));
+  const uint32_t at = (uint32_t)(out - pix);
+  const long long cos_l = group_cos<kPixFrac>(lane);
+  const int l = lane & 7;
+  if (__any_sync(0xffffffffu, __popc(mlo) + __popc(mhi) >= kBlockTies)) {
+    const uint64_t left = decide_blocks<PUBIMG, STAGED>(mlo, mhi, pub_g, priv0, k, table, pix, at);
+    mlo = (uint32_t)left;
+    mhi = (uint32_t)(left >> 32);
+    who = __ballot_sync(0xffffffffu, left != 0);
+  }
   while (who) {
     const TieTurn t = take_ties(who, mlo, mhi, lane);
     const uint32_t to = __shfl_sync(0xffffffffu, at, t.src);
@@ -222,7 +241,7 @@ __device__ __forceinline__ void decide_pixels(uint32_t mlo, uint32_t mhi, const 
       for (int i = 0; i < 4; ++i) {
         int q[2];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) q[h] = coef(pub, priv, 8 * l + 2 * i + h);
+        for (int h = 0; h < 2; ++h) q[h] = coefficient<PUBIMG, STAGED>(pub, priv, k, 8 * l + 2 * i + h);
         Q[i] = __byte_perm((uint32_t)q[0], (uint32_t)q[1], 0x5410u);
       }
 #pragma unroll
@@ -232,7 +251,7 @@ __device__ __forceinline__ void decide_pixels(uint32_t mlo, uint32_t mhi, const 
       }
     }
     const int p = round_group<kPixFrac, 1 << 22>(group_sum(n, lane), cos_l, t.on, lane, esc, fail);
-    if (t.on && l == 0) put(to, t.pos, p);
+    if (t.on && l == 0) put_pixel(pix + to, t.pos, p);
     who = __ballot_sync(0xffffffffu, (mlo | mhi) != 0);
   }
   if (lane == 0) {

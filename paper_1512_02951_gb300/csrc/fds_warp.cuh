@@ -162,9 +162,9 @@ __device__ __forceinline__ float column_pass(const float2 (&P)[8][4], int j, flo
 // two to four turns.  What bounds it is issue where ties are many and the chain of a turn (loads from
 // L2, three exchanges, twice) where one block has many.  A whole warp for each value, as before, made
 // content with many near ties slow; 2048 x 2048, k = 5, us: protect of black and white noise 57.9 ->
-// 33.1, of a slow ramp 81.6 -> 44.1, of a block of four ties repeated 303 -> 37.5; the public image of
-// text 48.6 -> 21.0; restore of DC-only blocks half a level off (every pixel a tie, k = 0) 3457 -> 124;
-// smooth scenes with ten ties a thousand channel-blocks 21.1 -> 20.8 and 24.3 -> 22.9.
+// 33.6, of a slow ramp 81.6 -> 42.9, of a block of four ties repeated 303 -> 39.5; the public image of
+// text 48.6 -> 20.0; restore of DC-only blocks half a level off (every pixel a tie, k = 0) 3457 -> 119;
+// smooth scenes with ten ties a thousand channel-blocks 21.1 -> 20.8 and 24.3 -> 22.8.
 
 // zigzag index by position 8 u + v
 struct ZigzagTable {
