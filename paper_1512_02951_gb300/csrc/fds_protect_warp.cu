@@ -5,10 +5,10 @@
 // and private parts are 64 (63 - k) and 64 (k + 1) bytes, whole 16-byte units.  Each warp works
 // on subtiles of its own with its own shared-memory area, and no barrier joins the warps after
 // the AES table is filled.  What bounds it is the issue of instructions, not memory (4096 x 4096,
-// k = 5: 41.8 M warp instructions = 33 us of issue slots against 22.6 us for the 151 MB), so the
+// k = 5: 41.5 M warp instructions = 33 us of issue slots against 22.6 us for the 151 MB), so the
 // warps have to keep issuing.  The form before it, groups of six warps that met at three named
 // barriers per 192 channel-blocks, spent its time at those barriers: 4.5 of the six warps had
-// AES blocks to do, and issue activity was 57 %; here it is 69 %.  Per subtile:
+// AES blocks to do, and issue activity was 57 %; here it is 72 %.  Per subtile:
 //   1. its pixels are in the warp's buffer (bulk copies that complete on the warp's mbarrier);
 //      row butterflies; the buffer is free, so the next subtile's pixels start loading
 //   2. column butterflies by pairs of columns, rounded and written as int16 to the staging area;
@@ -20,7 +20,7 @@
 //      three), encrypted, and leave
 // Counter blocks that share all but their last byte share the first AES round and most of the
 // second (aes_window): 133 table lookups a block instead of 160.
-// Measured on 4096 x 4096, k = 5: 72.3 -> 54.3 us; 3240 x 2592, k = 9: 55.9 -> 38.6 us (before:
+// Measured on 4096 x 4096, k = 5: 72.3 -> 53.5 us; 3240 x 2592, k = 9: 55.9 -> 37.2 us (before:
 // the grouped form; its 8-byte pixel loads and 240 AES blocks on 192 threads cost the latter
 // more).  16 warps of 128 registers; 20 of 96 measured 53.6 and 39.6 us, with spills.  Pixels two
 // subtiles ahead, or loaded with cp.async through L1, measured slower (59 / 64 us against 51 and
@@ -331,8 +331,8 @@ __device__ __forceinline__ void decide_ties(Block block, uint64_t pitch, uint32_
 
 // ---- packed storage (Sect. 6.4.3, Table 5): after a subtile's ties are decided its staged
 // coefficients are packed, the public part in place and out at once, the private parts of a few
-// subtiles side by side until they are encrypted.  The packing itself is the cost (11 bits: 61.6 M
-// warp instructions for 4096 x 4096, k = 5, against 41.8 M for int16): 80 us a launch, 104 us in
+// subtiles side by side until they are encrypted.  The packing itself is the cost (11 bits: 60.9 M
+// warp instructions for 4096 x 4096, k = 5, against 41.5 M for int16): 78 us a launch, 104 us in
 // the grouped form, 101 us before private words were built per channel-block and fields were
 // placed by multiply-adds.
 
@@ -726,7 +726,7 @@ static __constant__ AccTable c_acc = make_acc_table();
 // Protect of a batch: every tile of 64 blocks of every image, six subtiles a tile.  A CTA has a
 // run of the batch's tiles, taken by its warps as PlanClaim says; or (a.dispenser) every warp takes
 // tiles from one counter.  Bound by issue, as one image: 1000 images (2.97 GB in and out), k = 0,
-// 1210 -> 797 us (24 warps of 80 registers per SM, which spilled and met at three barriers a tile, before).
+// 1210 -> 786 us (24 warps of 80 registers per SM, which spilled and met at three barriers a tile, before).
 template <int K>
 __global__ void __launch_bounds__(kWarps * 32, 1) protect_plan_kernel(const __grid_constant__ TileArgs a) {
   extern __shared__ __align__(128) uint8_t smem_cta[];

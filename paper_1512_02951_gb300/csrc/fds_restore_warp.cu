@@ -5,9 +5,9 @@
 //
 // As in the warp form of protect, each warp works on subtiles of 32 channel-blocks of its own,
 // with no barrier between warps after the AES table is filled.  It is bound by the issue of
-// instructions (4096 x 4096, k = 5: 47.5 M warp instructions = 37.7 us of issue slots against
+// instructions (4096 x 4096, k = 5: 45.5 M warp instructions = 36.2 us of issue slots against
 // 22.6 us for the 151 MB); two CTAs of six warps that met at three barriers per 192
-// channel-blocks issued in 61 % of the cycles, sixteen independent warps in 72 %.  Per subtile:
+// channel-blocks issued in 61 % of the cycles, sixteen independent warps in 71 %.  Per subtile:
 //   1. its public part has arrived (bulk copy on the warp's mbarrier); two columns at a time the
 //      coefficients are gathered, converted and transformed (the loads of the next two stay
 //      behind: with all 64 in flight the kernel spilled 200 bytes and took 78 us); the buffer is
@@ -21,7 +21,7 @@
 // Private parts come in runs of subtiles whose keystream blocks fill whole warps (k = 5: four
 // subtiles, 96 blocks), one run ahead, and are decrypted in place.  The last two or so subtiles a
 // warp are claimed one by one, so that a CTA's warps end together.
-// Measured on 4096 x 4096: k = 5 79.0 -> 59.9 us.  Testing a row for values outside [0, 255] and
+// Measured on 4096 x 4096: k = 5 79.0 -> 60.4 us; the public-image form 66.6 -> 45.4 us.  Testing a row for values outside [0, 255] and
 // clamping only then (96 instructions a subtile less) measured no faster: 60.6 us.
 #include "fds_aux.h"
 #include "fds_warp.cuh"
@@ -486,8 +486,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1) restore_warp_kernel(const __gr
 // A subtile's packed parts land as they lie in the streams (4-byte granular: widened to 16-byte
 // boundaries for a bulk copy), the private ones of a run of subtiles at a time, and are unpacked
 // into an int16 staging area, which the transform and the exact decisions read; a landing area is
-// free, and loads again, as soon as it is unpacked.  Bound by issue: 4096 x 4096, k = 5,
-// 104 -> 76 us (11 and 8 bits).
+// free, and loads again, as soon as it is unpacked.  Bound by issue (4096 x 4096, k = 5: 56.4 M warp
+// instructions, issued in 69 % of the cycles): 104 -> 76 us (11 and 8 bits).
 constexpr int kUPix = 0;
 constexpr int kUStage = kUPix + 8 * kRPitch;      // int16 coefficients of a subtile
 constexpr int kULand = kUStage + kWCb * 128;      // public landing, private landing
@@ -774,7 +774,8 @@ static __constant__ RunTable c_run = make_run_table();
 
 // Restore of a batch (the tiles as in protect_plan_kernel).  Where the next run is of an image
 // with another k, its parts lie elsewhere in the buffers and are loaded only when the run before
-// is done.  Bound by issue, as one image: 300 images (742 MB in and out), k = 5, 445 -> 306 us (two
+// is done.  Bound by issue (241 M warp instructions, issued in 66 % of the cycles: its code is the
+// largest, and fetching it the first stall): 300 images (742 MB in and out), k = 5, 445 -> 308 us (two
 // CTAs per SM, a tile of six warps each, before).
 template <int K>
 __global__ void __launch_bounds__(kWarps * 32, 1) restore_plan_kernel(const __grid_constant__ TileArgs a) {

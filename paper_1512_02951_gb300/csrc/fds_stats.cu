@@ -13,8 +13,8 @@
 // direction's sums of x, y, x^2, y^2 lack of the totals are the first and last rows and columns,
 // which four CTAs of their own add up; the CTA that finishes last writes the 54 sums.
 //
-// Four rows' loads are in flight per warp; what bounds it is their latency (4096 x 4096: 13.2 M warp
-// instructions, the ALU 39 % busy, 32.7 us cold under ncu and about 28 us after the image has been
+// Four rows' loads are in flight per warp; what bounds it is their latency (4096 x 4096: 13.5 M warp
+// instructions, the ALU 37 % busy, 32.9 us cold under ncu and about 28 us after the image has been
 // written, against 7.5 us for the 50 MB).  A row's loads at a time took 37 us; the kernel before
 // (pixel rows staged in shared memory, a byte at a time, three launches with the clears) took 114
 // us and 85 M warp instructions.
